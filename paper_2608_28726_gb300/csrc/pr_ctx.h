@@ -55,6 +55,7 @@ struct pr_ctx {
   void* lm_parts = nullptr;
   size_t lm_parts_bytes = 0;
   bool lm_ready = false;
+  bool qmlp_ready = false;  // pr_quantile_score: shared memory opt-in made
   // PR_OPT_TIMING: events after each kernel of the last multi-kernel call
   int32_t timing = 0;
   cudaEvent_t tev[PR_MAX_TIMED + 1] = {};

@@ -8,15 +8,13 @@
 // One CTA per request.  Up to Q_SMALL rows two warps per feature sort its
 // column's order-preserving 32-bit keys (padded to 256) in registers, four
 // per lane (a bitonic network inside the lanes, across them by shfl.xor, and
-// one stage between the two warps).  Up to Q_CAP rows the
-// four columns are bitonic-sorted together: up to 1,024 rows each thread
-// holds a run of keys in registers (register and warp-shuffle stages, one
-// stage through shared memory), above that in shared memory; longer requests
-// find each needed order statistic by radix selection (four 8-bit passes of
-// shared histograms over the request's rows in global memory).  All three
-// give the exact order statistics.  The MLP runs in the same CTA with
-// fixed-order sums (four threads per hidden unit, quarters added in a fixed
-// butterfly).
+// one stage between the two warps).  Up to Q_MID rows the four columns are
+// bitonic-sorted together, each thread holding a run of keys in registers
+// (register and warp-shuffle stages, one stage through shared memory).  Longer
+// requests select: histograms of the keys find the few keys around each needed
+// rank, and only those are sorted (q_select).  All three give the exact order
+// statistics.  The MLP runs in the same CTA with fixed-order sums (four
+// threads per hidden unit, quarters added in a fixed butterfly).
 #pragma once
 
 #include "pr_device.cuh"
@@ -27,8 +25,14 @@ constexpr int Q_NT = 256;
 constexpr int Q_NQ = 7;             // quantile levels
 constexpr int Q_NS = 4 * Q_NQ;      // summary length
 constexpr int Q_H = 64;             // hidden width
-constexpr int Q_CAP = 2048;         // rows sorted in shared memory
-constexpr int Q_SMALL = 256;        // rows ranked by counting (one per thread)
+constexpr int Q_SMALL = 256;        // rows sorted in registers, two warps per column
+// Rows sorted whole: 12.4 us for a lone request of 513 to 1,024 rows whatever its
+// values (graph replay).  From 1,025 rows, where 2,048 keys per column no longer
+// fit the registers and the sort through shared memory took 62 us, the selection
+// takes 10.3 us, 22 to 32 us when its bins are crowded, which is why shorter
+// requests keep the sort (2,048 rows: 11.7 against 62.5 us, crowded 30 to 49;
+// 4,000 rows: 17.6 against 360 us by a radix selection of one rank at a time).
+constexpr int Q_MID = 1024;
 __constant__ int32_t q_level_a[Q_NQ] = {0, 1, 1, 1, 3, 9, 1};
 __constant__ int32_t q_level_b[Q_NQ] = {1, 10, 4, 2, 4, 10, 1};
 
@@ -44,8 +48,25 @@ constexpr int QS_W1 = 0, QS_B1 = Q_H * (Q_NS + 1), QS_W2 = QS_B1 + Q_H,
               QS_B2 = QS_W2 + Q_H * (Q_H + 1), QS_W3 = QS_B2 + Q_H, QS_B3 = QS_W3 + Q_H,
               QS_SIZE = QS_B3 + 1;
 constexpr int QW_PER_T = (QW_SIZE + Q_NT - 1) / Q_NT;  // weights each thread fetches
-static_assert(QS_SIZE <= 4 * Q_CAP, "the weights fit in the key buffer");
-static_assert(4 * Q_SMALL + QS_SIZE <= 4 * Q_CAP, "beside the keys of a short request too");
+
+// q_select: histograms of Q_BINS bins per feature, scanned by 64 threads in runs
+// of Q_RUN bins (one word of padding per run, so that the runs lie in different
+// banks), then of Q_SUB bins for each crowded bin
+constexpr int Q_BINS = 2048, Q_SUB = 64, Q_RUN = Q_BINS / 64;
+constexpr int Q_HW = Q_BINS + Q_BINS / Q_RUN;  // words of a feature's histogram
+constexpr int Q_NR = 2 * Q_NQ;              // ranks per feature (12 distinct ones)
+constexpr int Q_FEW = 42;                   // most keys of a bin that are collected
+constexpr int Q_CAND = 512;                 // collected keys per feature
+constexpr int Q_REC = 8;                    // records a thread holds in registers
+static_assert(12 * Q_FEW <= Q_CAND, "the bins of all needed ranks fit");
+constexpr int Q_SUB_WORDS = 4 * 12 * (Q_SUB + 1);  // counts of up to 12 crowded bins per feature
+static_assert(Q_SUB_WORDS + 12 * Q_SUB <= 4 * Q_HW, "in the place of the histograms");
+// dynamic shared memory (words): the MLP's weights, in whose place q_select
+// keeps its histograms and marks before, and the keys of a column set
+constexpr int Q_HM_WORDS = 4 * Q_HW + Q_BINS;  // histograms, a byte of marks per bin
+constexpr int Q_W_WORDS = (QS_SIZE > Q_HM_WORDS ? QS_SIZE : Q_HM_WORDS) + 3 & ~3;
+constexpr int Q_DYN = Q_W_WORDS + 4 * Q_CAND;
+static_assert(4 * Q_MID <= Q_DYN && 4 * Q_SMALL + QS_SIZE <= Q_DYN, "whole columns");
 static_assert(Q_SMALL == 256 && Q_NT == 256, "two warps per column sort 256 keys");
 static_assert(Q_NT == 4 * Q_H && Q_NS % 4 == 0 && Q_H % 4 == 0, "four threads per hidden unit");
 
@@ -84,57 +105,6 @@ __device__ __forceinline__ float q_unkey(uint32_t k) {
 
 // record slot of feature f: l, m, h, rho
 __device__ __forceinline__ int q_slot(int f) { return f == 0 ? 0 : f == 1 ? 1 : f == 2 ? 4 : 5; }
-
-// Key of rank r (0-based, ascending) among the keys of feature f in rows
-// [lo, lo + T), by radix selection over global memory.  Whole CTA.
-__device__ uint32_t q_select(const float* __restrict__ feat, int64_t lo, int T, int f, int r,
-                             uint32_t* hist, uint32_t* bcast) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint32_t prefix = 0, mask = 0;
-  uint32_t rank = (uint32_t)r;
-  const int slot = q_slot(f);
-  for (int shift = 24; shift >= 0; shift -= 8) {
-    if (tid < 256) hist[tid] = 0;
-    __syncthreads();
-    for (int t = tid; t < T; t += Q_NT) {
-      const uint32_t k = q_key(feat[(lo + t) * NFEAT + slot]);
-      if ((k & mask) == prefix) atomicAdd(&hist[(k >> shift) & 0xff], 1u);
-    }
-    __syncthreads();
-    if (warp == 0) {  // the digit whose cumulative count passes `rank`
-      uint32_t c[8], s = 0;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        c[e] = hist[lane * 8 + e];
-        s += c[e];
-      }
-      uint32_t x = s;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(FULL, x, o);
-        if (lane >= o) x += y;
-      }
-      const unsigned hit = __ballot_sync(FULL, x > rank);
-      const int L = __ffs(hit) - 1;  // first lane whose inclusive count passes rank
-      if (lane == L) {
-        uint32_t cum = x - s;
-        int d = lane * 8;
-        for (int e = 0; e < 8; ++e, ++d) {
-          if (rank < cum + c[e]) break;
-          cum += c[e];
-        }
-        bcast[0] = (uint32_t)d;
-        bcast[1] = rank - cum;
-      }
-    }
-    __syncthreads();
-    prefix |= bcast[0] << shift;
-    mask |= 0xffu << shift;
-    rank = bcast[1];
-    __syncthreads();
-  }
-  return prefix;
-}
 
 // Ascending bitonic sort of the 256 keys of one column held by two warps:
 // lane l of warp `half` holds keys c = 128 half + 4 l .. + 3 in v.  Stages of
@@ -242,11 +212,322 @@ __device__ void q_bitonic(uint32_t* qs, int ln2) {
   for (int e = 0; e < E; ++e) col[c0 + e] = v[e];
 }
 
+// keys [lo, lo + range] in `bins` equal steps: step of a key at distance d from
+// lo is umulhi(d, mul), or d itself when mul is 0 (at most `bins` keys).  The
+// multiplier is rounded down, so the last step stays below `bins`.
+__device__ __forceinline__ uint32_t q_mul(uint32_t range, int bins) {
+  if (range < (uint32_t)bins) return 0u;
+  return (uint32_t)__fdiv_rz((float)bins * 4294963200.f, (float)range + 1.f);
+}
+__device__ __forceinline__ uint32_t q_step(uint32_t d, uint32_t mul) {
+  return mul ? __umulhi(d, mul) : d;
+}
+
+// The order statistics of a request of T > Q_MID rows, by selection: whole
+// CTA, quantile tid of the summary in *out for tid < Q_NS.
+//   1. every feature's smallest and largest key (up to Q_REC * Q_NT rows the
+//      records stay in registers, more rows are read again in each pass)
+//   2. a histogram of Q_BINS equal steps of key between the two (key space is
+//      about logarithmic in the value, which suits log-probabilities,
+//      probabilities and position fractions alike)
+//   3. the bin of every needed rank and the count of keys before it
+//   4. the keys of those bins: bins of up to Q_FEW keys are collected, of a
+//      crowded bin the smallest and largest key are kept
+//   5. crowded bins whose keys differ are divided again, by Q_SUB, until the
+//      ranks' bins hold few keys or one key many times (at most five rounds
+//      for 32-bit keys; none on data without clusters)
+//   6. the collected keys, about 150 per feature, are sorted; bins are
+//      disjoint and ascending, so a rank's key stands at a known place
+// Bound by the latency of this chain and, for long requests, of the passes.
+// `idle` runs before the sort (loads that the caller wants in flight).
+template <typename F>
+__device__ __forceinline__ void q_select(const float* __restrict__ feat, int64_t lo, int T,
+                                         uint32_t* dyn, uint32_t (*qx)[Q_SMALL], float* out,
+                                         F idle) {
+  __shared__ uint32_t s_red[8][Q_NT / 32], s_rank[Q_NR], s_pre[4][64], s_half[4], s_n[4];
+  __shared__ uint32_t s_base[4][Q_NR], s_cnt[4][Q_NR], s_lo[4][Q_NR], s_hi[4][Q_NR];
+  __shared__ uint32_t s_glo[4][Q_NR], s_ghi[4][Q_NR], s_gmul[4][Q_NR], s_bin0[4][Q_NR];
+  __shared__ int s_grp[4][Q_NR], s_gend[4][Q_NR], s_off[4][Q_NR];
+  uint32_t* hist = dyn;                                     // [4][Q_HW]
+  uint8_t* mark = reinterpret_cast<uint8_t*>(dyn + 4 * Q_HW);  // [4][Q_BINS]
+  // of the crowded bins: [4][12][Q_SUB + 1] counts and [4][12][Q_SUB] marks
+  uint8_t* sub_mark = reinterpret_cast<uint8_t*>(dyn + Q_SUB_WORDS);
+  uint32_t* cand = dyn + Q_W_WORDS;                         // [4][Q_CAND]
+  constexpr uint8_t COLLECT = 0xff;  // a mark: collect the bin's keys; r + 1: extremes to rank r
+  constexpr int CHUNK = Q_REC * Q_NT;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool once = T <= CHUNK;
+  uint32_t k[Q_REC][4];
+  auto load = [&](uint32_t c0) {
+#pragma unroll
+    for (int i = 0; i < Q_REC; ++i) {
+      const uint32_t t = c0 + (uint32_t)(i * Q_NT + tid);
+      if (t < (uint32_t)T) {
+        const float4* rec = reinterpret_cast<const float4*>(feat + (lo + t) * NFEAT);
+        const float4 r0 = __ldg(rec), r1 = __ldg(rec + 1);
+        k[i][0] = q_key(r0.x);  // l
+        k[i][1] = q_key(r0.y);  // m
+        k[i][2] = q_key(r1.x);  // h
+        k[i][3] = q_key(r1.y);  // rho
+      }
+    }
+  };
+  // body(f, key) for every key of the request
+  auto each_key = [&](bool held, auto body) {
+    for (uint32_t c0 = 0; c0 < (uint32_t)T; c0 += CHUNK) {
+      if (!held) load(c0);
+#pragma unroll
+      for (int i = 0; i < Q_REC; ++i)
+        if (c0 + (uint32_t)(i * Q_NT + tid) < (uint32_t)T) {
+#pragma unroll
+          for (int f = 0; f < 4; ++f) body(f, k[i][f]);
+        }
+    }
+  };
+
+  auto clear = [&](int words) {
+    for (int i = tid; i < words / 4; i += Q_NT)
+      reinterpret_cast<uint4*>(dyn)[i] = make_uint4(0u, 0u, 0u, 0u);
+  };
+  static_assert(Q_HM_WORDS % 4 == 0 && Q_SUB_WORDS % 4 == 0 && Q_SUB % 4 == 0, "16-byte stores");
+  clear(Q_HM_WORDS);
+  if (tid < Q_NR) {  // rank 2 j: the lower order statistic of level j; 2 j + 1: the upper
+    const int64_t num = (int64_t)q_level_a[tid >> 1] * (T - 1);
+    const int b = q_level_b[tid >> 1];
+    const int64_t i = num / b;
+    s_rank[tid] = (uint32_t)((tid & 1) && num != i * b ? i + 1 : i);
+  }
+  if (tid < 4) s_n[tid] = 0u;
+  uint32_t kmin[4] = {~0u, ~0u, ~0u, ~0u}, kmax[4] = {0u, 0u, 0u, 0u}, mul[4];
+  each_key(false, [&](int f, uint32_t key) {
+    kmin[f] = min(kmin[f], key);
+    kmax[f] = max(kmax[f], key);
+  });
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    const uint32_t a = __reduce_min_sync(FULL, kmin[f]), b = __reduce_max_sync(FULL, kmax[f]);
+    if (lane == 0) {
+      s_red[f][warp] = a;
+      s_red[4 + f][warp] = b;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    kmin[f] = s_red[f][0];
+    kmax[f] = s_red[4 + f][0];
+#pragma unroll
+    for (int w = 1; w < Q_NT / 32; ++w) {
+      kmin[f] = min(kmin[f], s_red[f][w]);
+      kmax[f] = max(kmax[f], s_red[4 + f][w]);
+    }
+    mul[f] = q_mul(kmax[f] - kmin[f], Q_BINS);
+  }
+  each_key(once, [&](int f, uint32_t key) {
+    const uint32_t b = q_step(key - kmin[f], mul[f]);
+    atomicAdd(hist + f * Q_HW + b + b / Q_RUN, 1u);
+  });
+  __syncthreads();
+
+  {  // 64 threads per feature: the counts before each run of bins
+    const int f = tid >> 6, u = tid & 63;
+    const uint32_t* h = hist + f * Q_HW + (Q_RUN + 1) * u;
+    uint32_t sum = 0;
+#pragma unroll
+    for (int i = 0; i < Q_RUN; ++i) sum += h[i];
+    uint32_t x = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(FULL, x, o);
+      if (lane >= o) x += y;
+    }
+    s_pre[f][u] = x - sum;
+    if (u == 31) s_half[f] = x;
+  }
+  __syncthreads();
+  // the bin of each rank (one warp per feature, one lane per rank), marked by
+  // its first rank: collect its keys, or keep their extremes at that rank
+  const int f_of = warp >> 1, j_of = min(lane, Q_NR - 1);
+  auto settle = [&](uint32_t base, uint32_t cnt, uint8_t* m) {
+    const uint32_t prev = __shfl_up_sync(FULL, base, 1);
+    if (lane >= Q_NR || !m) return;
+    s_base[f_of][lane] = base;
+    s_cnt[f_of][lane] = cnt;
+    s_lo[f_of][lane] = ~0u;
+    s_hi[f_of][lane] = 0u;
+    if (lane == 0 || base != prev) *m = cnt <= (uint32_t)Q_FEW ? COLLECT : (uint8_t)(lane + 1);
+  };
+  if ((warp & 1) == 0) {
+    const uint32_t r = s_rank[j_of];
+    int u = 0;
+#pragma unroll
+    for (int o = 32; o > 0; o >>= 1) {  // the last run whose count before is <= r
+      const int v = u + o;
+      if (s_pre[f_of][v] + (v >= 32 ? s_half[f_of] : 0u) <= r) u = v;
+    }
+    const uint32_t* h = hist + f_of * Q_HW + (Q_RUN + 1) * u;
+    uint32_t c = s_pre[f_of][u] + (u >= 32 ? s_half[f_of] : 0u), base = c, cnt = 0;
+    int at = 0;
+#pragma unroll
+    for (int i = 0; i < Q_RUN; ++i) {
+      const uint32_t n = h[i];
+      if (r >= c && r < c + n) {
+        at = i;
+        base = c;
+        cnt = n;
+      }
+      c += n;
+    }
+    settle(base, cnt, mark + f_of * Q_BINS + Q_RUN * u + at);
+    if (lane < Q_NR) s_bin0[f_of][lane] = base;
+  }
+  __syncthreads();
+  auto take = [&](int f, uint32_t key, uint32_t m) {
+    if (m == COLLECT) {
+      cand[f * Q_CAND + atomicAdd(&s_n[f], 1u)] = key;
+    } else if (m) {  // most keys of a bin lie inside the extremes seen so far
+      if (key < *(volatile uint32_t*)&s_lo[f][m - 1]) atomicMin(&s_lo[f][m - 1], key);
+      if (key > *(volatile uint32_t*)&s_hi[f][m - 1]) atomicMax(&s_hi[f][m - 1], key);
+    }
+  };
+  auto mark_of = [&](int f, uint32_t key) -> uint32_t {
+    return mark[f * Q_BINS + (int)q_step(key - kmin[f], mul[f])];
+  };
+  each_key(once, [&](int f, uint32_t key) { take(f, key, mark_of(f, key)); });
+
+  // crowded bins with different keys: divided again between their extremes
+  for (;;) {
+    __syncthreads();
+    bool mixed = false;
+    if ((warp & 1) == 0) {
+      const uint32_t base = s_base[f_of][j_of], bin0 = s_bin0[f_of][j_of];
+      const uint32_t prev = __shfl_up_sync(FULL, base, 1);
+      const uint32_t prev0 = __shfl_up_sync(FULL, bin0, 1);
+      const uint32_t a = s_lo[f_of][j_of], b = s_hi[f_of][j_of];
+      mixed = lane < Q_NR && (lane == 0 || base != prev) && a < b;
+      const unsigned bal = __ballot_sync(FULL, mixed);
+      // a rank's group is the one that its bin's first rank opens; the groups of
+      // a bin of the first histogram end where those of the next one start
+      const unsigned upto = 0xffffffffu >> (31 - lane);
+      const unsigned firsts = __ballot_sync(FULL, lane == 0 || base != prev);
+      const unsigned firsts0 = __ballot_sync(FULL, lane == 0 || bin0 != prev0);
+      const int head = 31 - __clz(firsts & upto);
+      const int g = __popc(bal & ((1u << head) - 1u));
+      const unsigned later = firsts0 & ~upto;
+      const int next = later ? __ffs(later) - 1 : 31;
+      if (lane < Q_NR) {
+        s_grp[f_of][lane] = g;
+        s_gend[f_of][lane] = __popc(bal & ((1u << next) - 1u));
+        s_off[f_of][lane] = (bal >> head) & 1u;  // whether the rank is in a group
+      }
+      if (mixed) {
+        s_glo[f_of][g] = a;
+        s_ghi[f_of][g] = b;
+        s_gmul[f_of][g] = q_mul(b - a, Q_SUB);
+      }
+    }
+    if (!__syncthreads_or(mixed)) break;
+    clear(Q_SUB_WORDS + 12 * Q_SUB);
+    __syncthreads();
+    // group and step of a key, as f * 12 + group and 0 .. Q_SUB - 1; -1: none
+    auto sub_of = [&](int f, uint32_t key, int& at) -> int {
+      const uint32_t m = mark_of(f, key);
+      if (m == 0u || m == COLLECT) return -1;
+      for (int g = s_grp[f][m - 1]; g < s_gend[f][m - 1]; ++g)
+        if (key >= s_glo[f][g] && key <= s_ghi[f][g]) {
+          at = f * 12 + g;
+          return (int)q_step(key - s_glo[f][g], s_gmul[f][g]);
+        }
+      return -1;
+    };
+    each_key(once, [&](int f, uint32_t key) {
+      int at;
+      const int s = sub_of(f, key, at);
+      if (s >= 0) atomicAdd(dyn + at * (Q_SUB + 1) + s, 1u);
+    });
+    __syncthreads();
+    if ((warp & 1) == 0) {
+      const int at = f_of * 12 + s_grp[f_of][j_of];
+      const bool in = s_off[f_of][j_of] != 0;
+      const uint32_t r = s_rank[j_of];
+      uint32_t c = s_base[f_of][j_of], base = c, cnt = 0;
+      uint8_t* m = nullptr;
+      if (in)
+        for (int i = 0; i < Q_SUB; ++i) {
+          const uint32_t n = dyn[at * (Q_SUB + 1) + i];
+          if (r >= c && r < c + n) {
+            m = sub_mark + at * Q_SUB + i;
+            base = c;
+            cnt = n;
+          }
+          c += n;
+        }
+      __syncwarp();
+      settle(base, cnt, m);
+    }
+    __syncthreads();
+    each_key(once, [&](int f, uint32_t key) {
+      int at;
+      const int s = sub_of(f, key, at);
+      if (s >= 0) take(f, key, sub_mark[at * Q_SUB + s]);
+    });
+  }
+
+  idle();
+  if ((warp & 1) == 0) {  // where the collected keys of each rank's bin start
+    const uint32_t base = s_base[f_of][j_of], cnt = s_cnt[f_of][j_of];
+    const uint32_t prev = __shfl_up_sync(FULL, base, 1);
+    const bool few = cnt <= (uint32_t)Q_FEW;
+    uint32_t x = few && lane < Q_NR && (lane == 0 || base != prev) ? cnt : 0u;
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(FULL, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane < Q_NR) s_off[f_of][lane] = few ? (int)(x - cnt) : -1;
+  }
+  const uint32_t nmax = max(max(s_n[0], s_n[1]), max(s_n[2], s_n[3]));
+  if (nmax <= (uint32_t)Q_SMALL) {
+    const int f = warp >> 1, half = warp & 1;
+    uint32_t* col = cand + f * Q_CAND + half * 128 + lane * 4;
+    uint32_t v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      v[e] = (uint32_t)(half * 128 + lane * 4 + e) < s_n[f] ? col[e] : 0xffffffffu;
+    q_sort256_pair(v, half, lane, qx[f], 1 + f);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) col[e] = v[e];
+  } else {
+    for (int i = tid; i < 4 * Q_CAND; i += Q_NT)
+      if ((uint32_t)(i % Q_CAND) >= s_n[i / Q_CAND]) cand[i] = 0xffffffffu;
+    __syncthreads();
+    q_bitonic<Q_CAND / 64>(cand, 9);
+  }
+  __syncthreads();
+  if (tid < Q_NS) {
+    const int f = tid / Q_NQ, lv = tid - f * Q_NQ;
+    float x[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      int j = 2 * lv + e;
+      if (s_off[f][j] >= 0) {
+        x[e] = q_unkey(cand[f * Q_CAND + s_off[f][j] + (int)(s_rank[j] - s_base[f][j])]);
+      } else {
+        while (j > 0 && s_base[f][j - 1] == s_base[f][j]) --j;
+        x[e] = q_unkey(s_lo[f][j]);
+      }
+    }
+    const int64_t num = (int64_t)q_level_a[lv] * (T - 1);
+    const int b = q_level_b[lv], rem = (int)(num % b);
+    *out = rem ? x[0] + ((float)rem / (float)b) * (x[1] - x[0]) : x[0];
+  }
+}
+
 __global__ void __launch_bounds__(Q_NT, 3) qmlp_requests(const QArgs a) {
-  extern __shared__ __align__(16) uint32_t qs[];  // [4][n2] keys (shared-memory path)
+  extern __shared__ __align__(16) uint32_t qs[];  // Q_DYN words
   __shared__ float qv[Q_NS];
   __shared__ float h1[Q_H], h2[Q_H];
-  __shared__ uint32_t hist[256], bcast[2], wfl[Q_NT / 32];
+  __shared__ uint32_t wfl[Q_NT / 32];
   __shared__ uint32_t qx[4][Q_SMALL];  // exchange between the two warps of a column
   __shared__ float zpart[2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -263,13 +544,17 @@ __global__ void __launch_bounds__(Q_NT, 3) qmlp_requests(const QArgs a) {
   }
   const int T = (int)(hi - lo);
   // the MLP's weights, fetched now (coalesced) so that their latency overlaps
-  // the key loads and the sort
+  // the key loads and the sort; a selection, whose records take the registers,
+  // fetches them before it sorts
   float wr[QW_PER_T];
+  auto fetch_w = [&]() {
 #pragma unroll
-  for (int i = 0; i < QW_PER_T; ++i) {
-    const int g = tid + i * Q_NT;
-    wr[i] = g < QW_SIZE ? __ldg(a.w + g) : 0.f;
-  }
+    for (int i = 0; i < QW_PER_T; ++i) {
+      const int g = tid + i * Q_NT;
+      wr[i] = g < QW_SIZE ? __ldg(a.w + g) : 0.f;
+    }
+  };
+  if (T <= Q_MID) fetch_w();
   if (T == 0) {
     if (tid == 0) {
       a.score[r] = 0.f;
@@ -323,7 +608,7 @@ __global__ void __launch_bounds__(Q_NT, 3) qmlp_requests(const QArgs a) {
       if (rem) q = xl + ((float)rem / (float)b) * (q_unkey(col[lo_i + 1]) - xl);
       qv[tid] = q;
     }
-  } else if (T <= Q_CAP) {
+  } else if (T <= Q_MID) {
     int ln2 = 9;  // n2 = 2^ln2 >= T, at least 512
     while ((1 << ln2) < T) ++ln2;
     const int n2 = 1 << ln2;
@@ -346,31 +631,8 @@ __global__ void __launch_bounds__(Q_NT, 3) qmlp_requests(const QArgs a) {
       qs[3 * n2 + t] = k3;
     }
     __syncthreads();
-    if (ln2 == 9) {
-      q_bitonic<8>(qs, 9);
-    } else if (ln2 == 10) {
-      q_bitonic<16>(qs, 10);
-    } else {  // 2,048 keys per column: shared-memory stages (32 keys per thread
-              // would take the registers that the other requests' CTAs need)
-      const int half = n2 >> 1, lh = ln2 - 1;
-      for (int k = 2; k <= n2; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-          for (int idx = tid; idx < 4 * half; idx += Q_NT) {
-            const int f = idx >> lh, t = idx & (half - 1);
-            const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
-            const int l = i + j;
-            uint32_t* col = qs + (f << ln2);
-            const uint32_t x = col[i], y = col[l];
-            const bool up = (i & k) == 0;
-            if ((x > y) == up) {
-              col[i] = y;
-              col[l] = x;
-            }
-          }
-          __syncthreads();
-        }
-      }
-    }
+    if (ln2 == 9) q_bitonic<8>(qs, 9);
+    else q_bitonic<16>(qs, 10);
     __syncthreads();
     if (tid < Q_NS) {
       const int f = tid / Q_NQ, j = tid - f * Q_NQ;
@@ -387,19 +649,7 @@ __global__ void __launch_bounds__(Q_NT, 3) qmlp_requests(const QArgs a) {
       qv[tid] = q;
     }
   } else {
-    for (int f = 0; f < 4; ++f)
-      for (int j = 0; j < Q_NQ; ++j) {
-        const int64_t num = (int64_t)q_level_a[j] * (T - 1);
-        const int b = q_level_b[j];
-        const int lo_i = (int)(num / b), rem = (int)(num - (int64_t)lo_i * b);
-        const float xl = q_unkey(q_select(a.feat, lo, T, f, lo_i, hist, bcast));
-        float q = xl;
-        if (rem) {
-          const float xh = q_unkey(q_select(a.feat, lo, T, f, min(lo_i + 1, T - 1), hist, bcast));
-          q = xl + ((float)rem / (float)b) * (xh - xl);
-        }
-        if (tid == 0) qv[f * Q_NQ + j] = q;
-      }
+    q_select(a.feat, lo, T, qs, qx, qv + min(tid, Q_NS - 1), fetch_w);
   }
   __syncthreads();
 

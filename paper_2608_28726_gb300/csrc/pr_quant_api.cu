@@ -40,7 +40,12 @@ pr_status pr_quantile_score(pr_ctx* c, const float* feat, const uint32_t* row_fl
   a.ship = ship;
   a.req_flags = req_flags;
   a.ctx_flags = c->flags;
-  prk::qmlp_requests<<<(unsigned)n_req, prk::Q_NT, 4 * prk::Q_CAP * sizeof(uint32_t), s>>>(a);
+  if (!c->qmlp_ready) {
+    PR_CUDA(cudaFuncSetAttribute(prk::qmlp_requests, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(prk::Q_DYN * sizeof(uint32_t))));
+    c->qmlp_ready = true;
+  }
+  prk::qmlp_requests<<<(unsigned)n_req, prk::Q_NT, prk::Q_DYN * sizeof(uint32_t), s>>>(a);
   PR_CUDA(cudaGetLastError());
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return timing_mark(c, s);

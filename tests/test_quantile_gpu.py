@@ -58,9 +58,33 @@ def check(B, ctx, feat, offsets, tau=0.5, row_flags=None, seed=6001):
 
 
 def test_quantile_lengths_both_paths(B, ctx):
-    # 1 .. 2,048 rows sort in shared memory; 2,049 and 5,000 use radix selection
+    # up to 256 rows sort in registers, up to 1,024 in shared memory, longer ones select
     lengths = [1, 2, 3, 10, 11, 31, 32, 33, 257, 1000, 2048, 2049, 5000]
     feat, offsets = workloads.head_features(lengths, 7100)
+    check(B, ctx, feat, offsets)
+
+
+@pytest.mark.parametrize("T", [1024, 1025, 2047, 2048, 2049, 4097, 9000])
+@pytest.mark.parametrize("values", ["plain", "ties", "constant", "clusters", "near_ties"])
+def test_quantile_selection(B, ctx, T, values):
+    """The selection of long requests: both sides of its smallest length and of
+    the rows held in registers, and values that crowd its histogram bins (a
+    few levels; one; clusters far apart, inside which all keys differ; runs of
+    neighbouring floats)."""
+    feat, offsets = workloads.head_features([T, 40, T + 3], 7300 + T)
+    used = [0, 1, 4]
+    if values == "ties":
+        feat[:, used] = np.round(feat[:, used] * 8) / 8
+    elif values == "constant":
+        feat[:, used] = np.float32(-0.25)
+    elif values == "clusters":
+        feat[:, used] = 0.5 + 1e-3 * feat[:, used]
+        feat[::97, used] = -3e30
+        feat[5::301, used] = 3e30
+    elif values == "near_ties":
+        bits = np.float32(0.75).view(np.uint32) + np.arange(len(feat)) % 700
+        feat[:, used] = bits.astype(np.uint32).view(np.float32)[:, None]
+        feat[7::500, used] = 0.0
     check(B, ctx, feat, offsets)
 
 
