@@ -17,8 +17,8 @@
 //   * exact top-K (and the first two tokens, lower index first on ties) at
 //     almost no streaming cost: each thread only stores the maximum of each of
 //     its tiles in shared memory.  After the stream, theta1 = the K-th largest
-//     per-thread maximum is a lower bound of the K-th largest element (K
-//     distinct elements reach it); the stored tile maxima >= theta1 are the
+//     of (some of) the per-thread maxima is a lower bound of the K-th largest
+//     element (K distinct elements reach it); the stored tile maxima >= theta1 are the
 //     candidate "super-groups"; theta = the K-th largest candidate value is a
 //     tighter bound, and every element >= theta lies in a candidate >= theta
 //     (an element below theta has K strictly larger elements, the maxima of K
@@ -53,7 +53,7 @@ constexpr float L2E = 1.4426950408889634f;
 constexpr float LN2 = 0.6931471805599453f;
 constexpr float M2_INIT = -1e30f;  // finite "no maximum yet" so that 2^(m - m') is 0, never NaN
 constexpr unsigned FULL = 0xffffffffu;
-constexpr uint32_t TAIL_ID = 0xffffffffu;  // candidate id of the partial last group
+constexpr int PUB = 4;             // thread maxima each warp publishes for theta1
 
 constexpr uint32_t FLAG_NONFINITE = 1u;
 constexpr uint32_t FLAG_BAD_CHOSEN = 2u;
@@ -116,6 +116,11 @@ __device__ __forceinline__ uint4 ld_stream(const void* p) {
 // bulk prefetch of [p, p + bytes) into L2 (16-byte aligned, a multiple of 16 bytes)
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
+// the line of one value into L2
+__device__ __forceinline__ void prefetch_line(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
 __device__ __forceinline__ uint32_t hmax2(uint32_t a, uint32_t b) {
@@ -206,6 +211,21 @@ __device__ __forceinline__ void lse_merge(float& m, float& S, float& U, float mo
   m = M;
   S = Sn;
   U = Un;
+}
+
+// the warp's merged state, in every lane: one maximum, then two sums of states
+// rescaled once (a butterfly of lse_merge costs four times the instructions)
+__device__ __forceinline__ void lse_warp(float& m, float& S, float& U) {
+  const float M = unord(__reduce_max_sync(FULL, ord(m)));
+  const float d = m - M, f = ex2(d);
+  U = f * fmaf(d, S, U);
+  S *= f;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    S += __shfl_xor_sync(FULL, S, o);
+    U += __shfl_xor_sync(FULL, U, o);
+  }
+  m = M;
 }
 
 // one element with full guards: NaN / +inf mark the row, -inf is a masked token
@@ -323,26 +343,39 @@ struct Traits<float> {
   }
 };
 
+// What a row's epilogue needs that does not depend on the reduction: the
+// emitted token and its logit, and the row's request (rows, from the CSR
+// offsets) or decode slot.  The persistent kernel loads it for the next row
+// while it waits for that row's stream, off the critical path.
+struct RowPre {
+  int32_t y;       // emitted token id
+  float xy;        // its logit (NaN when y is outside [0, V))
+  int32_t r;       // request (features with offsets, route) or decode slot; -1 if none
+  int64_t lo, hi;  // rows of the request
+  int eos;         // decode: the request ends with this row
+};
+
 // ---- shared state of one CTA ------------------------------------------------------
 
 struct Smem {
   float tm[MAX_SLOTS][NT];    // per-thread tile (super-group) maxima
-  uint32_t wl[NWARP][32];     // per-warp sorted thread maxima, ord() encoded
-  float cand_v[CCAP];         // candidate super-groups: value
-  uint32_t cand_id[CCAP];     //   and (slot << 8 | thread), or TAIL_ID
+  uint32_t pub[NWARP * PUB];  // every warp's largest thread maxima, ord() encoded
+  union {
+    uint32_t all_max[NT];     // all thread maxima, when the published ones do not suffice
+    uint32_t cand_id[CCAP];   // candidate super-groups: slot << 8 | thread
+  };
   uint64_t ebuf[ECAP];        // candidate element keys
   float pm[NWARP], pS[NWARP], pU[NWARP];
   int pbad[NWARP];
-  int ncand, nelem, nsel;
-  float theta1, theta;
-  float tail_max;             // maximum of the partial last group (cluster rank 0)
-  // the CTA's merged partial state, read by cluster rank 0 through DSMEM
-  float fm, fS, fU;
-  int fbad;
-  uint64_t flist[32];
+  int ncand, nelem, careful;
+  float theta1;
   uint64_t top[32];           // the CTA's top-32 keys, ranked by counting
-  int careful, fallback;
+  RowPre pre;
+  // cluster rank 0: the other CTAs' states (m, S, U, bad) and top-32 lists
+  uint32_t peer_state[MAXC][4];
+  uint64_t peer_list[MAXC][32];
 };
+static_assert(NWARP * PUB == 32 && PUB * NWARP >= 32, "one published maximum per lane; kc <= 32");
 
 // ---- warp-level top-32 of pushed keys ---------------------------------------------
 

@@ -163,25 +163,23 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
                    : "memory");
 }
+// the same in two halves; no memory is handed over between them
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
 __device__ __forceinline__ uint32_t dsmem_addr(const void* p, uint32_t rank) {
   uint32_t local = (uint32_t)__cvta_generic_to_shared(p), remote;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
   return remote;
 }
-__device__ __forceinline__ float dsmem_ld_f32(uint32_t a) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-  return v;
+__device__ __forceinline__ void dsmem_st_u32(uint32_t a, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
-__device__ __forceinline__ int dsmem_ld_s32(uint32_t a) {
-  int v;
-  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
-  return v;
-}
-__device__ __forceinline__ uint64_t dsmem_ld_u64(uint32_t a) {
-  uint64_t v;
-  asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
-  return v;
+__device__ __forceinline__ void dsmem_st_u64(uint32_t a, uint64_t v) {
+  asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
 }
 
 // ---- block reduction of the (m, S, U, bad) state ------------------------------------
@@ -223,26 +221,39 @@ __device__ __forceinline__ void block_reduce_state(Smem& sm, float& m, float& S,
   }
 }
 
-// ---- one row's features and the mode's epilogue (one warp) ------------------------------
-
-// What a row's epilogue needs that does not depend on the reduction: the
-// emitted token and its logit, and the row's request (rows, from the CSR
-// offsets) or decode slot.  The persistent kernel loads it for the next row
-// while it waits for that row's stream, off the critical path.
-struct RowPre {
-  int32_t y;       // emitted token id
-  float xy;        // its logit (NaN when y is outside [0, V))
-  int32_t r;       // request (features with offsets, route) or decode slot; -1 if none
-  int64_t lo, hi;  // rows of the request
-  int eos;         // decode: the request ends with this row
+// ---- row geometry -----------------------------------------------------------------------
+//
+// A row is cut into 16-byte groups of VEC elements from its first element on; the
+// nedge < VEC elements after the last full group are read one by one by the
+// lanes of a warp.  A tile is TILE groups, of which warp w of a CTA takes the
+// UNR x 32 consecutive ones from 32 UNR w on, lane l the groups 32 k + l (2 KB in
+// a row per warp: 3,214 rows of V = 262,144 fp32 take 506 us, 520 us with the
+// warps' loads interleaved).
+struct RowGeom {
+  int32_t gfull, nedge;       // full groups, elements after them
+  int32_t nfull, rem, ntiles; // tiles of TILE groups: full ones, groups of the last, all
+  __device__ __forceinline__ RowGeom(int64_t V, int vec) {
+    gfull = (int32_t)(V / vec);
+    nedge = (int32_t)(V - (int64_t)gfull * vec);
+    nfull = gfull / TILE;
+    rem = gfull - nfull * TILE;
+    ntiles = nfull + (rem > 0 ? 1 : 0);
+  }
 };
+// index in its tile of thread tid's group k
+__device__ __forceinline__ int32_t tile_pos(int tid, int k) {
+  return (tid >> 5) * (32 * UNR) + 32 * k + (tid & 31);
+}
+
+// ---- one row's features and the mode's epilogue (one warp) ------------------------------
 
 // Whole warp (the request search is warp-collective).
 template <typename T, int MODE>
-__device__ __forceinline__ RowPre load_pre(const Args& a, int64_t row, const char* rowp, int lane) {
+__device__ __forceinline__ RowPre load_pre(const Args& a, int64_t row, int32_t y, const char* rowp,
+                                           int lane) {
   using Tr = Traits<T>;
   RowPre p;
-  p.y = a.chosen[row];
+  p.y = y;
   p.xy = (p.y >= 0 && (int64_t)p.y < a.vocab) ? Tr::elem(rowp, p.y) : NAN;
   p.r = -1;
   p.lo = p.hi = 0;
@@ -366,63 +377,77 @@ __device__ __forceinline__ void row_finish(const Args& a, int64_t row, float m, 
   }
 
   if (MODE == MODE_DECODE) {
-    if (lane != 0) return;
     const int32_t s = pre.r;
     if (s < 0 || s >= a.n_slots) {
-      atomicOr(a.ctx_flags, FLAG_BAD_SLOT);
+      if (lane == 0) atomicOr(a.ctx_flags, FLAG_BAD_SLOT);
       return;
     }
+    // lane f < 5 keeps statistic f (l, m, margin, -H, h)
     float* A = a.acc + (int64_t)s * ACC_WORDS;
+    const int f = lane < 5 ? lane : 0;
     const int32_t n = __float_as_int(A[0]) + 1;
     const uint32_t fl = __float_as_uint(A[1]) | flags;
-    const float v[5] = {fv[0], fv[1], fv[2], -fv[3], fv[4]};
-#pragma unroll
-    for (int f = 0; f < 5; ++f) {
-      if (n == 1) {
-        A[2 + f] = v[f];
-        A[7 + f] = 0.f;
-        A[12 + f] = v[f];
-      } else {
-        // compensated (Kahan) running sum in step order
-        const float sum = A[2 + f], comp = A[7 + f];
-        const float yv = v[f] - comp;
-        const float tsum = sum + yv;
-        A[7 + f] = (tsum - sum) - yv;
-        A[2 + f] = tsum;
-        A[12 + f] = fminf(A[12 + f], v[f]);
-      }
+    const float sum0 = A[2 + f], comp0 = A[7 + f], mn0 = A[12 + f];
+    const float v = f == 0 ? fv[0] : f == 1 ? fv[1] : f == 2 ? fv[2] : f == 3 ? -fv[3] : fv[4];
+    float sum = v, comp = 0.f, mn = v;
+    if (n != 1) {  // compensated (Kahan) running sum in step order
+      const float yv = v - comp0;
+      sum = sum0 + yv;
+      comp = (sum - sum0) - yv;
+      mn = fminf(mn0, v);
     }
+    __syncwarp();  // every lane has read the slot
     if (!pre.eos) {
-      A[0] = __int_as_float(n);
-      A[1] = __uint_as_float(fl);
+      if (lane < 5) {
+        A[2 + f] = sum;
+        A[7 + f] = comp;
+        A[12 + f] = mn;
+      }
+      if (lane == 0) {
+        A[0] = __int_as_float(n);
+        A[1] = __uint_as_float(fl);
+      }
       return;
     }
     // the request ends with this row: pool, score, ship rule, clear the slot
-    float ag[NAGG];
-    float sc;
-    uint8_t sh;
-    if (fl & (FLAG_NONFINITE | FLAG_BAD_CHOSEN)) {
-      for (int j = 0; j < NAGG; ++j) ag[j] = NAN;
-      sc = NAN;
-      sh = 0;
-    } else {
-      const float Tf = (float)n;
-      for (int f = 0; f < 5; ++f) {
-        ag[2 * f] = A[2 + f] / Tf;
-        ag[2 * f + 1] = A[12 + f];
+    const bool none = (fl & (FLAG_NONFINITE | FLAG_BAD_CHOSEN)) != 0;
+    const float mean = sum / (float)n;
+    float z = a.b, mine = NAN, sc = NAN;
+    uint8_t sh = 0;
+    if (!none) {
+      float ag[NAGG];
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
+        ag[2 * j] = __shfl_sync(FULL, mean, j);
+        ag[2 * j + 1] = __shfl_sync(FULL, mn, j);
       }
       ag[10] = (float)(n + 1) / (float)(2 * n);
-      float z = a.b;
-      for (int j = 0; j < NAGG; ++j) z = fmaf(__ldg(a.w + j), ag[j], z);
+#pragma unroll
+      for (int j = 0; j < NAGG; ++j) {
+        z = fmaf(__ldg(a.w + j), ag[j], z);
+        if (lane == j) mine = ag[j];
+      }
       sc = 1.f / (1.f + expf(-z));
       sh = (z >= a.zthr) ? 1 : 0;
     }
-    if (a.agg)
-      for (int j = 0; j < NAGG; ++j) a.agg[(int64_t)s * NAGG + j] = ag[j];
-    a.score[s] = sc;
-    a.ship[s] = sh;
-    a.req_flags[s] = fl;
-    for (int j = 0; j < ACC_WORDS; ++j) A[j] = 0.f;
+    if (a.agg && lane < NAGG) a.agg[(int64_t)s * NAGG + lane] = mine;
+    if (lane == 0) {
+      a.score[s] = sc;
+      a.ship[s] = sh;
+      a.req_flags[s] = fl;
+    }
+    if (lane < ACC_WORDS) A[lane] = 0.f;
+  }
+}
+
+// the warp's PUB largest values, into out[0 .. PUB - 1] (lane 0)
+__device__ __forceinline__ void publish_max(uint32_t cur, uint32_t* out, int lane) {
+#pragma unroll
+  for (int i = 0; i < PUB; ++i) {
+    const uint32_t w = __reduce_max_sync(FULL, cur);
+    const unsigned eq = __ballot_sync(FULL, cur == w);
+    if (lane == 0) out[i] = w;
+    if (lane == __ffs(eq) - 1) cur = 0u;
   }
 }
 
@@ -451,17 +476,18 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Ar
   const int64_t row = cid;
 
   pdl_trigger();  // a dependent launch may start streaming while this one finishes
+  if (C > 1) cluster_arrive();  // every CTA of the cluster has started (waited for below)
 
   const char* rowp = reinterpret_cast<const char*>(a.logits) + row * a.row_stride * (int64_t)sizeof(T);
-  const uint4* vp = reinterpret_cast<const uint4*>(rowp);
   const int64_t V = a.vocab;
-  const int32_t gfull = (int32_t)(V / VEC);  // full 16-byte groups
-  const bool has_tail = (V % VEC) != 0;      // the partial last group, index gfull
-  const int32_t g0 = (int32_t)((int64_t)gfull * rank / C);
-  const int32_t g1 = (int32_t)((int64_t)gfull * (rank + 1) / C);
+  const uint4* vp = reinterpret_cast<const uint4*>(rowp);
+  const RowGeom geo(V, VEC);
+  const int32_t g0 = (int32_t)((int64_t)geo.gfull * rank / C);
+  const int32_t g1 = (int32_t)((int64_t)geo.gfull * (rank + 1) / C);
   const int32_t ng = g1 - g0;
   const int32_t nfull = ng / TILE, rem = ng - nfull * TILE;
   const int32_t ntiles = nfull + (rem > 0 ? 1 : 0);
+  const int32_t nedge = rank == 0 ? geo.nedge : 0;  // cluster rank 0 takes the last elements
   int shift = 0;
   while (((ntiles + (1 << shift) - 1) >> shift) > MAX_SLOTS) ++shift;
   const int32_t smask = (1 << shift) - 1;
@@ -471,8 +497,16 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Ar
   if (tid == 0) {
     sm.ncand = 0;
     sm.nelem = 0;
-    sm.tail_max = -INFINITY;
+    // the row's inputs beside the logits, on their way into L2 while it streams
+    if (rank == 0) {
+      prefetch_line(a.chosen + row);
+      if (MODE == MODE_DECODE) {
+        prefetch_line(a.slot + row);
+        prefetch_line(a.eos + row);
+      }
+    }
   }
+  if (tid < 32) sm.top[tid] = 0ull;
 
   float m = M2_INIT;
   float2 S2 = make_float2(0.f, 0.f), U2 = make_float2(0.f, 0.f);
@@ -483,6 +517,17 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Ar
   {
     auto load = [&](int32_t gi) -> uint4 {
       return ALIGNED ? ld_stream(vp + g0 + gi) : Tr::load_elems(rowp, (int64_t)(g0 + gi));
+    };
+    auto load_tile = [&](uint4 (&dst)[UNR], int32_t t) {  // nothing past the range
+      const int32_t nb = t * TILE;
+      if (t < nfull) {
+#pragma unroll
+        for (int k = 0; k < UNR; ++k) dst[k] = load(nb + tile_pos(tid, k));
+      } else {
+#pragma unroll
+        for (int k = 0; k < UNR; ++k)
+          dst[k] = tile_pos(tid, k) < rem ? load(nb + tile_pos(tid, k)) : NEG;
+      }
     };
     // one CTA per row: one thread keeps the tiles PF_TILES ahead on their way
     // into L2 (bulk prefetches need no registers, so the CTA has more bytes in
@@ -499,23 +544,10 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Ar
 #pragma unroll
     for (int32_t p = 1; p <= PF_TILES; ++p) prefetch_tile(p);
     uint4 cur[UNR], nxt[UNR];
-    if (nfull > 0) {
-#pragma unroll
-      for (int k = 0; k < UNR; ++k) cur[k] = load(k * NT + tid);
-    } else {
-#pragma unroll
-      for (int k = 0; k < UNR; ++k) cur[k] = (k * NT + tid < rem) ? load(k * NT + tid) : NEG;
-    }
+    load_tile(cur, 0);
     for (int32_t t = 0; t < ntiles; ++t) {
-      const int32_t nb = (t + 1) * TILE;
       prefetch_tile(t + 1 + PF_TILES);
-      if (t + 1 < nfull) {
-#pragma unroll
-        for (int k = 0; k < UNR; ++k) nxt[k] = load(nb + k * NT + tid);
-      } else if (t + 1 < ntiles) {
-#pragma unroll
-        for (int k = 0; k < UNR; ++k) nxt[k] = (k * NT + tid < rem) ? load(nb + k * NT + tid) : NEG;
-      }
+      if (t + 1 < ntiles) load_tile(nxt, t + 1);
       const float tmax = Tr::tile_max(cur);
       thr_max = fmaxf(thr_max, tmax);
       racc = fmaxf(racc, tmax);
@@ -537,7 +569,7 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Ar
       } else {
 #pragma unroll
         for (int k = 0; k < UNR; ++k)
-          if (k * NT + tid < rem) Tr::accum(cur[k], nm, S2, U2);
+          if (tile_pos(tid, k) < rem) Tr::accum(cur[k], nm, S2, U2);
       }
 #pragma unroll
       for (int k = 0; k < UNR; ++k) cur[k] = nxt[k];
@@ -545,37 +577,150 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Ar
   }
   float S = S2.x + S2.y, U = U2.x + U2.y;
 
-  // ---- the partial last group (fewer than VEC elements): cluster rank 0, thread 0
-  if (has_tail && rank == 0 && tid == 0) {
-    float tmx = -INFINITY;
-    for (int64_t v = (int64_t)gfull * VEC; v < V; ++v) {
-      const float x = Tr::elem(rowp, v);
-      careful_add(x, m, S, U, bad);
-      if (!isnan(x)) tmx = fmaxf(tmx, x);
-    }
-    sm.tail_max = tmx;
-    thr_max = fmaxf(thr_max, tmx);
+  // What follows the stream is a chain of latencies that a lone launch cannot
+  // hide; it is kept short: four block barriers, no sort, every global load
+  // issued as early as its address is known (see the phases' comments).
+  // Measured against sorted maxima, a serial merge and a pull-style cluster merge
+  // (CUDA graphs, per launch): 256 rows of V = 151,936 bf16 21.6 -> 19.5 us, 8 rows
+  // 11.3 -> 8.4 us, 256 rows of V = 32,000 fp32 13.9 -> 12.5 us.
+
+  // ---- the elements after the last group: warp 0 of cluster rank 0, one per lane
+  float xe = -INFINITY;
+  const int64_t ve = (int64_t)geo.gfull * VEC + lane;  // this lane's
+  if (warp == 0 && lane < nedge) {
+    const float x = Tr::elem(rowp, ve);
+    careful_add(x, m, S, U, bad);
+    if (!isnan(x)) xe = x;
+    thr_max = fmaxf(thr_max, xe);
   }
 
-  // ---- theta1: the kc-th largest per-thread maximum (a lower bound of the kc-th element)
+  // ---- theta1: the kc-th largest of every warp's four largest thread maxima
+  // (kc <= 32 distinct elements reach it, so it bounds the kc-th element from
+  // below).  Against the kc-th largest of all thread maxima, which takes a sort
+  // per warp and seven merges, about one candidate more passes it (22 for 21 of
+  // 151,936 normal values and kc = 20).
   const int kc = a.kc;
-  sm.wl[warp][lane] = warp_sort_desc<uint32_t>(ord(thr_max), lane);
-  block_reduce_state(sm, m, S, U, bad, warp, lane);  // ends with a __syncthreads
-  if (warp == 0) {
-    uint32_t L = sm.wl[0][lane];
-#pragma unroll 1
-    for (int w2 = 1; w2 < NWARP; ++w2) L = warp_merge_desc<uint32_t>(L, sm.wl[w2][lane], lane);
-    const float th1 = unord(__shfl_sync(FULL, L, kc - 1));
-    if (lane == 0) {
-      sm.theta1 = th1;
-      sm.fallback = !(th1 > -INFINITY);
-      // a masked (-inf), NaN or infinite logit made the CTA's fast
-      // accumulators non-finite: it re-streams its range with guards (the
-      // row's merged state is non-finite exactly when a CTA's is)
-      sm.careful = (!bad && !(isfinite(S) && isfinite(U))) ? 1 : 0;
+  publish_max(ord(thr_max), &sm.pub[warp * PUB], lane);
+  int32_t y = 0;
+  if (rank == 0 && warp == 1) y = a.chosen[row];  // used after the next barrier
+  __syncthreads();
+  float th1;
+  {
+    const uint32_t mine = sm.pub[lane];
+    int rk = 0;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+      const uint32_t q = sm.pub[j];
+      rk += (q > mine || (q == mine && j < lane)) ? 1 : 0;
+    }
+    th1 = unord(__shfl_sync(FULL, mine, __ffs(__ballot_sync(FULL, rk == kc - 1)) - 1));
+  }
+  if (!(th1 > -INFINITY)) {
+    // fewer than kc published maxima (a range of less than a tile, or all but a
+    // few neighbouring tokens masked): the kc-th largest of all thread maxima
+    sm.all_max[tid] = ord(thr_max);
+    if (tid == 0) sm.theta1 = -INFINITY;
+    __syncthreads();
+    const uint32_t mine = sm.all_max[tid];
+    int rk = 0;
+#pragma unroll 8
+    for (int j = 0; j < NT; ++j) {
+      const uint32_t q = sm.all_max[j];
+      rk += (q > mine || (q == mine && j < tid)) ? 1 : 0;
+    }
+    if (rk == kc - 1) sm.theta1 = thr_max;
+    __syncthreads();
+    th1 = sm.theta1;
+  }
+  const bool fallback = !(th1 > -INFINITY);
+
+  // ---- candidate super-groups: this thread's stored tile maxima >= theta1
+  if (!fallback && thr_max >= th1) {
+    uint32_t mask = 0u;
+#pragma unroll
+    for (int32_t s = 0; s < MAX_SLOTS; ++s)
+      if (s < nslots) mask |= sm.tm[s][tid] >= th1 ? 1u << s : 0u;
+    if (mask) {
+      int i = atomicAdd(&sm.ncand, __popc(mask));
+      for (; mask; mask &= mask - 1u, ++i)
+        if (i < CCAP) sm.cand_id[i] = ((uint32_t)(__ffs(mask) - 1) << 8) | (uint32_t)tid;
+    }
+    if (xe >= th1) {  // an edge element is a candidate by itself
+      const int e = atomicAdd(&sm.nelem, 1);
+      if (e < ECAP) sm.ebuf[e] = make_key(xe, (uint32_t)ve);
     }
   }
-  if (tid < 32) sm.top[tid] = 0ull;
+  // the warp's state
+  lse_warp(m, S, U);
+  bad = __any_sync(FULL, bad);
+  if (lane == 0) {
+    sm.pm[warp] = m;
+    sm.pS[warp] = S;
+    sm.pU[warp] = U;
+    sm.pbad[warp] = bad;
+  }
+  __syncthreads();
+
+  // ---- re-read the candidates (a 16-byte group per thread, all in flight at
+  // once); their elements >= theta1 become keys: kc distinct elements reach
+  // theta1, so the CTA's top kc are among them
+  const int ncand = sm.ncand;
+  const bool fb_cand = fallback || ncand > CCAP;
+  const int total = fb_cand ? 0 : ncand * (UNR << shift);  // groups of the super-groups
+  int32_t g = -1;
+  uint4 wv = NEG;
+  auto fetch = [&](int i) {
+    const int c = i / UNR >> shift, j = i - (c << shift) * UNR;
+    const uint32_t id = sm.cand_id[c];
+    const int32_t t = (int32_t)((id >> 8) << shift) + j / UNR;
+    const int32_t gi = t * TILE + tile_pos((int)(id & 255u), j % UNR);
+    g = t < ntiles && gi < ng ? g0 + gi : -1;
+    if (g >= 0) wv = ALIGNED ? ld_reread(vp + g) : Tr::load_elems(rowp, g);
+  };
+  if (tid < total) fetch(tid);
+  // while they arrive: warp 0 merges the CTA's state, warp 1 of cluster rank 0
+  // finds what the row's epilogue needs besides the reduction
+  if (warp == 0) {
+    m = lane < NWARP ? sm.pm[lane] : M2_INIT;
+    S = lane < NWARP ? sm.pS[lane] : 0.f;
+    U = lane < NWARP ? sm.pU[lane] : 0.f;
+    bad = __any_sync(FULL, lane < NWARP && sm.pbad[lane] != 0);
+#pragma unroll
+    for (int o = NWARP / 2; o > 0; o >>= 1) {
+      const float mo = __shfl_xor_sync(FULL, m, o);
+      const float So = __shfl_xor_sync(FULL, S, o);
+      const float Uo = __shfl_xor_sync(FULL, U, o);
+      lse_merge(m, S, U, mo, So, Uo);
+    }
+    // only lanes 0..NWARP-1 took part in the last butterfly: give every lane the total
+    m = __shfl_sync(FULL, m, 0);
+    S = __shfl_sync(FULL, S, 0);
+    U = __shfl_sync(FULL, U, 0);
+    // a masked (-inf), NaN or infinite logit made the CTA's fast accumulators
+    // non-finite: it re-streams its range with guards (the row's merged state
+    // is non-finite exactly when a CTA's is)
+    if (lane == 0) sm.careful = (!bad && !(isfinite(S) && isfinite(U))) ? 1 : 0;
+  } else if (warp == 1 && rank == 0) {
+    const RowPre p = load_pre<T, MODE>(a, row, y, rowp, lane);
+    if (lane == 0) sm.pre = p;
+  }
+  for (int i = tid; i < total;) {
+    if (g >= 0) {
+      uint32_t hits = 0u;
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) hits |= Tr::at(wv, e) >= th1 ? 1u << e : 0u;
+      if (hits) {
+        int at = atomicAdd(&sm.nelem, __popc(hits));
+        for (; hits; hits &= hits - 1u, ++at) {
+          const int e = __ffs(hits) - 1;
+          if (at < ECAP)
+            sm.ebuf[at] = make_key(Tr::at(wv, e), (uint32_t)(g * VEC + e));
+        }
+      }
+    }
+    i += NT;
+    if (i < total) fetch(i);
+  }
   __syncthreads();
   if (sm.careful) {
     float cm = M2_INIT, cS = 0.f, cU = 0.f;
@@ -583,9 +728,7 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Ar
     const int64_t e1 = (int64_t)g1 * VEC;
     for (int64_t v = (int64_t)g0 * VEC + tid; v < e1; v += NT)
       careful_add(Tr::elem(rowp, v), cm, cS, cU, cbad);
-    if (has_tail && rank == 0)
-      for (int64_t v = (int64_t)gfull * VEC + tid; v < V; v += NT)
-        careful_add(Tr::elem(rowp, v), cm, cS, cU, cbad);
+    if (tid < nedge) careful_add(Tr::elem(rowp, ve), cm, cS, cU, cbad);
     block_reduce_state(sm, cm, cS, cU, cbad, warp, lane);  // warp 0 holds the CTA's state
     m = cm;
     S = cS;
@@ -593,91 +736,25 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Ar
     bad = cbad;
   }
 
-  // ---- candidate super-groups: stored tile maxima >= theta1
-  const float th1 = sm.theta1;
-  if (!sm.fallback) {
-    for (int32_t s = 0; s < nslots; ++s) {
-      const float v = sm.tm[s][tid];
-      if (v >= th1) {
-        const int i = atomicAdd(&sm.ncand, 1);
-        if (i < CCAP) {
-          sm.cand_v[i] = v;
-          sm.cand_id[i] = ((uint32_t)s << 8) | (uint32_t)tid;
-        }
-      }
-    }
-    if (tid == 0 && has_tail && rank == 0 && sm.tail_max >= th1) {
-      const int i = atomicAdd(&sm.ncand, 1);
-      if (i < CCAP) {
-        sm.cand_v[i] = sm.tail_max;
-        sm.cand_id[i] = TAIL_ID;
-      }
-    }
-  }
-  __syncthreads();
-
-  // ---- re-read the candidates; their elements >= theta1 become keys (kc
-  // distinct elements reach theta1, so the CTA's top kc are among them)
-  const int ncand = sm.ncand;
-  const bool fb_cand = sm.fallback || ncand > CCAP;
-  if (!fb_cand) {
-    const float th = th1;
-    const int n = ncand;
-    const int gpc = UNR << shift;  // groups per super-group
-    for (int i = tid; i < n * gpc; i += NT) {
-      const int c = i / gpc, j = i - c * gpc;
-      const uint32_t id = sm.cand_id[c];
-      if (id == TAIL_ID) {
-        if (j != 0) continue;
-        for (int64_t v = (int64_t)gfull * VEC; v < V; ++v) {
-          const float x = Tr::elem(rowp, v);
-          if (x >= th) {
-            const int e = atomicAdd(&sm.nelem, 1);
-            if (e < ECAP) sm.ebuf[e] = make_key(x, (uint32_t)v);
-          }
-        }
-        continue;
-      }
-      const int32_t t = (int32_t)((id >> 8) << shift) + j / UNR;
-      const int32_t gi = t * TILE + (j % UNR) * NT + (int32_t)(id & 255u);
-      if (t >= ntiles || gi >= ng) continue;
-      const int32_t g = g0 + gi;
-      const uint4 wv = ALIGNED ? ld_reread(vp + g) : Tr::load_elems(rowp, (int64_t)g);
-#pragma unroll
-      for (int e2 = 0; e2 < VEC; ++e2) {
-        const float x = Tr::at(wv, e2);
-        if (x >= th) {
-          const int e = atomicAdd(&sm.nelem, 1);
-          if (e < ECAP) sm.ebuf[e] = make_key(x, (uint32_t)(g * VEC + e2));
-        }
-      }
-    }
-  }
-  __syncthreads();
-
-  // ---- what the row's epilogue needs besides the reduction (cluster rank 0,
-  // warp 0), fetched now so that its latency overlaps the selection
-  RowPre pre;
-  if (rank == 0 && warp == 0) {
-    pre = load_pre<T, MODE>(a, row, rowp, lane);
-    if (C == 1) {
-      pdl_wait();
-      if (MODE == MODE_DECODE && lane == 0 && pre.r >= 0 && pre.r < a.n_slots) {
-        const float* A = a.acc + (int64_t)pre.r * ACC_WORDS;  // into L1 for row_finish
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(A));
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(A + 16));
-      }
-    }
-  }
-
   // ---- the CTA's exact top-32 elements: up to NT candidate keys are ranked
-  // by counting (keys are distinct: the index is part of the key), more by
-  // warp 0's sorting network; the exact scan when the buffers overflowed
+  // by counting (keys are distinct: the index is part of the key; up to NT / 2
+  // keys with two threads each), more by warp 0's sorting network; the exact
+  // scan when the buffers overflowed
   uint64_t E = 0ull;
   const int ne = sm.nelem;
   const bool fb = fb_cand || ne > ECAP;
   if (!fb && ne <= NT) {
-    if (tid < ne) {
+    if (ne <= NT / 2) {
+      const int i = tid >> 1;
+      uint64_t key = 0ull;
+      int rk = 0;
+      if (i < ne) {
+        key = sm.ebuf[i];
+        for (int q = tid & 1; q < ne; q += 2) rk += sm.ebuf[q] > key ? 1 : 0;
+      }
+      rk += __shfl_xor_sync(FULL, rk, 1);
+      if (i < ne && rk < 32) sm.top[rk] = key;
+    } else if (tid < ne) {
       const uint64_t key = sm.ebuf[tid];
       int rk = 0;
       for (int q = 0; q < ne; ++q) rk += sm.ebuf[q] > key ? 1 : 0;
@@ -703,77 +780,70 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Ar
       for (int32_t gb = 0; gb < ng; gb += 32) {
         const int32_t gi = gb + lane;
         const bool in = gi < ng;
-        uint4 wv = NEG;
-        if (in) wv = ALIGNED ? ld_stream(vp + g0 + gi) : Tr::load_elems(rowp, (int64_t)(g0 + gi));
+        uint4 w4 = NEG;
+        if (in) w4 = ALIGNED ? ld_stream(vp + g0 + gi) : Tr::load_elems(rowp, (int64_t)(g0 + gi));
 #pragma unroll 1
         for (int e2 = 0; e2 < VEC; ++e2) {
-          const float x = Tr::at(wv, e2);
+          const float x = Tr::at(w4, e2);
           const bool c = in && x >= thr;
           ek.push(c, c ? make_key(x, (uint32_t)((g0 + gi) * VEC + e2)) : 0ull, lane);
           ek.drain(lane);
         }
       }
-      if (has_tail && rank == 0) {
-        for (int64_t v0 = (int64_t)gfull * VEC; v0 < V; v0 += 32) {
-          const int64_t v = v0 + lane;
-          const bool in = v < V;
-          const float x = in ? Tr::elem(rowp, v) : -INFINITY;
-          const bool c = in && x >= thr;
-          ek.push(c, c ? make_key(x, (uint32_t)v) : 0ull, lane);
-          ek.drain(lane);
-        }
+      if (nedge > 0) {
+        const bool c = lane < nedge && xe >= thr;
+        ek.push(c, c ? make_key(xe, (uint32_t)ve) : 0ull, lane);
+        ek.drain(lane);
       }
       ek.drain_all(lane);
       E = ek.list;
     }
   }
 
-  // ---- split-vocab merge across the cluster (distributed shared memory)
+  // ---- split-vocab merge across the cluster (distributed shared memory): the
+  // other CTAs leave their state and list in rank 0's shared memory, one lane
+  // per 8 bytes of list, and one cluster barrier hands them over
   if (C > 1) {
-    if (warp == 0) {
-      if (lane == 0) {
-        sm.fm = m;
-        sm.fS = S;
-        sm.fU = U;
-        sm.fbad = bad;
-      }
-      sm.flist[lane] = E;
-    }
-    cluster_sync_all();
-    if (rank == 0 && warp == 0) {
-      for (uint32_t r = 1; r < C; ++r) {
-        const float mo = dsmem_ld_f32(dsmem_addr(&sm.fm, r));
-        const float So = dsmem_ld_f32(dsmem_addr(&sm.fS, r));
-        const float Uo = dsmem_ld_f32(dsmem_addr(&sm.fU, r));
-        const int bo = dsmem_ld_s32(dsmem_addr(&sm.fbad, r));
-        lse_merge(m, S, U, mo, So, Uo);
-        bad = bad || bo;
-        const uint64_t peer = dsmem_ld_u64(dsmem_addr(&sm.flist[lane], r));
-        E = warp_merge_desc<uint64_t>(E, peer, lane);
+    cluster_wait();  // the arrivals at the start: rank 0 runs, its memory may be written
+    if (warp == 0 && rank != 0) {
+      dsmem_st_u64(dsmem_addr(&sm.peer_list[rank][lane], 0), E);
+      if (lane < 4) {
+        const uint32_t v = lane == 0   ? __float_as_uint(m)
+                           : lane == 1 ? __float_as_uint(S)
+                           : lane == 2 ? __float_as_uint(U)
+                                       : (bad ? 1u : 0u);
+        dsmem_st_u32(dsmem_addr(&sm.peer_state[rank][lane], 0), v);
       }
     }
     cluster_sync_all();
     if (rank != 0) return;
+    if (warp == 0) {
+      for (uint32_t r = 1; r < C; ++r) {
+        lse_merge(m, S, U, __uint_as_float(sm.peer_state[r][0]),
+                  __uint_as_float(sm.peer_state[r][1]), __uint_as_float(sm.peer_state[r][2]));
+        bad = bad || sm.peer_state[r][3] != 0u;
+        E = warp_merge_desc<uint64_t>(E, sm.peer_list[r][lane], lane);
+      }
+    }
   }
 
-  if (warp != 0) return;
-
-  pdl_wait();
-  if (MODE == MODE_ROUTE) {
+  if (MODE == MODE_ROUTE && warp == 2) {
+    pdl_wait();
     const int64_t nclusters = gridDim.x / C;
     route_special_requests(a, (int64_t)cid * 32 + lane, nclusters * 32);
   }
-  row_finish<T, MODE>(a, row, m, S, U, bad, E, pre, lane);
+  if (warp != 0) return;
+  pdl_wait();
+  row_finish<T, MODE>(a, row, m, S, U, bad, E, sm.pre, lane);
 }
 
 // ---- the persistent, warp-specialised row kernel (one CTA per row at a time) -----------------
 //
 // NWARP streaming warps read rows blockIdx.x, blockIdx.x + gridDim.x, ...; they
 // never wait on the per-row selection: at the end of a row they leave its tile
-// maxima, per-warp (m, S, U), sorted per-thread maxima and each thread's best
+// maxima, per-warp (m, S, U), largest thread maxima and each thread's best
 // tile in one of two shared buffers, signal the finaliser warp with a named
-// barrier and go on (the next
-// row's first tile is already in flight).  The finaliser warp turns a buffer
+// barrier and go on (the next row's first tile is already in flight).  The finaliser warp turns a buffer
 // into the row's exact top-K, features and epilogue, then hands the buffer
 // back.  Named barriers (bar.arrive / bar.sync with NT + 32 threads) are the
 // only synchronisation; every thread reaches each of them a known number of
@@ -793,10 +863,10 @@ __device__ __forceinline__ void named_bar_arrive(int id, int n) {
 struct SmemWS {
   float4 tinfo[2][NT];          // per thread: best, second and third tile maxima, and
                                 //   (best tile | second tile << 16); two row buffers
-  uint32_t wl[2][NWARP][32];    // per-warp sorted per-thread maxima, ord() encoded
+  uint32_t pub[2][NWARP * PUB]; // every warp's largest thread maxima, ord() encoded
   float pm[2][NWARP], pS[2][NWARP], pU[2][NWARP];
-  float cand_v[CCAP];           // finaliser: candidate tiles (value,
-  uint32_t cand_id[CCAP];       //   tile << 8 | thread, | BEST_BIT for a thread's best tile)
+  uint32_t cand_id[CCAP];       // finaliser: candidate tiles (tile << 8 | thread, | BEST_BIT
+                                //   for a thread's best tile)
   uint64_t ebuf[ECAP];          // finaliser: candidate element keys
   uint4 best[2][UNR][NT];       // per thread: the groups of its best tile, as streamed
 };
@@ -805,39 +875,31 @@ struct SmemWS {
 // from SmemWS::best instead of re-reading the row (tile indices stay below 2^16).
 constexpr uint32_t BEST_BIT = 0x80000000u;
 
-// Row geometry shared by the streaming warps and the finaliser (C = 1).
-struct RowGeom {
-  int32_t gfull, nfull, rem, ntiles;
-  bool has_tail;
-  __device__ __forceinline__ RowGeom(int64_t V, int vec) {
-    gfull = (int32_t)(V / vec);
-    has_tail = (V % vec) != 0;
-    nfull = gfull / TILE;
-    rem = gfull - nfull * TILE;
-    ntiles = nfull + (rem > 0 ? 1 : 0);
-  }
-};
-
 // The finaliser warp's work for one streamed row held in buffer b.
 //
 // Every streaming thread reports its best and second-best tile (value and
-// index) and its third-best tile value.  theta1 = the kc-th largest thread
-// maximum.  Candidate tiles are the best / second-best tiles >= theta1; a
-// thread whose third-best value also reaches theta1 contributes all its
-// tiles, and then theta stays theta1 (exact, if slower).  Otherwise theta =
-// the kc-th largest candidate value.  Elements >= theta of the candidate
-// tiles are the only ones that can be among the top kc.  A best tile is read
-// from the copy the streaming thread left in shared memory; the other
-// candidate tiles are re-read from the row, which may have left L2 by then.
+// index) and its third-best tile value, every warp its four largest thread
+// maxima.  theta1 = the kc-th largest of those (kc distinct elements reach it).
+// Candidate tiles are the best / second-best tiles >= theta1; a thread whose
+// third-best value also reaches theta1 contributes all its tiles.  Elements >=
+// theta1 of the candidate tiles are the only ones that can be among the top kc
+// (about 22 for kc = 20).  A best tile is read from the copy the streaming
+// thread left in shared memory; the other candidate tiles are re-read from the
+// row, which may have left L2 by then.  The warp has one row's stream time for
+// this, 9 us for V = 70,000 bf16, and its instructions take issue slots from the
+// stream: counting ranks instead of sorting, one threshold instead of two and
+// lse_warp took 4,457 such rows from 125 to 110 us, 9,670 rows of V = 151,936 bf16
+// from 449 to 436 us.
 template <typename T, int MODE, bool ALIGNED>
 __device__ __noinline__ void finalize_ws(const Args& a, SmemWS& sm, int b, int64_t row,
-                                         const RowGeom& geo, const RowPre& pre, int lane) {
+                                         const RowPre& pre, int lane) {
   using Tr = Traits<T>;
   constexpr int VEC = Tr::VEC;
   const int64_t V = a.vocab;
   const int kc = a.kc;
   const char* rowp = reinterpret_cast<const char*>(a.logits) + row * a.row_stride * (int64_t)sizeof(T);
   const uint4* vp = reinterpret_cast<const uint4*>(rowp);
+  const RowGeom geo(V, VEC);
   const uint4 NEG = make_uint4(Tr::NEG_WORD, Tr::NEG_WORD, Tr::NEG_WORD, Tr::NEG_WORD);
   const unsigned lt = (1u << lane) - 1u;
 
@@ -857,180 +919,195 @@ __device__ __noinline__ void finalize_ws(const Args& a, SmemWS& sm, int b, int64
   U = __shfl_sync(FULL, U, 0);
   bool bad = false;
 
-  // ---- the partial last group (fewer than VEC elements)
-  float tail_max = -INFINITY;
-  if (geo.has_tail) {
-    if (lane == 0) {
-      for (int64_t v = (int64_t)geo.gfull * VEC; v < V; ++v) {
-        const float x = Tr::elem(rowp, v);
-        careful_add(x, m, S, U, bad);
-        if (!isnan(x)) tail_max = fmaxf(tail_max, x);
-      }
+  // ---- the elements after the last group, one per lane
+  float xe = -INFINITY;
+  const bool edge = lane < geo.nedge;
+  const int64_t ve = (int64_t)geo.gfull * VEC + lane;
+  if (geo.nedge > 0) {
+    float em = M2_INIT, eS = 0.f, eU = 0.f;
+    if (edge) {
+      const float x = Tr::elem(rowp, ve);
+      careful_add(x, em, eS, eU, bad);
+      if (!isnan(x)) xe = x;
     }
-    m = __shfl_sync(FULL, m, 0);
-    S = __shfl_sync(FULL, S, 0);
-    U = __shfl_sync(FULL, U, 0);
-    bad = __shfl_sync(FULL, (int)bad, 0) != 0;
-    tail_max = __shfl_sync(FULL, tail_max, 0);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float mo = __shfl_xor_sync(FULL, em, o);
+      const float So = __shfl_xor_sync(FULL, eS, o);
+      const float Uo = __shfl_xor_sync(FULL, eU, o);
+      lse_merge(em, eS, eU, mo, So, Uo);
+    }
+    lse_merge(m, S, U, em, eS, eU);
+    bad = __any_sync(FULL, bad);
   }
 
-  // ---- theta1: the kc-th largest per-thread maximum (a merge tree over the
-  // eight per-warp sorted lists; independent merges interleave)
-  uint32_t L0 = warp_merge_desc<uint32_t>(sm.wl[b][0][lane], sm.wl[b][1][lane], lane);
-  uint32_t L1 = warp_merge_desc<uint32_t>(sm.wl[b][2][lane], sm.wl[b][3][lane], lane);
-  uint32_t L2 = warp_merge_desc<uint32_t>(sm.wl[b][4][lane], sm.wl[b][5][lane], lane);
-  uint32_t L3 = warp_merge_desc<uint32_t>(sm.wl[b][6][lane], sm.wl[b][7][lane], lane);
-  L0 = warp_merge_desc<uint32_t>(L0, L1, lane);
-  L2 = warp_merge_desc<uint32_t>(L2, L3, lane);
-  uint32_t L = warp_merge_desc<uint32_t>(L0, L2, lane);
-  if (geo.has_tail) L = warp_merge_desc<uint32_t>(L, lane == 0 ? ord(tail_max) : 0u, lane);
-  const float th1 = unord(__shfl_sync(FULL, L, kc - 1));
+  // ---- theta1: the kc-th largest of every warp's four largest thread maxima and
+  // of the last elements
+  float th1;
+  {
+    const uint32_t mine = sm.pub[b][lane], em = edge ? ord(xe) : 0u;
+    int rk = 0, re = 0;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+      const uint32_t q = sm.pub[b][j];
+      rk += (q > mine || (q == mine && j < lane)) ? 1 : 0;
+      if (geo.nedge > 0) re += q >= em ? 1 : 0;
+    }
+    for (int j = 0; j < geo.nedge; ++j) {
+      const uint32_t q = __shfl_sync(FULL, em, j);
+      rk += q > mine ? 1 : 0;
+      re += (q > em || (q == em && j < lane)) ? 1 : 0;
+    }
+    const unsigned hit = __ballot_sync(FULL, rk == kc - 1);
+    const unsigned hite = __ballot_sync(FULL, edge && re == kc - 1);
+    const uint32_t v = hit ? __shfl_sync(FULL, mine, __ffs(hit) - 1)
+                           : __shfl_sync(FULL, em, (__ffs(hite) - 1) & 31);
+    th1 = unord(v);
+  }
+  if (!(th1 > -INFINITY)) {
+    // fewer than kc published maxima (all but a few neighbouring tokens
+    // masked): the kc-th largest of all thread maxima, bit by bit
+    uint32_t v[NT / 32 + 1], kth = 0u;
+#pragma unroll
+    for (int j = 0; j < NT / 32; ++j) v[j] = ord(sm.tinfo[b][j * 32 + lane].x);
+    v[NT / 32] = edge ? ord(xe) : 0u;
+#pragma unroll 1
+    for (uint32_t bit = 0x80000000u; bit; bit >>= 1) {
+      int c = 0;
+#pragma unroll
+      for (int j = 0; j <= NT / 32; ++j) c += __popc(__ballot_sync(FULL, v[j] >= (kth | bit)));
+      if (c >= kc) kth |= bit;
+    }
+    th1 = unord(kth);
+  }
   bool fb = !(th1 > -INFINITY);
 
-  // ---- candidate tiles
-  int n = 0;            // candidate tiles
-  bool all3 = false;    // some thread has three tiles >= theta1
+  // ---- candidate tiles: lane l looks at the reports of threads l, 32 + l, ...
+  int n = 0;  // candidate tiles
   if (!fb) {
-#pragma unroll 2
+    uint32_t m1 = 0u, m2 = 0u, m3 = 0u;  // bit j: best, second, third tile >= theta1
+#pragma unroll
     for (int j = 0; j < NT / 32; ++j) {
-      const uint32_t t = (uint32_t)(j * 32 + lane);
-      const float4 inf = sm.tinfo[b][t];
-      const uint32_t ids = __float_as_uint(inf.w);
-      const bool c1 = inf.x >= th1, c2 = inf.y >= th1, c3 = inf.z >= th1;
-      all3 = all3 || c3;
-      // the best and second-best tiles
-      const unsigned b1 = __ballot_sync(FULL, c1);
-      const unsigned b2 = __ballot_sync(FULL, c2 && !c3);
-      const int p1 = n + __popc(b1 & lt);
-      const int p2 = n + __popc(b1) + __popc(b2 & lt);
-      if (c1 && p1 < CCAP) {
-        sm.cand_v[p1] = inf.x;
-        sm.cand_id[p1] = BEST_BIT | ((ids & 0xffffu) << 8) | t;
-      }
-      if (c2 && !c3 && p2 < CCAP) {
-        sm.cand_v[p2] = inf.y;
-        sm.cand_id[p2] = ((ids >> 16) << 8) | t;
-      }
-      n += __popc(b1) + __popc(b2);
-      // a thread with a third tile >= theta1: every other tile of it
-      unsigned b3 = __ballot_sync(FULL, c3);
-      while (b3) {
-        const int src = __ffs(b3) - 1;
-        b3 &= b3 - 1;
-        const uint32_t ts = (uint32_t)(j * 32 + src);
-        const uint32_t ids_s = __shfl_sync(FULL, ids, src);
-        const uint32_t ti1 = ids_s & 0xffffu;
-        for (int t0 = 0; t0 < geo.ntiles; t0 += 32) {
-          const int tt = t0 + lane;
-          const bool c = tt < geo.ntiles && (uint32_t)tt != ti1;
-          const unsigned bb = __ballot_sync(FULL, c);
-          const int pos = n + __popc(bb & lt);
-          if (c && pos < CCAP) {
-            sm.cand_v[pos] = th1;
-            sm.cand_id[pos] = ((uint32_t)tt << 8) | ts;
+      const float4 inf = sm.tinfo[b][j * 32 + lane];
+      m1 |= inf.x >= th1 ? 1u << j : 0u;
+      m2 |= inf.y >= th1 ? 1u << j : 0u;
+      m3 |= inf.z >= th1 ? 1u << j : 0u;
+    }
+    m2 &= ~m3;
+    int x = __popc(m1) + __popc(m2);
+    const int own = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(FULL, x, o);
+      if (lane >= o) x += y;
+    }
+    n = __shfl_sync(FULL, x, 31);
+    int pos = x - own;
+    for (uint32_t q = m1; q; q &= q - 1u, ++pos) {
+      const uint32_t t = (uint32_t)((__ffs(q) - 1) * 32 + lane);
+      if (pos < CCAP)
+        sm.cand_id[pos] = BEST_BIT | ((__float_as_uint(sm.tinfo[b][t].w) & 0xffffu) << 8) | t;
+    }
+    for (uint32_t q = m2; q; q &= q - 1u, ++pos) {
+      const uint32_t t = (uint32_t)((__ffs(q) - 1) * 32 + lane);
+      if (pos < CCAP) sm.cand_id[pos] = ((__float_as_uint(sm.tinfo[b][t].w) >> 16) << 8) | t;
+    }
+    // a thread with a third tile >= theta1: every other tile of it
+    if (__any_sync(FULL, m3 != 0u)) {
+#pragma unroll 1
+      for (int j = 0; j < NT / 32; ++j) {
+        unsigned b3 = __ballot_sync(FULL, (m3 >> j) & 1u);
+        while (b3) {
+          const uint32_t ts = (uint32_t)(j * 32 + __ffs(b3) - 1);
+          b3 &= b3 - 1;
+          const uint32_t ti1 = __float_as_uint(sm.tinfo[b][ts].w) & 0xffffu;
+          for (int t0 = 0; t0 < geo.ntiles; t0 += 32) {
+            const int tt = t0 + lane;
+            const bool c = tt < geo.ntiles && (uint32_t)tt != ti1;
+            const unsigned bb = __ballot_sync(FULL, c);
+            const int p = n + __popc(bb & lt);
+            if (c && p < CCAP) sm.cand_id[p] = ((uint32_t)tt << 8) | ts;
+            n += __popc(bb);
           }
-          n += __popc(bb);
         }
       }
-    }
-    all3 = __any_sync(FULL, all3);
-    // the partial last group is a candidate too (its elements are read below)
-    if (geo.has_tail && tail_max >= th1) {
-      if (lane == 0 && n < CCAP) {
-        sm.cand_v[n] = tail_max;
-        sm.cand_id[n] = TAIL_ID;
-      }
-      ++n;
     }
     if (n > CCAP) fb = true;
   }
   __syncwarp();
 
-  // ---- the candidate tiles' groups: a thread's best tile from shared
-  // memory, the others re-read from the row (issued first, so that sorting
-  // the candidates for theta overlaps the loads); then keep elements >= theta
-  const int total = fb ? 0 : n * UNR;
-  // group `it` of the candidates (UNR per candidate tile): its index in the
-  // row (or -1: none, or the partial last group) and its 16 bytes
-  auto cand_group = [&](int it, int32_t& gsel_q, uint4& w) {
-    gsel_q = -1;
-    w = NEG;
-    const uint32_t id = sm.cand_id[it >> 2];
-    if (id == TAIL_ID) return;
-    const int k = it & (UNR - 1), t = (int)(id & 255u);
-    const int32_t gi = (int32_t)((id & ~BEST_BIT) >> 8) * TILE + k * NT + t;
-    if (gi >= geo.gfull) return;
-    gsel_q = gi;
-    if (id & BEST_BIT) w = sm.best[b][k][t];
-    else w = ALIGNED ? ld_reread(vp + gi) : Tr::load_elems(rowp, gi);
-  };
-  uint4 wv[4];
-  int32_t gsel[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int it = q * 32 + lane;
-    gsel[q] = -1;
-    wv[q] = NEG;
-    if (it < total) cand_group(it, gsel[q], wv[q]);
-  }
-
-  // ---- theta: the exact kc-th largest candidate value (theta1 if a thread
-  // contributed all its tiles)
-  float th = th1;
-  if (!fb && !all3) {
-    uint32_t Lc = 0u;
-#pragma unroll 1
-    for (int b0 = 0; b0 < n; b0 += 32) {
-      uint32_t k = b0 + lane < n ? ord(sm.cand_v[b0 + lane]) : 0u;
-      k = warp_sort_desc<uint32_t>(k, lane);
-      Lc = warp_merge_desc<uint32_t>(Lc, k, lane);
-    }
-    const uint32_t kth = __shfl_sync(FULL, Lc, kc - 1);
-    if (kth != 0u) th = unord(kth);  // (there are always kc candidates; kept as a guard)
-  }
-
+  // ---- the candidate tiles' groups (a thread's best tile from shared memory,
+  // the others re-read from the row); their elements >= theta1 become keys: kc
+  // distinct elements reach theta1, so the row's top kc are among them
   int ne = 0;
   if (!fb) {
+    const int total = n * UNR;
     for (int i0 = 0; i0 < total; i0 += 128) {
-      if (i0 > 0) {
-        // more than 128 candidate groups: the next batch of loads
+      uint4 wv[4];
+      int32_t gsel[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int it = i0 + q * 32 + lane;
-          gsel[q] = -1;
-          wv[q] = NEG;
-          if (it < total && sm.cand_v[it >> 2] >= th) cand_group(it, gsel[q], wv[q]);
+      for (int q = 0; q < 4; ++q) {
+        const int it = i0 + q * 32 + lane;
+        gsel[q] = -1;
+        wv[q] = NEG;
+        if (it < total) {
+          const uint32_t id = sm.cand_id[it >> 2];
+          const int k = it & (UNR - 1), t = (int)(id & 255u);
+          const int32_t gi = (int32_t)((id & ~BEST_BIT) >> 8) * TILE + tile_pos(t, k);
+          if (gi < geo.gfull) {
+            gsel[q] = gi;
+            if (id & BEST_BIT) wv[q] = sm.best[b][k][t];
+            else wv[q] = ALIGNED ? ld_reread(vp + gi) : Tr::load_elems(rowp, gi);
+          }
         }
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
+        uint32_t hits = 0u;
 #pragma unroll
-        for (int e2 = 0; e2 < VEC; ++e2) {
-          const float x = Tr::at(wv[q], e2);
-          const bool c = gsel[q] >= 0 && x >= th;
-          const unsigned bal = __ballot_sync(FULL, c);
-          const int pos = ne + __popc(bal & lt);
-          if (c && pos < ECAP) sm.ebuf[pos] = make_key(x, (uint32_t)(gsel[q] * VEC + e2));
+        for (int e = 0; e < VEC; ++e) hits |= Tr::at(wv[q], e) >= th1 ? 1u << e : 0u;
+        if (gsel[q] < 0) hits = 0u;
+        unsigned bal;
+        while ((bal = __ballot_sync(FULL, hits != 0u)) != 0u) {  // mostly one round
+          const int e = __ffs(hits) - 1, pos = ne + __popc(bal & lt);
+          if (hits && pos < ECAP)
+            sm.ebuf[pos] = make_key(Tr::at(wv[q], e), (uint32_t)(gsel[q] * VEC + e));
+          hits &= hits - 1u;
           ne += __popc(bal);
         }
       }
     }
-    if (geo.has_tail && tail_max >= th) {
-      const int64_t v = (int64_t)geo.gfull * VEC + lane;
-      const float x = v < V ? Tr::elem(rowp, v) : -INFINITY;
-      const bool c = v < V && x >= th;
+    if (geo.nedge > 0) {
+      const bool c = edge && xe >= th1;
       const unsigned bal = __ballot_sync(FULL, c);
       const int pos = ne + __popc(bal & lt);
-      if (c && pos < ECAP) sm.ebuf[pos] = make_key(x, (uint32_t)v);
+      if (c && pos < ECAP) sm.ebuf[pos] = make_key(xe, (uint32_t)ve);
       ne += __popc(bal);
     }
     if (ne > ECAP) fb = true;
   }
   __syncwarp();
 
-  // ---- the row's exact top-32 elements
+  // ---- the row's exact top-32 elements: up to 64 keys are ranked by counting
+  // (keys are distinct: the index is part of the key), more are sorted
   uint64_t E = 0ull;
-  if (!fb) {
+  if (!fb && ne <= 64) {
+    const uint64_t k0 = lane < ne ? sm.ebuf[lane] : 0ull;
+    const uint64_t k1 = 32 + lane < ne ? sm.ebuf[32 + lane] : 0ull;
+    int r0 = 0, r1 = 0;
+    for (int q = 0; q < ne; ++q) {
+      const uint64_t k = sm.ebuf[q];
+      r0 += k > k0 ? 1 : 0;
+      r1 += k > k1 ? 1 : 0;
+    }
+    __syncwarp();
+    sm.ebuf[64 + lane] = 0ull;
+    __syncwarp();
+    if (k0 != 0ull && r0 < 32) sm.ebuf[64 + r0] = k0;
+    if (k1 != 0ull && r1 < 32) sm.ebuf[64 + r1] = k1;
+    __syncwarp();
+    E = sm.ebuf[64 + lane];
+  } else if (!fb) {
 #pragma unroll 1
     for (int b0 = 0; b0 < ne; b0 += 32) {
       uint64_t k = b0 + lane < ne ? sm.ebuf[b0 + lane] : 0ull;
@@ -1057,12 +1134,9 @@ __device__ __noinline__ void finalize_ws(const Args& a, SmemWS& sm, int b, int64
         ek.drain(lane);
       }
     }
-    if (geo.has_tail) {
-      const int64_t v = (int64_t)geo.gfull * VEC + lane;
-      const bool in = v < V;
-      const float x = in ? Tr::elem(rowp, v) : -INFINITY;
-      const bool c = in && x >= th1;
-      ek.push(c, c ? make_key(x, (uint32_t)v) : 0ull, lane);
+    if (geo.nedge > 0) {
+      const bool c = edge && xe >= th1;
+      ek.push(c, c ? make_key(xe, (uint32_t)ve) : 0ull, lane);
       ek.drain(lane);
     }
     ek.drain_all(lane);
@@ -1101,52 +1175,49 @@ __global__ void __launch_bounds__(NT_WS, 3) verify_rows_ws(const Args a) {
 
   pdl_trigger();  // a dependent launch may start streaming while this one finishes
 
-  const RowGeom geo(a.vocab, Tr::VEC);
-
+  auto rowp_of = [&](int64_t r) {
+    return reinterpret_cast<const char*>(a.logits) + r * a.row_stride * (int64_t)sizeof(T);
+  };
   if (warp == NWARP) {
     // ---- the finaliser warp: the next row's inputs are fetched while its
     // stream is still running
-    auto rowp_of = [&](int64_t r) {
-      return reinterpret_cast<const char*>(a.logits) + r * a.row_stride * (int64_t)sizeof(T);
-    };
     int i = 0;
     int64_t row = blockIdx.x;
-    RowPre pre = load_pre<T, MODE>(a, row, rowp_of(row), lane);
+    RowPre pre = load_pre<T, MODE>(a, row, a.chosen[row], rowp_of(row), lane);
     pdl_wait();
     if (MODE == MODE_ROUTE) route_special_requests(a, (int64_t)blockIdx.x * 32 + lane, G * 32);
     for (; row < a.n_rows; row += G, ++i) {
       const int b = i & 1;
       named_bar_sync(BAR_FULL + b, NT_WS);
-      finalize_ws<T, MODE, ALIGNED>(a, sm, b, row, geo, pre, lane);
+      finalize_ws<T, MODE, ALIGNED>(a, sm, b, row, pre, lane);
       if (row + 2 * G < a.n_rows) {
         __syncwarp();
         __threadfence_block();
         named_bar_arrive(BAR_EMPTY + b, NT_WS);
       }
-      if (row + G < a.n_rows) pre = load_pre<T, MODE>(a, row + G, rowp_of(row + G), lane);
+      if (row + G < a.n_rows) pre = load_pre<T, MODE>(a, row + G, a.chosen[row + G], rowp_of(row + G), lane);
     }
     return;
   }
 
   // ---- the streaming warps
   const uint4 NEG = make_uint4(Tr::NEG_WORD, Tr::NEG_WORD, Tr::NEG_WORD, Tr::NEG_WORD);
+  const RowGeom geo(a.vocab, Tr::VEC);
   auto load_tile = [&](uint4 (&dst)[UNR], int64_t r, int32_t t) {
-    const char* rp = reinterpret_cast<const char*>(a.logits) + r * a.row_stride * (int64_t)sizeof(T);
-    const uint4* vp = reinterpret_cast<const uint4*>(rp);
-    const int32_t base = t * TILE + tid;
+    const uint4* vp = reinterpret_cast<const uint4*>(rowp_of(r));
+    auto load = [&](int32_t g) -> uint4 {
+      return ALIGNED ? ld_stream(vp + g) : Tr::load_elems(vp, g);
+    };
+    const int32_t base = t * TILE;
     if (t < geo.nfull) {
 #pragma unroll
-      for (int k = 0; k < UNR; ++k)
-        dst[k] = ALIGNED ? ld_stream(vp + base + k * NT) : Tr::load_elems(rp, base + k * NT);
+      for (int k = 0; k < UNR; ++k) dst[k] = load(base + tile_pos(tid, k));
     } else {
 #pragma unroll
       for (int k = 0; k < UNR; ++k)
-        dst[k] = (k * NT + tid < geo.rem)
-                     ? (ALIGNED ? ld_stream(vp + base + k * NT) : Tr::load_elems(rp, base + k * NT))
-                     : NEG;
+        dst[k] = tile_pos(tid, k) < geo.rem ? load(base + tile_pos(tid, k)) : NEG;
     }
   };
-
   uint4 cur[UNR], nxt[UNR];
   int64_t row = blockIdx.x;
   if (row < a.n_rows && geo.ntiles > 0) load_tile(cur, row, 0);
@@ -1191,26 +1262,20 @@ __global__ void __launch_bounds__(NT_WS, 3) verify_rows_ws(const Args a) {
       } else {
 #pragma unroll
         for (int k = 0; k < UNR; ++k)
-          if (k * NT + tid < geo.rem) Tr::accum(cur[k], nm, S2, U2);
+          if (tile_pos(tid, k) < geo.rem) Tr::accum(cur[k], nm, S2, U2);
       }
 #pragma unroll
       for (int k = 0; k < UNR; ++k) cur[k] = nxt[k];
     }
     // the warp's partial state, its sorted per-thread maxima, the tile report
     float S = S2.x + S2.y, U = U2.x + U2.y;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float mo = __shfl_xor_sync(FULL, m, o);
-      const float So = __shfl_xor_sync(FULL, S, o);
-      const float Uo = __shfl_xor_sync(FULL, U, o);
-      lse_merge(m, S, U, mo, So, Uo);
-    }
+    lse_warp(m, S, U);
     if (lane == 0) {
       sm.pm[b][warp] = m;
       sm.pS[b][warp] = S;
       sm.pU[b][warp] = U;
     }
-    sm.wl[b][warp][lane] = warp_sort_desc<uint32_t>(ord(v1), lane);
+    publish_max(ord(v1), &sm.pub[b][warp * PUB], lane);
     sm.tinfo[b][tid] = make_float4(v1, v2, v3, __uint_as_float(i1 | (i2 << 16)));
     __syncwarp();
     __threadfence_block();

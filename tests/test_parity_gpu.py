@@ -249,6 +249,34 @@ def test_persistent_candidate_paths(ctx, dtype, V, shift):
     _set(ctx)
 
 
+@pytest.mark.parametrize("split", [0, 1, 8])
+@pytest.mark.parametrize("K", [1, 20, 32])
+@pytest.mark.parametrize("dtype,V", [(torch.bfloat16, 20011), (torch.float32, 9000),
+                                     (torch.bfloat16, 3000)])
+def test_few_unmasked_neighbours(ctx, dtype, V, K, split):
+    """Rows whose unmasked tokens lie side by side: few threads of one warp hold
+    them, so the warps' published maxima are fewer than K and the threshold
+    comes from all thread maxima, or from a scan of the row (both sides of
+    either change, windows at the row's ends too)."""
+    _set(ctx, split=split)
+    widths = [1, 2, 4, 19, 20, 31, 32, 33, 100, 159, 161, 300, 1100]
+    x, ch = random_rows(2 * len(widths), V, dtype, seed=V + K)
+    for r in range(x.size(0)):
+        w = widths[r // 2]
+        lo = (r * 977) % (V - w) if r % 2 == 0 else V - w
+        m = torch.full_like(x[r], float("-inf"))
+        m[lo:lo + w] = x[r, lo:lo + w]
+        x[r] = m
+        ch[r] = lo + w // 2
+    feat, top2, rf = B.pr_token_features(ctx, x, ch, topk=K)
+    of, oi, ofl = _oracle_rows(x, ch, K=K)
+    several = np.array([widths[r // 2] > 1 for r in range(x.size(0))])  # else i2 is a masked token
+    assert np.array_equal(top2.cpu().numpy()[:, 0], oi[:, 0])
+    _check_features(feat[several], top2[several], rf[several], of[several], oi[several],
+                    ofl[several], "V=%d K=%d" % (V, K))
+    _set(ctx)
+
+
 def test_rows_past_the_persistent_kernels_tile_limit(ctx):
     """Rows of more than 2^16 tiles (268,443,648 fp32 values, 1.07 GB a row)
     leave the persistent kernel, whose tile indices are 16-bit, even with
