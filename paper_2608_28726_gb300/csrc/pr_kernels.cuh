@@ -440,15 +440,27 @@ __device__ __forceinline__ void row_finish(const Args& a, int64_t row, float m, 
   }
 }
 
-// the warp's PUB largest values, into out[0 .. PUB - 1] (lane 0)
-__device__ __forceinline__ void publish_max(uint32_t cur, uint32_t* out, int lane) {
+// 32 of a CTA's largest thread maxima into pub[0 .. 31], from which theta1 comes:
+// every warp's PUB largest ones; of a range of less than a tile, whose first
+// warps hold all of it, the 32 / A largest ones of A warps, A the largest power
+// of two up to the number of warps with a group in every lane.
+__device__ __forceinline__ void publish_max(uint32_t cur, uint32_t* pub, int32_t groups, int warp,
+                                            int lane) {
+  if (groups >= TILE) {
 #pragma unroll
-  for (int i = 0; i < PUB; ++i) {
-    const uint32_t w = __reduce_max_sync(FULL, cur);
-    const unsigned eq = __ballot_sync(FULL, cur == w);
-    if (lane == 0) out[i] = w;
-    if (lane == __ffs(eq) - 1) cur = 0u;
+    for (int i = 0; i < PUB; ++i) {
+      const uint32_t w = __reduce_max_sync(FULL, cur);
+      const unsigned eq = __ballot_sync(FULL, cur == w);
+      if (lane == 0) pub[warp * PUB + i] = w;
+      if (lane == __ffs(eq) - 1) cur = 0u;
+    }
+    return;
   }
+  const int full = max(1, (groups + 32 * (UNR - 1)) / (32 * UNR));  // warps with 32 groups or more
+  const int A = full >= 8 ? 8 : full >= 4 ? 4 : full >= 2 ? 2 : 1, n = 32 / A;
+  if (warp >= A) return;
+  cur = warp_sort_desc<uint32_t>(cur, lane);
+  if (lane < n) pub[warp * n + lane] = cur;
 }
 
 // ---- the row kernel for split rows: one thread-block cluster of C CTAs per row ----------------
@@ -594,13 +606,13 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Ar
     thr_max = fmaxf(thr_max, xe);
   }
 
-  // ---- theta1: the kc-th largest of every warp's four largest thread maxima
+  // ---- theta1: the kc-th largest of the published thread maxima
   // (kc <= 32 distinct elements reach it, so it bounds the kc-th element from
   // below).  Against the kc-th largest of all thread maxima, which takes a sort
   // per warp and seven merges, about one candidate more passes it (22 for 21 of
   // 151,936 normal values and kc = 20).
   const int kc = a.kc;
-  publish_max(ord(thr_max), &sm.pub[warp * PUB], lane);
+  publish_max(ord(thr_max), sm.pub, ng, warp, lane);
   int32_t y = 0;
   if (rank == 0 && warp == 1) y = a.chosen[row];  // used after the next barrier
   __syncthreads();
@@ -615,9 +627,10 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Ar
     }
     th1 = unord(__shfl_sync(FULL, mine, __ffs(__ballot_sync(FULL, rk == kc - 1)) - 1));
   }
-  if (!(th1 > -INFINITY)) {
-    // fewer than kc published maxima (a range of less than a tile, or all but a
-    // few neighbouring tokens masked): the kc-th largest of all thread maxima
+  if (!(th1 > -INFINITY) && ng > 32 * UNR) {
+    // fewer than kc published maxima (all but a few neighbouring tokens masked;
+    // one warp's share has published all it has): the kc-th largest of all
+    // thread maxima
     sm.all_max[tid] = ord(thr_max);
     if (tid == 0) sm.theta1 = -INFINITY;
     __syncthreads();
@@ -878,8 +891,8 @@ constexpr uint32_t BEST_BIT = 0x80000000u;
 // The finaliser warp's work for one streamed row held in buffer b.
 //
 // Every streaming thread reports its best and second-best tile (value and
-// index) and its third-best tile value, every warp its four largest thread
-// maxima.  theta1 = the kc-th largest of those (kc distinct elements reach it).
+// index) and its third-best tile value, the warps their largest thread
+// maxima (publish_max).  theta1 = the kc-th largest of those (kc distinct elements reach it).
 // Candidate tiles are the best / second-best tiles >= theta1; a thread whose
 // third-best value also reaches theta1 contributes all its tiles.  Elements >=
 // theta1 of the candidate tiles are the only ones that can be among the top kc
@@ -941,8 +954,8 @@ __device__ __noinline__ void finalize_ws(const Args& a, SmemWS& sm, int b, int64
     bad = __any_sync(FULL, bad);
   }
 
-  // ---- theta1: the kc-th largest of every warp's four largest thread maxima and
-  // of the last elements
+  // ---- theta1: the kc-th largest of the published thread maxima and of the last
+  // elements
   float th1;
   {
     const uint32_t mine = sm.pub[b][lane], em = edge ? ord(xe) : 0u;
@@ -1275,7 +1288,7 @@ __global__ void __launch_bounds__(NT_WS, 3) verify_rows_ws(const Args a) {
       sm.pS[b][warp] = S;
       sm.pU[b][warp] = U;
     }
-    publish_max(ord(v1), &sm.pub[b][warp * PUB], lane);
+    publish_max(ord(v1), sm.pub[b], geo.gfull, warp, lane);
     sm.tinfo[b][tid] = make_float4(v1, v2, v3, __uint_as_float(i1 | (i2 << 16)));
     __syncwarp();
     __threadfence_block();
