@@ -33,6 +33,7 @@
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 namespace prk {
@@ -60,6 +61,7 @@ constexpr uint32_t FLAG_BAD_CHOSEN = 2u;
 constexpr uint32_t FLAG_EMPTY_REQ = 4u;
 constexpr uint32_t FLAG_BAD_OFFSETS = 8u;
 constexpr uint32_t FLAG_BAD_SLOT = 16u;
+constexpr uint32_t FLAG_TIMEOUT = 32u;
 
 enum Mode { MODE_FEATURES = 0, MODE_ROUTE = 1, MODE_DECODE = 2 };
 

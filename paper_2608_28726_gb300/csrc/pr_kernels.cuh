@@ -245,6 +245,122 @@ __device__ __forceinline__ int32_t tile_pos(int tid, int k) {
   return (tid >> 5) * (32 * UNR) + 32 * k + (tid & 31);
 }
 
+// Rows that start off the 16-byte grid (rows of an odd vocabulary stored side
+// by side): a group starts s bytes (a multiple of the element size) into a
+// 16-byte word of the grid and is read with the widest aligned loads that cover
+// it, two or three; a bf16 group that starts inside a 4-byte word takes five such
+// words (the fifth in x) and cut_groups shifts them into place.  Loads that
+// share a sector meet in L1.  The groups, and with them every sum, are those of
+// an aligned row.  (The split kernel's way; the persistent kernel has a ring, see
+// RingWS.)  350 rows of V = 70,001 bf16: 20.3 us per launch in a CUDA graph, 27.3
+// with every group loaded by its elements.
+__device__ __forceinline__ uint32_t ld_l1_32(const char* p) {
+  uint32_t r;
+  asm volatile("ld.global.nc.L2::256B.u32 %0, [%1];" : "=r"(r) : "l"(p));
+  return r;
+}
+__device__ __forceinline__ void ld_l1_64(const char* p, uint32_t& x, uint32_t& y) {
+  asm volatile("ld.global.nc.L2::256B.v2.u32 {%0,%1}, [%2];" : "=r"(x), "=r"(y) : "l"(p));
+}
+__device__ __forceinline__ void ld_l1_128(const char* p, uint32_t& x, uint32_t& y, uint32_t& z,
+                                          uint32_t& w) {
+  asm volatile("ld.global.nc.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(x), "=r"(y), "=r"(z), "=r"(w)
+               : "l"(p));
+}
+// the group S bytes into the grid word at p
+template <int S>
+__device__ __forceinline__ void ld_group(const char* p, uint4& w, uint32_t& x) {
+  uint32_t unused;
+  if (S == 0) {
+    ld_l1_128(p, w.x, w.y, w.z, w.w);
+  } else if (S == 2) {
+    ld_l1_128(p, w.x, w.y, w.z, w.w);
+    x = ld_l1_32(p + 16);
+  } else if (S == 4) {
+    w.x = ld_l1_32(p + 4);
+    ld_l1_64(p + 8, w.y, w.z);
+    w.w = ld_l1_32(p + 16);
+  } else if (S == 6) {
+    w.x = ld_l1_32(p + 4);
+    ld_l1_64(p + 8, w.y, w.z);
+    ld_l1_64(p + 16, w.w, x);
+  } else if (S == 8) {
+    ld_l1_64(p + 8, w.x, w.y);
+    ld_l1_64(p + 16, w.z, w.w);
+  } else if (S == 10) {
+    ld_l1_64(p + 8, w.x, w.y);
+    ld_l1_128(p + 16, w.z, w.w, x, unused);
+  } else if (S == 12) {
+    w.x = ld_l1_32(p + 12);
+    ld_l1_64(p + 16, w.y, w.z);
+    w.w = ld_l1_32(p + 24);
+  } else {
+    w.x = ld_l1_32(p + 12);
+    ld_l1_128(p + 16, w.y, w.z, w.w, x);
+  }
+}
+// groups n0 + tile_pos(tid, k) < n of the row whose group 0 starts s bytes into
+// the grid word at p
+template <int S>
+__device__ __forceinline__ void ld_groups(const char* p, int32_t n0, int32_t n, int tid,
+                                          uint4 (&w)[UNR], uint32_t (&x)[UNR], const uint4& none) {
+  const char* q = p + 16 * (int64_t)(n0 + tile_pos(tid, 0));
+  if (n0 + TILE <= n) {
+#pragma unroll
+    for (int k = 0; k < UNR; ++k) ld_group<S>(q + 512 * k, w[k], x[k]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < UNR; ++k) {
+      w[k] = none;
+      x[k] = none.x;
+      if (n0 + tile_pos(tid, k) < n) ld_group<S>(q + 512 * k, w[k], x[k]);
+    }
+  }
+}
+template <typename T>
+__device__ __forceinline__ void ld_tile_off_grid(const T* rowt, int32_t n0, int32_t n, bool rim,
+                                                 int tid, uint4 (&w)[UNR], uint32_t (&x)[UNR],
+                                                 const uint4& none) {
+  const int s = (int)(reinterpret_cast<uintptr_t>(rowt) & 15u);
+  const char* p = reinterpret_cast<const char*>(rowt) - s;
+  if (rim) {  // the first or last tile of the call's buffer: no byte outside it
+#pragma unroll
+    for (int k = 0; k < UNR; ++k) {
+      const int32_t g = n0 + tile_pos(tid, k);
+      w[k] = g < n ? Traits<T>::load_elems(rowt, g) : none;
+      x[k] = none.x;
+      if (s & 2) {  // as cut_group expects it
+        x[k] = w[k].w >> 16;
+        w[k] = make_uint4(w[k].x << 16, __funnelshift_l(w[k].x, w[k].y, 16),
+                          __funnelshift_l(w[k].y, w[k].z, 16), __funnelshift_l(w[k].z, w[k].w, 16));
+      }
+    }
+    return;
+  }
+  if (sizeof(T) == 4 || (s & 2) == 0) {
+    if (s == 0) ld_groups<0>(p, n0, n, tid, w, x, none);
+    else if (s == 4) ld_groups<4>(p, n0, n, tid, w, x, none);
+    else if (s == 8) ld_groups<8>(p, n0, n, tid, w, x, none);
+    else ld_groups<12>(p, n0, n, tid, w, x, none);
+  } else {
+    if (s == 2) ld_groups<2>(p, n0, n, tid, w, x, none);
+    else if (s == 6) ld_groups<6>(p, n0, n, tid, w, x, none);
+    else if (s == 10) ld_groups<10>(p, n0, n, tid, w, x, none);
+    else ld_groups<14>(p, n0, n, tid, w, x, none);
+  }
+}
+template <typename T>
+__device__ __forceinline__ void cut_groups(const T* rowt, uint4 (&w)[UNR], const uint32_t (&x)[UNR]) {
+  if constexpr (sizeof(T) == 2) {
+    if ((reinterpret_cast<uintptr_t>(rowt) & 2u) == 0) return;
+#pragma unroll
+    for (int k = 0; k < UNR; ++k)
+      w[k] = make_uint4(__funnelshift_r(w[k].x, w[k].y, 16), __funnelshift_r(w[k].y, w[k].z, 16),
+                        __funnelshift_r(w[k].z, w[k].w, 16), __funnelshift_r(w[k].w, x[k], 16));
+  }
+}
+
 // ---- one row's features and the mode's epilogue (one warp) ------------------------------
 
 // Whole warp (the request search is warp-collective).
@@ -470,13 +586,14 @@ __device__ __forceinline__ void publish_max(uint32_t cur, uint32_t* pub, int32_t
 // row: 354-row batches of V = 32,000 fp32 10.0 us per batch with five
 // against 11.5 us with four (two consecutive launches then fit on the GPU
 // together), 256-row decode steps of V = 151,936 bf16 11.1 against 10.7 us.
-template <typename T>
+// Off the 16-byte grid, where a group's loads need more registers, four.
+template <typename T, bool ALIGNED>
 constexpr int rows_min_blocks() {
-  return sizeof(T) == 4 ? 5 : 4;
+  return sizeof(T) == 4 && ALIGNED ? 5 : 4;
 }
 
 template <typename T, int MODE, bool ALIGNED>
-__global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Args a) {
+__global__ void __launch_bounds__(NT, rows_min_blocks<T, ALIGNED>()) verify_rows(const Args a) {
   __shared__ Smem sm;
   using Tr = Traits<T>;
   constexpr int VEC = Tr::VEC;
@@ -492,6 +609,7 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Ar
 
   const char* rowp = reinterpret_cast<const char*>(a.logits) + row * a.row_stride * (int64_t)sizeof(T);
   const int64_t V = a.vocab;
+  const T* rowt = reinterpret_cast<const T*>(rowp);
   const uint4* vp = reinterpret_cast<const uint4*>(rowp);
   const RowGeom geo(V, VEC);
   const int32_t g0 = (int32_t)((int64_t)geo.gfull * rank / C);
@@ -527,18 +645,28 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Ar
 
   // ---- stream the groups [g0, g1): tile t holds groups t*TILE + k*NT + tid ------------
   {
-    auto load = [&](int32_t gi) -> uint4 {
-      return ALIGNED ? ld_stream(vp + g0 + gi) : Tr::load_elems(rowp, (int64_t)(g0 + gi));
-    };
-    auto load_tile = [&](uint4 (&dst)[UNR], int32_t t) {  // nothing past the range
+    // the groups of tile t (off the grid: uncut), nothing past the range
+    auto load_tile = [&](uint4 (&dst)[UNR], uint32_t (&ext)[UNR], int32_t t) {
       const int32_t nb = t * TILE;
-      if (t < nfull) {
+      if (ALIGNED) {
+        // one pointer per tile for bf16 (16 decode steps of 256 rows 341 us, 360 with
+        // an index per load); fp32 at 48 registers spills less with the indices
+        // (353 rows of V = 32,000 16.6 us against 16.8)
+        const uint4* q = vp + (g0 + nb + tile_pos(tid, 0));
+        auto load = [&](int k) {
+          return ld_stream(sizeof(T) == 2 ? q + 32 * k : vp + g0 + nb + tile_pos(tid, k));
+        };
+        if (t < nfull) {
 #pragma unroll
-        for (int k = 0; k < UNR; ++k) dst[k] = load(nb + tile_pos(tid, k));
+          for (int k = 0; k < UNR; ++k) dst[k] = load(k);
+        } else {
+#pragma unroll
+          for (int k = 0; k < UNR; ++k) dst[k] = tile_pos(tid, k) < rem ? load(k) : NEG;
+        }
       } else {
-#pragma unroll
-        for (int k = 0; k < UNR; ++k)
-          dst[k] = tile_pos(tid, k) < rem ? load(nb + tile_pos(tid, k)) : NEG;
+        const bool rim = (row == 0 && rank == 0 && t == 0) ||
+                         (row == a.n_rows - 1 && rank == C - 1 && t == ntiles - 1);
+        ld_tile_off_grid(rowt, g0 + nb, g1, rim, tid, dst, ext, NEG);
       }
     };
     // one CTA per row: one thread keeps the tiles PF_TILES ahead on their way
@@ -548,18 +676,23 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Ar
     // without; with clusters, whose CTAs already keep HBM busy, it slowed
     // the step)
     auto prefetch_tile = [&](int32_t t) {
-      if (PF_TILES > 0 && ALIGNED && C == 1 && tid == 0 && t < ntiles) {
+      if (PF_TILES > 0 && C == 1 && tid == 0 && t < ntiles) {
         const int32_t gs = t * TILE;
-        prefetch_l2(vp + g0 + gs, (uint32_t)min(TILE, ng - gs) * 16u);
+        // (off the grid: the 16-byte words below the groups; t > 0)
+        prefetch_l2(reinterpret_cast<const uint4*>(reinterpret_cast<uintptr_t>(vp + g0 + gs) &
+                                                   ~(uintptr_t)15),
+                    (uint32_t)min(TILE, ng - gs) * 16u);
       }
     };
 #pragma unroll
     for (int32_t p = 1; p <= PF_TILES; ++p) prefetch_tile(p);
     uint4 cur[UNR], nxt[UNR];
-    load_tile(cur, 0);
+    uint32_t ext[UNR], ext_n[UNR];  // off the grid: the groups' fifth words
+    load_tile(cur, ext, 0);
     for (int32_t t = 0; t < ntiles; ++t) {
       prefetch_tile(t + 1 + PF_TILES);
-      if (t + 1 < ntiles) load_tile(nxt, t + 1);
+      if (t + 1 < ntiles) load_tile(nxt, ext_n, t + 1);
+      if (!ALIGNED) cut_groups(rowt, cur, ext);
       const float tmax = Tr::tile_max(cur);
       thr_max = fmaxf(thr_max, tmax);
       racc = fmaxf(racc, tmax);
@@ -584,7 +717,10 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T>()) verify_rows(const Ar
           if (tile_pos(tid, k) < rem) Tr::accum(cur[k], nm, S2, U2);
       }
 #pragma unroll
-      for (int k = 0; k < UNR; ++k) cur[k] = nxt[k];
+      for (int k = 0; k < UNR; ++k) {
+        cur[k] = nxt[k];
+        if (!ALIGNED) ext[k] = ext_n[k];
+      }
     }
   }
   float S = S2.x + S2.y, U = U2.x + U2.y;
@@ -1069,8 +1205,9 @@ __device__ __noinline__ void finalize_ws(const Args& a, SmemWS& sm, int b, int64
           const int32_t gi = (int32_t)((id & ~BEST_BIT) >> 8) * TILE + tile_pos(t, k);
           if (gi < geo.gfull) {
             gsel[q] = gi;
-            if (id & BEST_BIT) wv[q] = sm.best[b][k][t];
-            else wv[q] = ALIGNED ? ld_reread(vp + gi) : Tr::load_elems(rowp, gi);
+            if (!ALIGNED) wv[q] = Tr::load_elems(rowp, gi);
+            else if (id & BEST_BIT) wv[q] = sm.best[b][k][t];
+            else wv[q] = ld_reread(vp + gi);
           }
         }
       }
@@ -1178,6 +1315,86 @@ __device__ __noinline__ void finalize_ws(const Args& a, SmemWS& sm, int b, int64
   row_finish<T, MODE>(a, row, m, S, U, bad, E, pre, lane);
 }
 
+// Rows off the 16-byte grid (rows of an odd vocabulary stored side by side): each
+// streaming warp brings its share of a tile, as the 16-byte words of the grid
+// that cover it, into its own ring of RING_STAGES shared-memory stages with one
+// bulk copy, two tiles ahead, and cuts a group out of two neighbouring words
+// when it reads it.  The groups, and with them every sum, are those of an
+// aligned row.  The ring lies where an aligned row keeps its best tiles, so that
+// three CTAs fit an SM all the same.
+// Measured on 4,457 rows of V = 70,001 bf16 (624 MB): 144 us (4.3 TB/s); 199 us
+// when every group was loaded by its elements, 163 to 186 us with narrower loads
+// into registers, shuffles between lanes or 4-byte cp.async, whose instructions
+// kept the warps from covering the memory latency.  V = 151,935: 287 for 407 us;
+// fp32, where an element load is 4 bytes, is level (218 us for 1.25 GB).
+constexpr int RING_STAGES = 3;
+constexpr int RING_WARP = 32 * UNR * 16;    // bytes of a tile that a warp takes
+constexpr int RING_STAGE = RING_WARP + 16;  // and the word after them
+struct RingWS {
+  unsigned char stage[NWARP][RING_STAGES][RING_STAGE];
+  uint64_t bar[NWARP][RING_STAGES];  // a stage's copy has landed
+};
+constexpr size_t WS_SMEM_ALIGNED = sizeof(SmemWS);
+constexpr size_t WS_SMEM_RING = offsetof(SmemWS, best) + sizeof(RingWS);
+static_assert(offsetof(SmemWS, best) % 16 == 0 && RING_STAGE % 16 == 0, "bulk copies");
+constexpr uint64_t RING_WAIT_NS = 2000000000ull;  // a wait gives up after 2 s
+
+__device__ __forceinline__ bool ring_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// bounded wait for a stage: false (and the flag) when its copy has not landed
+static __device__ __noinline__ bool ring_wait_slow(uint32_t bar, uint32_t parity, uint32_t* flags) {
+  uint64_t t0, t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+  for (;;) {
+    for (int i = 0; i < 256; ++i)
+      if (ring_test(bar, parity)) return true;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    if (t - t0 > RING_WAIT_NS) break;
+  }
+  atomicOr(flags, FLAG_TIMEOUT);
+  return false;
+}
+// the group S bytes into the grid word at st (shared memory)
+template <int S>
+__device__ __forceinline__ uint4 ring_group(const unsigned char* st) {
+  const uint4 a = *reinterpret_cast<const uint4*>(st);
+  if (S == 0) return a;
+  uint32_t w[8] = {a.x, a.y, a.z, a.w, 0u, 0u, 0u, 0u};
+  constexpr int NEXT = (S + 3) / 4;  // words of the next grid word
+  if (NEXT == 1) {
+    w[4] = *reinterpret_cast<const uint32_t*>(st + 16);
+  } else if (NEXT == 2) {
+    const uint2 b = *reinterpret_cast<const uint2*>(st + 16);
+    w[4] = b.x;
+    w[5] = b.y;
+  } else {
+    const uint4 b = *reinterpret_cast<const uint4*>(st + 16);
+    w[4] = b.x;
+    w[5] = b.y;
+    w[6] = b.z;
+    w[7] = b.w;
+  }
+  uint32_t o[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    o[j] = (S & 2) ? __funnelshift_r(w[j + S / 4], w[j + S / 4 + 1], 16) : w[j + S / 4];
+  return make_uint4(o[0], o[1], o[2], o[3]);
+}
+template <int S>
+__device__ __forceinline__ void ring_tile(const unsigned char* st, uint4 (&c)[UNR]) {
+#pragma unroll
+  for (int k = 0; k < UNR; ++k) c[k] = ring_group<S>(st + 512 * k);
+}
+
 template <typename T, int MODE, bool ALIGNED>
 __global__ void __launch_bounds__(NT_WS, 3) verify_rows_ws(const Args a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1218,22 +1435,86 @@ __global__ void __launch_bounds__(NT_WS, 3) verify_rows_ws(const Args a) {
   const RowGeom geo(a.vocab, Tr::VEC);
   auto load_tile = [&](uint4 (&dst)[UNR], int64_t r, int32_t t) {
     const uint4* vp = reinterpret_cast<const uint4*>(rowp_of(r));
-    auto load = [&](int32_t g) -> uint4 {
-      return ALIGNED ? ld_stream(vp + g) : Tr::load_elems(vp, g);
-    };
     const int32_t base = t * TILE;
     if (t < geo.nfull) {
 #pragma unroll
-      for (int k = 0; k < UNR; ++k) dst[k] = load(base + tile_pos(tid, k));
+      for (int k = 0; k < UNR; ++k) dst[k] = ld_stream(vp + base + tile_pos(tid, k));
     } else {
 #pragma unroll
       for (int k = 0; k < UNR; ++k)
-        dst[k] = tile_pos(tid, k) < geo.rem ? load(base + tile_pos(tid, k)) : NEG;
+        dst[k] = tile_pos(tid, k) < geo.rem ? ld_stream(vp + base + tile_pos(tid, k)) : NEG;
     }
   };
+  // off the grid: this warp's ring, and the next tile to bring in
+  RingWS& ring = *reinterpret_cast<RingWS*>(smem_raw + offsetof(SmemWS, best));
+  int64_t ahead_row = blockIdx.x;
+  int32_t ahead_t = 0;
+  int ahead_stage = 0, stage = 0;
+  uint32_t parity = 0u;
+  bool landed = true;
+  auto bring = [&]() {
+    if (ahead_row >= a.n_rows || !landed) return;
+    const char* rp = rowp_of(ahead_row);
+    const int s = (int)(reinterpret_cast<uintptr_t>(rp) & 15u);
+    const int32_t g = ahead_t * TILE + warp * (32 * UNR);  // the warp's first group
+    const int32_t n = min(32 * UNR, geo.gfull - g);        // its groups
+    // grid words [lo, hi) of the warp's share; the words that reach past the
+    // call's buffer are left out and their elements of the row copied singly
+    int32_t lo = 0, hi = n + (s ? 1 : 0);
+    const bool first = s != 0 && ahead_row == 0 && g == 0;
+    const bool last = s != 0 && ahead_row == a.n_rows - 1 && g + n == geo.gfull &&
+                      geo.nedge * (int)sizeof(T) < 16 - s;
+    unsigned char* dst = ring.stage[warp][ahead_stage];
+    if (n > 0 && (first || last)) {
+      const int el = lane * (int)sizeof(T);  // one element per lane
+      auto copy1 = [&](int at, const char* from) {
+        if (sizeof(T) == 2)
+          *reinterpret_cast<uint16_t*>(dst + at) = *reinterpret_cast<const uint16_t*>(from);
+        else
+          *reinterpret_cast<uint32_t*>(dst + at) = *reinterpret_cast<const uint32_t*>(from);
+      };
+      if (first && s + el < 16) copy1(s + el, rp + el);
+      if (last && el < s) copy1(16 * n + el, rp + 16 * (int64_t)geo.gfull - s + el);
+    }
+    if (first) lo = 1;
+    if (last) hi = n;
+    if (lane == 0 && n > 0) {
+      const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&ring.bar[warp][ahead_stage]);
+      const uint32_t bytes = (uint32_t)max(hi - lo, 0) * 16u;
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
+                   : "memory");
+      if (bytes)
+        asm volatile(
+            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
+                "r"((uint32_t)__cvta_generic_to_shared(dst + 16 * lo)),
+            "l"(rp - s + 16 * ((int64_t)g + lo)), "r"(bytes), "r"(bar)
+            : "memory");
+    }
+    if (++ahead_t == geo.ntiles) {
+      ahead_t = 0;
+      ahead_row += G;
+    }
+    ahead_stage = ahead_stage + 1 == RING_STAGES ? 0 : ahead_stage + 1;
+  };
+
   uint4 cur[UNR], nxt[UNR];
   int64_t row = blockIdx.x;
-  if (row < a.n_rows && geo.ntiles > 0) load_tile(cur, row, 0);
+  if (geo.ntiles > 0) {
+    if (ALIGNED) {
+      if (row < a.n_rows) load_tile(cur, row, 0);
+    } else {
+      if (lane == 0) {
+        for (int j = 0; j < RING_STAGES; ++j)
+          asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(
+                           (uint32_t)__cvta_generic_to_shared(&ring.bar[warp][j]))
+                       : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      }
+      __syncwarp();
+      for (int j = 0; j < RING_STAGES - 1; ++j) bring();
+    }
+  }
   int i = 0;
   while (row < a.n_rows) {
     const int b = i & 1;
@@ -1245,12 +1526,44 @@ __global__ void __launch_bounds__(NT_WS, 3) verify_rows_ws(const Args a) {
     float v1 = -INFINITY, v2 = -INFINITY, v3 = -INFINITY;
     uint32_t i1 = 0, i2 = 0;
     for (int32_t t = 0; t < geo.ntiles; ++t) {
-      if (t + 1 < geo.ntiles) load_tile(nxt, row, t + 1);
-      else if (next < a.n_rows) load_tile(nxt, next, 0);
+      if (ALIGNED) {
+        if (t + 1 < geo.ntiles) load_tile(nxt, row, t + 1);
+        else if (next < a.n_rows) load_tile(nxt, next, 0);
+      } else {
+        __syncwarp();  // every lane is done with the stage that is filled next
+        bring();
+        const bool some = t * TILE + warp * (32 * UNR) < geo.gfull;  // the warp has a share
+        const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&ring.bar[warp][stage]);
+        if (some && landed) {
+          if (!ring_test(bar, (parity >> stage) & 1u))
+            landed = ring_wait_slow(bar, (parity >> stage) & 1u, a.ctx_flags);
+          if (landed) parity ^= 1u << stage;
+        }
+        __syncwarp();
+        const unsigned char* st = ring.stage[warp][stage] + 16 * lane;
+        const int s = (int)(reinterpret_cast<uintptr_t>(rowp_of(row)) & 15u);
+        if ((s & 2) == 0) {
+          if (s == 0) ring_tile<0>(st, cur);
+          else if (s == 4) ring_tile<4>(st, cur);
+          else if (s == 8) ring_tile<8>(st, cur);
+          else ring_tile<12>(st, cur);
+        } else if constexpr (sizeof(T) == 2) {
+          if (s == 2) ring_tile<2>(st, cur);
+          else if (s == 6) ring_tile<6>(st, cur);
+          else if (s == 10) ring_tile<10>(st, cur);
+          else ring_tile<14>(st, cur);
+        }
+        if (t >= geo.nfull) {
+#pragma unroll
+          for (int k = 0; k < UNR; ++k)
+            if (tile_pos(tid, k) >= geo.rem) cur[k] = NEG;
+        }
+        stage = stage + 1 == RING_STAGES ? 0 : stage + 1;
+      }
       const float tmax = Tr::tile_max(cur);
       {
         const bool c1 = tmax > v1, c2 = tmax > v2;
-        if (c1) {  // a new best tile: keep its groups for the finaliser
+        if (ALIGNED && c1) {  // a new best tile: keep its groups for the finaliser
 #pragma unroll
           for (int k = 0; k < UNR; ++k) sm.best[b][k][tid] = cur[k];
         }
@@ -1278,7 +1591,8 @@ __global__ void __launch_bounds__(NT_WS, 3) verify_rows_ws(const Args a) {
           if (tile_pos(tid, k) < geo.rem) Tr::accum(cur[k], nm, S2, U2);
       }
 #pragma unroll
-      for (int k = 0; k < UNR; ++k) cur[k] = nxt[k];
+      for (int k = 0; k < UNR; ++k)
+        if (ALIGNED) cur[k] = nxt[k];
     }
     // the warp's partial state, its sorted per-thread maxima, the tile report
     float S = S2.x + S2.y, U = U2.x + U2.y;
@@ -1296,6 +1610,10 @@ __global__ void __launch_bounds__(NT_WS, 3) verify_rows_ws(const Args a) {
     row = next;
     ++i;
   }
+  if (!ALIGNED && !landed)  // a wait ran out: no copy may be in flight when the CTA ends
+    for (int j = 0; j < RING_STAGES; ++j)
+      ring_wait_slow((uint32_t)__cvta_generic_to_shared(&ring.bar[warp][j]), (parity >> j) & 1u,
+                     a.ctx_flags);
 }
 
 // ---- standalone pooling kernel: one warp per request ----------------------------------

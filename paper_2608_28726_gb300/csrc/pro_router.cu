@@ -65,15 +65,17 @@ void* ws_kernel(pr_dtype dt, int mode, bool aligned) {
   return ws_kernel_ptr<float, prk::MODE_DECODE>(aligned);
 }
 
+size_t ws_smem(bool aligned) { return aligned ? prk::WS_SMEM_ALIGNED : prk::WS_SMEM_RING; }
+
 // shared memory opt-in and residency of the persistent kernel, once per instantiation
 pr_status ws_setup(pr_ctx* c, pr_dtype dt, int mode, bool aligned, int* bps) {
   int& v = c->ws_bps[dt == PR_DTYPE_BF16 ? 1 : 0][mode][aligned ? 1 : 0];
   if (v == 0) {
     void* f = ws_kernel(dt, mode, aligned);
     PR_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(prk::SmemWS)));
+                                 (int)ws_smem(aligned)));
     int n = 0;
-    PR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, prk::NT_WS, sizeof(prk::SmemWS)));
+    PR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, prk::NT_WS, ws_smem(aligned)));
     v = n > 0 ? n : 1;
   }
   *bps = v;
@@ -92,6 +94,8 @@ pr_status ws_setup(pr_ctx* c, pr_dtype dt, int mode, bool aligned, int* bps) {
 //    against 13.9 us with the persistent kernel);
 //  * fewer rows: the largest split (<= 8) whose CTAs still fit in one wave;
 //  * more rows: the persistent kernel.
+// The shape does not depend on the rows' alignment, so that neither do the bits
+// of the results.
 // The persistent kernel keeps a thread's best tile indices in 16 bits, so rows
 // of more than 2^16 tiles (over 536 M bf16 or 268 M fp32 values) take one CTA
 // per row instead, the forced split 1 included.
@@ -126,7 +130,7 @@ pr_status launch_rows(pr_ctx* c, pr_dtype dt, int mode, const prk::Args& a, cuda
     memset(&cfg, 0, sizeof cfg);
     cfg.gridDim = dim3((unsigned)grid, 1, 1);
     cfg.blockDim = dim3(prk::NT_WS, 1, 1);
-    cfg.dynamicSmemBytes = sizeof(prk::SmemWS);
+    cfg.dynamicSmemBytes = ws_smem(a.aligned != 0);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

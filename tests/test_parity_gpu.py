@@ -91,7 +91,7 @@ def test_features_topk(ctx, K, renorm, split):
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("shift", [1, 3])
 def test_features_unaligned_rows(ctx, dtype, shift, split):
-    """Row starts off the 16-byte grid take the element-load path."""
+    """Row starts off the 16-byte grid."""
     _set(ctx, split=split)
     V = 2053
     base, ch = random_rows(12, V + shift + 5, dtype, seed=7 + shift)
@@ -100,6 +100,32 @@ def test_features_unaligned_rows(ctx, dtype, shift, split):
     feat, top2, rf = B.pr_token_features(ctx, x, ch % V, topk=20)
     of, oi, ofl = _oracle_rows(x.contiguous(), ch % V)
     _check_features(feat, top2, rf, of, oi, ofl, "unaligned")
+    _set(ctx)
+
+
+@pytest.mark.parametrize("split", [0, 1, 8])
+@pytest.mark.parametrize("dtype,V", [(torch.bfloat16, 9000), (torch.bfloat16, 40009),
+                                     (torch.float32, 4512), (torch.float32, 20003)])
+def test_row_alignment_does_not_change_the_bits(ctx, dtype, V, split):
+    """The same rows on the 16-byte grid and at every offset from it, in buffers
+    that end with the last row's last token, give the same bits; 620 rows, so
+    that the persistent kernel's rings run across rows."""
+    _set(ctx, split=split)
+    n, step = 620, 16 // dtype.itemsize
+    src, ch = random_rows(n, V, dtype, seed=V)
+    grid = torch.zeros(n, (V + step - 1) // step * step, dtype=dtype, device="cuda")
+    grid[:, :V] = src
+    ref = B.pr_token_features(ctx, grid, ch, topk=20, vocab=V)
+    of, oi, ofl = _oracle_rows(src[::97], ch[::97])
+    _check_features(ref[0][::97], ref[1][::97], ref[2][::97], of, oi, ofl, "on the grid")
+    for shift in range(1, step):
+        for stride in {V, V + shift}:
+            flat = torch.zeros(shift + (n - 1) * stride + V, dtype=dtype, device="cuda")
+            x = flat[shift:].as_strided((n, V), (stride, 1), shift)
+            x.copy_(src)
+            got = B.pr_token_features(ctx, x, ch, topk=20)
+            for a, b in zip(got, ref):
+                assert torch.equal(a, b), (shift, stride)
     _set(ctx)
 
 
@@ -232,8 +258,8 @@ def test_persistent_candidate_paths(ctx, dtype, V, shift):
     """The persistent kernel's candidate tiles: a thread's best tile from shared
     memory, its second-best and (for a thread with three tiles above theta1)
     all its other tiles from the row, on both shared buffers (600 rows, more
-    than one per CTA); with shift 1 the rows start off the 16-byte grid and
-    take the element-load path."""
+    than one per CTA); with shift 1 the rows start off the 16-byte grid (all
+    candidates from the row)."""
     _set(ctx, split=1)
     pad = (-V) % 8 + 8  # a row stride of a multiple of 16 bytes
     base, ch = random_rows(600, V + pad, dtype, seed=4242)
