@@ -254,8 +254,12 @@ pr_status pr_aggregate_score(pr_ctx* c, const float* feat, const uint32_t* row_f
   a.ship = ship;
   a.req_flags = req_flags;
   a.ctx_flags = c->flags;
-  const unsigned grid = (unsigned)((n_req + prk::NWARP - 1) / prk::NWARP);
-  prk::pool_requests<<<grid, prk::NT, 0, reinterpret_cast<cudaStream_t>(stream)>>>(a);
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  if (n_req <= prk::POOL_FEW)
+    prk::pool_requests<1, 16><<<(unsigned)n_req, 32, 0, s>>>(a);
+  else
+    prk::pool_requests<prk::NWARP, 4>
+        <<<(unsigned)((n_req + prk::NWARP - 1) / prk::NWARP), prk::NT, 0, s>>>(a);
   PR_CUDA(cudaGetLastError());
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return PR_OK;

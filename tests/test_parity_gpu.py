@@ -103,6 +103,38 @@ def test_features_unaligned_rows(ctx, dtype, shift, split):
     _set(ctx)
 
 
+@pytest.mark.parametrize("n_req", [1, 30, 4096, 4097])
+def test_aggregate_lengths(ctx, n_req):
+    """The pooling call at the edges of its rows in flight (32, 128 and 512 rows
+    per round) and on both sides of the switch to eight requests per CTA."""
+    edges = [1, 31, 32, 33, 127, 128, 129, 511, 512, 513, 1024, 1500, 0]
+    lengths = [edges[r % len(edges)] if n_req <= 30 else r % 40 for r in range(n_req)]
+    off = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n_req)
+    feat = torch.randn(int(off[-1]), 8, generator=g, device="cuda")
+    rf = torch.zeros(int(off[-1]), dtype=torch.int32, device="cuda")
+    w = torch.randn(11, generator=g, device="cuda") * 0.3
+    bad = [r for r in range(n_req) if lengths[r] > 2][::7]
+    for r in bad:
+        rf[int(off[r + 1]) - 1] = 1
+    agg, score, ship, fl = B.pr_aggregate_score(ctx, feat, torch.from_numpy(off).cuda(), w, 0.1, 0.5,
+                                                row_flags=rf)
+    f = feat.double().cpu().numpy()[:, [0, 1, 2, 3, 4]] * np.array([1, 1, 1, -1, 1])
+    want = np.full((n_req, 11), np.nan)
+    for r in range(n_req):
+        v = f[off[r]:off[r + 1]]
+        if len(v) and r not in bad:
+            want[r, 0:10:2], want[r, 1:10:2] = v.mean(0), v.min(0)
+            want[r, 10] = (len(v) + 1) / (2 * len(v))
+    assert_close(agg.cpu().numpy(), want, "agg")
+    z = want @ w.double().cpu().numpy() + np.float32(0.1)
+    s = np.where(np.array(lengths) == 0, 0.0, 1 / (1 + np.exp(-z)))
+    assert_close(score.cpu().numpy(), s, "score")
+    want_fl = [4 if lengths[r] == 0 else int(r in bad) for r in range(n_req)]
+    assert fl.cpu().tolist() == want_fl
+
+
 @pytest.mark.parametrize("split", [0, 1, 8])
 @pytest.mark.parametrize("dtype,V", [(torch.bfloat16, 9000), (torch.bfloat16, 40009),
                                      (torch.float32, 4512), (torch.float32, 20003)])
