@@ -14,6 +14,7 @@
 struct pr_ctx {
   int device = 0;
   int num_sms = 0;
+  int sm_smem = 0;                // shared memory of an SM (bytes)
   int64_t max_rows = 0;
   int32_t max_requests = 0;
   // options
@@ -40,6 +41,8 @@ struct pr_ctx {
   cudaEvent_t ev_free[2] = {nullptr, nullptr};
   // occupancy cache per (dtype, mode)
   int bps[2][3] = {{0, 0, 0}, {0, 0, 0}};
+  // split kernel: shared memory opt-in made, per (dtype, mode, aligned)
+  bool rows_ready[2][3][2] = {};
   // persistent kernel: CTAs per SM per (dtype, mode, aligned); 0 = not set up yet
   int ws_bps[2][3][2] = {};
   // scorer head: activation scratch (rows x prk::HSCR floats), grown on demand

@@ -69,6 +69,7 @@ struct HeadArgs {
   uint8_t* ship;
   uint32_t* req_flags;
   uint32_t* ctx_flags;
+  int32_t early;              // PR_OPT_OVERLAP
   // head_rows: the layer whose attention output is consumed (null for the
   // QKV-only launch) and the layer whose QKV is produced (null for the last)
   const float* lcur;
@@ -114,7 +115,9 @@ constexpr int HEMB_CHUNK = 256;
 __global__ void __launch_bounds__(NT) head_embed(const HeadArgs a) {
   __shared__ float2 pe_g[HD / 2];
   __shared__ __align__(16) float4 xs[HEMB_CHUNK];
-  pdl_trigger();
+  // the row kernels read the weights before their own wait: they may start
+  // once what precedes the call is complete (or at once with PR_OPT_OVERLAP)
+  pdl_enter(a.early != 0);
   pdl_wait();
   int64_t lo, hi;
   if (!head_request(a, blockIdx.x, lo, hi)) return;

@@ -13,11 +13,10 @@ using namespace prh;
 
 namespace {
 
-// One kernel of the scorer head's chain; `pdl` lets it start while the
-// previous kernel on the stream finishes (it waits before reading that
-// kernel's results).
+// One kernel of the scorer head's chain; it may start while the previous
+// kernel on the stream finishes (it waits before reading that kernel's results).
 pr_status launch_head(pr_ctx* c, const void* kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                      bool pdl, const prk::HeadArgs& a) {
+                      const prk::HeadArgs& a) {
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
   cfg.gridDim = grid;
@@ -28,7 +27,7 @@ pr_status launch_head(pr_ctx* c, const void* kernel, dim3 grid, dim3 block, size
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
+  cfg.numAttrs = 1;
   void* args[] = {const_cast<prk::HeadArgs*>(&a)};
   PR_CUDA(cudaLaunchKernelExC(&cfg, kernel, args));
   g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -100,11 +99,12 @@ pr_status pr_head_score(pr_ctx* c, const float* feat, const uint32_t* row_flags,
   a.ship = ship;
   a.req_flags = req_flags;
   a.ctx_flags = c->flags;
+  a.early = c->overlap;
   const float* layer0 = w + prk::H_PRE;
   auto layer = [&](int l) { return layer0 + (int64_t)l * prk::HL_SIZE; };
   const dim3 blk(prk::NT);
   st = launch_head(c, reinterpret_cast<const void*>(&prk::head_embed),
-                   dim3((unsigned)n_req, prk::HES), blk, 0, s, c->overlap != 0, a);
+                   dim3((unsigned)n_req, prk::HES), blk, 0, s, a);
   if (st != PR_OK) return st;
   if (n_rows > 0) {
     // one CTA per 128-row tile (the row kernels hold all 512 TMEM columns of an SM)
@@ -113,7 +113,7 @@ pr_status pr_head_score(pr_ctx* c, const float* feat, const uint32_t* row_flags,
     a.lcur = nullptr;
     a.lnext = layer(0);
     st = launch_head(c, reinterpret_cast<const void*>(&prk::head_rows<prk::HR_QKV>), dim3(ntiles),
-                     rblk, prk::HT_SMEM, s, true, a);
+                     rblk, prk::HT_SMEM, s, a);
     if (st != PR_OK) return st;
     // CTAs per (request, head): one per query block of a request of the mean
     // length, at least HA_QZ_MIN.  A CTA whose request has no block z exits at
@@ -127,20 +127,19 @@ pr_status pr_head_score(pr_ctx* c, const float* feat, const uint32_t* row_flags,
         prk::HA_QZ_MAX, std::max<int64_t>(prk::HA_QZ_MIN, (mean_t + prk::HA_M - 1) / prk::HA_M));
     for (int l = 0; l < n_layers; ++l) {
       st = launch_head(c, reinterpret_cast<const void*>(&prk::head_attn),
-                       dim3((unsigned)n_req, prk::HHEADS, gz), dim3(prk::HA_M), prk::HA_SMEM, s,
-                       true, a);
+                       dim3((unsigned)n_req, prk::HHEADS, gz), dim3(prk::HA_M), prk::HA_SMEM, s, a);
       if (st != PR_OK) return st;
       a.lcur = layer(l);
       const bool last = l + 1 == n_layers;
       a.lnext = last ? nullptr : layer(l + 1);
       const void* k = last ? reinterpret_cast<const void*>(&prk::head_rows<prk::HR_LAST>)
                            : reinterpret_cast<const void*>(&prk::head_rows<prk::HR_MID>);
-      st = launch_head(c, k, dim3(ntiles), rblk, prk::HT_SMEM, s, true, a);
+      st = launch_head(c, k, dim3(ntiles), rblk, prk::HT_SMEM, s, a);
       if (st != PR_OK) return st;
     }
   }
   return launch_head(c, reinterpret_cast<const void*>(&prk::head_pool), dim3((unsigned)n_req), blk, 0,
-                     s, true, a);
+                     s, a);
 }
 
 }  // extern "C"

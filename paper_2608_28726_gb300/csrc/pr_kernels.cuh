@@ -633,7 +633,7 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T, ALIGNED>()) verify_rows
   asm("mov.u32 %0, %%clusterid.x;" : "=r"(cid));
   const int64_t row = cid;
 
-  pdl_trigger();  // a dependent launch may start streaming while this one finishes
+  pdl_enter(a.early);
   if (C > 1) cluster_arrive();  // every CTA of the cluster has started (waited for below)
 
   const char* rowp = reinterpret_cast<const char*>(a.logits) + row * a.row_stride * (int64_t)sizeof(T);
@@ -1432,7 +1432,7 @@ __global__ void __launch_bounds__(NT_WS, 3) verify_rows_ws(const Args a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t G = gridDim.x;
 
-  pdl_trigger();  // a dependent launch may start streaming while this one finishes
+  pdl_enter(a.early);
 
   auto rowp_of = [&](int64_t r) {
     return reinterpret_cast<const char*>(a.logits) + r * a.row_stride * (int64_t)sizeof(T);
@@ -1674,6 +1674,7 @@ struct AggArgs {
 // internal linkage: the header is included by more than one translation unit
 template <int WARPS, int AHEAD>
 static __global__ void __launch_bounds__(32 * WARPS) pool_requests(const AggArgs a) {
+  pdl_enter(false);
   const int lane = threadIdx.x & 31;
   const int64_t r = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
   if (r >= a.n_req) return;

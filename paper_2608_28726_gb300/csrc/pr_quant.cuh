@@ -530,6 +530,7 @@ __global__ void __launch_bounds__(Q_NT, 3) qmlp_requests(const QArgs a) {
   __shared__ uint32_t wfl[Q_NT / 32];
   __shared__ uint32_t qx[4][Q_SMALL];  // exchange between the two warps of a column
   __shared__ float zpart[2];
+  pdl_enter(false);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t r = blockIdx.x;
   const int64_t lo = a.offsets[r], hi = a.offsets[r + 1];

@@ -45,8 +45,19 @@ pr_status pr_quantile_score(pr_ctx* c, const float* feat, const uint32_t* row_fl
                                  (int)(prk::Q_DYN * sizeof(uint32_t))));
     c->qmlp_ready = true;
   }
-  prk::qmlp_requests<<<(unsigned)n_req, prk::Q_NT, prk::Q_DYN * sizeof(uint32_t), s>>>(a);
-  PR_CUDA(cudaGetLastError());
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof cfg);
+  cfg.gridDim = dim3((unsigned)n_req);
+  cfg.blockDim = dim3(prk::Q_NT);
+  cfg.dynamicSmemBytes = prk::Q_DYN * sizeof(uint32_t);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  void* args[] = {&a};
+  PR_CUDA(cudaLaunchKernelExC(&cfg, reinterpret_cast<void*>(&prk::qmlp_requests), args));
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return timing_mark(c, s);
 }

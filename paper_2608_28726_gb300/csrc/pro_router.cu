@@ -116,8 +116,9 @@ LaunchShape choose_launch(pr_ctx* c, pr_dtype dt, int mode, int64_t n_rows, int6
   return {s, s == 1 && ws_fits};
 }
 
-pr_status launch_rows(pr_ctx* c, pr_dtype dt, int mode, const prk::Args& a, cudaStream_t st) {
+pr_status launch_rows(pr_ctx* c, pr_dtype dt, int mode, prk::Args& a, cudaStream_t st) {
   if (a.n_rows == 0) return PR_OK;
+  a.early = c->overlap;
   const LaunchShape shape = choose_launch(c, dt, mode, a.n_rows, a.vocab);
   const int C = shape.C;
   if (shape.persistent) {
@@ -136,8 +137,8 @@ pr_status launch_rows(pr_ctx* c, pr_dtype dt, int mode, const prk::Args& a, cuda
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = c->overlap ? 1 : 0;
-    void* args[] = {const_cast<prk::Args*>(&a)};
+    cfg.numAttrs = 1;
+    void* args[] = {&a};
     PR_CUDA(cudaLaunchKernelExC(&cfg, ws_kernel(dt, mode, a.aligned != 0), args));
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return PR_OK;
@@ -147,8 +148,26 @@ pr_status launch_rows(pr_ctx* c, pr_dtype dt, int mode, const prk::Args& a, cuda
   memset(&cfg, 0, sizeof cfg);
   cfg.gridDim = dim3((unsigned)(a.n_rows * C), 1, 1);
   cfg.blockDim = dim3(prk::NT, 1, 1);
-  cfg.dynamicSmemBytes = 0;
   cfg.stream = st;
+  // A launch that follows another of these finds its CTAs still on the SMs and
+  // would be spread around them, three on one SM and one on the next (16 decode
+  // steps of 256 rows then took 306, 388 or 428 us, whichever pattern the launches
+  // fell into).  Unused shared memory holds every SM to its even share; with
+  // the overlap option launches are meant to run side by side.
+  if (!c->overlap) {
+    const int share = (int)((a.n_rows * C + c->num_sms - 1) / c->num_sms);
+    if (share < blocks_per_sm(c, dt, mode)) {
+      bool& ready = c->rows_ready[dt == PR_DTYPE_BF16 ? 1 : 0][mode][a.aligned ? 1 : 0];
+      void* f = row_kernel(dt, mode, a.aligned != 0);
+      const int fixed = (int)sizeof(prk::Smem) + 1024;  // and what the system takes per CTA
+      if (!ready) {
+        PR_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     c->sm_smem / 2 + 1024 - fixed));
+        ready = true;
+      }
+      cfg.dynamicSmemBytes = (size_t)std::max(0, c->sm_smem / (share + 1) + 256 - fixed) & ~(size_t)127;
+    }
+  }
   cudaLaunchAttribute attr[2];
   int na = 0;
   if (C > 1) {
@@ -158,14 +177,12 @@ pr_status launch_rows(pr_ctx* c, pr_dtype dt, int mode, const prk::Args& a, cuda
     attr[na].val.clusterDim.z = 1;
     ++na;
   }
-  if (c->overlap) {
-    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[na].val.programmaticStreamSerializationAllowed = 1;
-    ++na;
-  }
+  attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[na].val.programmaticStreamSerializationAllowed = 1;
+  ++na;
   cfg.attrs = attr;
   cfg.numAttrs = na;
-  void* args[] = {const_cast<prk::Args*>(&a)};
+  void* args[] = {&a};
   PR_CUDA(cudaLaunchKernelExC(&cfg, row_kernel(dt, mode, a.aligned != 0), args));
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return PR_OK;
@@ -254,13 +271,22 @@ pr_status pr_aggregate_score(pr_ctx* c, const float* feat, const uint32_t* row_f
   a.ship = ship;
   a.req_flags = req_flags;
   a.ctx_flags = c->flags;
-  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (n_req <= prk::POOL_FEW)
-    prk::pool_requests<1, 16><<<(unsigned)n_req, 32, 0, s>>>(a);
-  else
-    prk::pool_requests<prk::NWARP, 4>
-        <<<(unsigned)((n_req + prk::NWARP - 1) / prk::NWARP), prk::NT, 0, s>>>(a);
-  PR_CUDA(cudaGetLastError());
+  const bool few = n_req <= prk::POOL_FEW;
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof cfg);
+  cfg.gridDim = dim3(few ? (unsigned)n_req : (unsigned)((n_req + prk::NWARP - 1) / prk::NWARP));
+  cfg.blockDim = dim3(few ? 32 : prk::NT);
+  cfg.stream = reinterpret_cast<cudaStream_t>(stream);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  void* args[] = {&a};
+  PR_CUDA(cudaLaunchKernelExC(&cfg,
+                              few ? reinterpret_cast<void*>(&prk::pool_requests<1, 16>)
+                                  : reinterpret_cast<void*>(&prk::pool_requests<prk::NWARP, 4>),
+                              args));
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return PR_OK;
 }

@@ -1,0 +1,84 @@
+"""The calls keep their stream's order although each may be set up while the
+kernel before it runs: inputs written by the kernel just before a call, by
+another stream joined with an event, and calls back to back on one context,
+eagerly and in a captured graph."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2608_28726_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2608_28726_gb300 import binding
+    return binding
+
+
+def _calls(B, ctx, x, ch, off, feat, hw, qw, w, out):
+    """route, features + pooling, a decode step, the head and the quantile scorer, back to back"""
+    score, ship, fl, agg, rec, top2, rf, hs, hsh, hf, qs, qsh, qf, qsum, ds, dsh, df, da = out
+    n = x.size(0)
+    B.pr_route(ctx, x, ch, off, w, 0.1, 0.5, score=score, ship=ship, req_flags=fl, agg=agg)
+    B.pr_token_features(ctx, x, ch, 20, off, rec, top2, rf)
+    B.pr_aggregate_score(ctx, rec, off, w, 0.1, 0.5, rf, agg, score, ship, fl)
+    slot = torch.arange(n, dtype=torch.int32, device="cuda")
+    eos = torch.ones(n, dtype=torch.uint8, device="cuda")
+    B.pr_decode_step(ctx, x, slot, ch, eos, w, 0.1, 0.5, ds, dsh, df, da)
+    B.pr_head_score(ctx, feat, off, hw, 1, 0.5, rf, hs, hsh, hf)
+    B.pr_quantile_score(ctx, feat, off, qw, 0.5, rf, qsum, qs, qsh, qf)
+
+
+@pytest.mark.parametrize("n,V", [(9, 20000), (200, 9001), (700, 5000)])
+def test_inputs_written_just_before_a_call(B, n, V):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    x0 = torch.randn(n, V, generator=g, device="cuda").bfloat16()
+    ch = torch.randint(0, V, (n,), generator=g, device="cuda", dtype=torch.int32)
+    off = torch.tensor([0, n // 3, n // 3, n], dtype=torch.int64, device="cuda")
+    feat_np, _ = W.head_features([n], 5)
+    f0 = torch.from_numpy(feat_np).cuda()
+    hw, qw = torch.from_numpy(W.head_weights(1)).cuda(), torch.from_numpy(W.qmlp_weights()).cuda()
+    w = torch.randn(11, generator=g, device="cuda") * 0.1
+    f32, u8, i32 = torch.float32, torch.uint8, torch.int32
+    spec = [((3,), f32), ((3,), u8), ((3,), i32), ((3, 11), f32), ((n, 8), f32), ((n, 2), i32),
+            ((n,), i32), ((3,), f32), ((3,), u8), ((3,), i32), ((3,), f32), ((3,), u8), ((3,), i32),
+            ((3, 28), f32), ((n,), f32), ((n,), u8), ((n,), i32), ((n, 11), f32)]
+    out = [torch.zeros(s, dtype=d, device="cuda") for s, d in spec]
+    ctx = B.pr_ctx_create(0, n, max(n, 3))
+    x, feat = x0.clone(), f0.clone()
+    args = (B, ctx, x, ch, off, feat, hw, qw, w, out)
+    _calls(*args)
+    torch.cuda.synchronize()
+    ref = [t.clone() for t in out]
+
+    def same():
+        return all(np.array_equal(a.cpu().numpy(), b.cpu().numpy(), equal_nan=a.is_floating_point())
+                   for a, b in zip(out, ref))
+
+    for _ in range(10):
+        for t in (*out, x, feat):
+            t.zero_()
+        feat.copy_(f0)
+        x.copy_(x0)
+        _calls(*args)
+        assert same()
+    side, main = torch.cuda.Stream(), torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=main):
+        for t in (*out, x, feat):
+            t.zero_()
+        side.wait_stream(main)
+        with torch.cuda.stream(side):
+            x.copy_(x0)
+            feat.copy_(f0)
+        main.wait_stream(side)
+        _calls(*args)
+        _calls(*args)
+    for _ in range(5):
+        graph.replay()
+        torch.cuda.synchronize()
+        assert same()
+    B.pr_ctx_destroy(ctx)
