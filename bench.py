@@ -1531,7 +1531,7 @@ def run_quantile_workload(args):
 
 
 SEL_FILES = ("pr_device.cuh", "pr_select.cuh", "pr_select_api.cu")
-SEL_PROFILE = os.path.join(ROOT, "profiles", "sel_scatter_u32_pool16m.md")
+SEL_PROFILE = os.path.join(ROOT, "profiles", "sel_bucket_u32_pool16m.md")
 SEL_N = 1 << 24
 
 
@@ -1547,7 +1547,7 @@ def sel_oracle_child(n: int):
 
 def run_selective_workload(args):
     """Coverage calibration plus AUROC / AUARC on a 2^24-score validation pool
-    (pr_selective_metrics): one radix sort and the metric scans per step."""
+    (pr_selective_metrics): one partition into buckets and their groups per step."""
     rank, world, local = dist_env()
     if world > 1:
         import torch.distributed as dist
@@ -1601,7 +1601,7 @@ def run_selective_workload(args):
     B.pr_ctx_set_option(ctx, B.PR_OPT_TIMING, 0)
     clocks = sampler.summary(t_wall0, t_wall1)
     sampler.stop()
-    scatter_ms = float(np.mean([k[i] for k in kms for i in (3, 6, 9, 12)]))
+    bucket_ms = float(np.mean([k[6] for k in kms]))
     per_kernel = np.mean(np.asarray(kms), axis=0).tolist()
     got = res["r"]
 
@@ -1624,9 +1624,9 @@ def run_selective_workload(args):
 
     peaks_file = os.path.join(ROOT, "MEASURED_PEAKS.json")
     peak = float(json.load(open(peaks_file))["hbm_gbs"]) if os.path.exists(peaks_file) else 6800.0
-    scatter_bytes = 10 * n  # read key + label, write key + label
-    step_bytes = 80 * n
-    achieved = scatter_bytes / (scatter_ms / 1e3) / 1e9
+    bucket_bytes = 4 * n  # read the items
+    step_bytes = 22 * n  # scores 3 times, labels twice, items written and read
+    achieved = bucket_bytes / (bucket_ms / 1e3) / 1e9
     if rank == 0:
         env = dict(os.environ, OMP_NUM_THREADS="1", OPENBLAS_NUM_THREADS="1", MKL_NUM_THREADS="1")
         out = subprocess.run([sys.executable, os.path.abspath(__file__), "--sel-oracle-child",
@@ -1649,9 +1649,9 @@ def run_selective_workload(args):
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak,
                          "traffic": profiled_file_traffic(SEL_PROFILE, SEL_FILES),
-                         "kernel": "sel_scatter (radix pass)",
-                         "algorithmic_bytes_per_launch": scatter_bytes,
-                         "avg_launch_ms": scatter_ms,
+                         "kernel": "sel_bucket",
+                         "algorithmic_bytes_per_launch": bucket_bytes,
+                         "avg_launch_ms": bucket_ms,
                          "step_algorithmic_bytes": step_bytes,
                          "step_achieved_gbs": step_bytes / (ms / 1e3) / 1e9,
                          "isolated_kernel_ms": per_kernel, "isolated_step_ms": iso_ms},

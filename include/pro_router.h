@@ -161,9 +161,10 @@ pr_status pr_last_error(pr_ctx* ctx, uint32_t* flags);
  * Per-kernel device times (milliseconds, launch order) of the last call made
  * with PR_OPT_TIMING = 1: for pr_head_score the embedding, the first QKV
  * projection, then per layer the attention and the row-local block, then the
- * pool; for pr_selective_metrics the key transform, per radix pass the
- * histogram, digit scan and scatter, then the label prefix, the tile scan,
- * the metrics (with labels) and the final reduction.  Waits for the call's last event.  Writes min(count, cap) values to
+ * pool; for pr_selective_metrics the histogram of leading bits, the plan of
+ * the buckets, their counts, their offsets, the scatter into them, the counts of
+ * crowded ones (above 65,535 scores), the buckets' groups and the final
+ * reduction.  Waits for the call's last event.  Writes min(count, cap) values to
  * `ms` and the count to *n (0 if no timed call was made).
  */
 pr_status pr_ctx_kernel_times(pr_ctx* ctx, float* ms, int32_t cap, int32_t* n);
@@ -453,10 +454,10 @@ typedef struct {
  *   out     host struct, written before the call returns
  * A tie group's order is undefined, so AUARC spreads its correct answers
  * evenly over its ranks (the expectation over orders) and AUROC counts ties
- * as 1/2.  Runs as one stable radix sort of the scores plus scans on
- * `stream` (17 kernels) and synchronises it; results are deterministic.  The
- * context holds a sort workspace of about 15 bytes per score, allocated (or
- * grown) by the first call with more scores than before -- that call
+ * as 1/2.  Runs as one partition of the scores into buckets, each resolved in
+ * shared memory, on `stream` (7 or 8 kernels) and synchronises it; results are
+ * deterministic.  The context holds a workspace of 8 to 14 bytes per score
+ * (0.3 MB for a few thousand), allocated (or grown) by the first call with more scores than before -- that call
  * synchronises the device.
  */
 pr_status pr_selective_metrics(pr_ctx* ctx, const float* scores, const uint8_t* labels, int64_t n,

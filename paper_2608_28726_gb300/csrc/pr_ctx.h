@@ -49,11 +49,10 @@ struct pr_ctx {
   float* head_scr = nullptr;
   int64_t head_scr_rows = 0;
   bool head_ready = false;
-  // pr_selective_metrics: sort workspace for up to sel_cap scores, grown on demand
+  // pr_selective_metrics: workspace of sel_cap bytes, grown on demand
   void* sel_ws = nullptr;
   int64_t sel_cap = 0;
-  // its persistent radix scatter: resident CTAs per SM; 0 = not set up yet
-  int sel_scatter_bps = 0;
+  bool sel_ready = false;  // shared memory opt-ins made
   // pr_lmhead_features: per-(row, split) states, grown on demand
   void* lm_parts = nullptr;
   size_t lm_parts_bytes = 0;

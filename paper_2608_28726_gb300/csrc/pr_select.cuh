@@ -3,41 +3,100 @@
 // coverage rule with ship fraction q, AUROC and AUARC, the area under the
 // accuracy of what ships against the fraction shipped).
 //
-// Everything follows from one ascending sort of the scores: a stable LSD radix
-// sort of 32-bit order-preserving keys carrying the 0/1 label, 8 bits per pass
-// (per-tile digit histograms, a per-digit scan over tiles, a scatter that
-// ranks equal digits inside a warp with match.any, keeping the order of equal
-// keys, and writes each digit's run contiguously).  Non-finite scores map to the largest key and sort last; the
-// metrics use the n_f finite ones.  In the sorted array a tie group is a run
-// of equal keys; a prefix count of labels gives every group's correct and
-// incorrect counts, from which
-//   AUROC  = sum over correct items of (incorrect below + 1/2 incorrect tied)
-//            / (P N), summed exactly in integers (twice the numerator),
-//   AUARC  = (1/n_f) sum over descending ranks k of C_k / k, C_k spreading a
-//            tie group's correct answers evenly over its ranks; each term as
-//            a float pair (about 44 bits), summed with compensation per
-//            thread, then in fp64 in a fixed order (per tile, over tiles),
-//   tau    = the k-th largest finite score, k = min(floor(q n + 1/2), n_f).
+// Everything follows from the scores' ascending order, in which the finite
+// scores' order-preserving 32-bit keys form tie groups (runs of equal keys); a
+// group of c items, p of them correct, with a items and Pa correct ones below
+// it, contributes
+//   to AUROC  p (2 (a - Pa) + (c - p)), twice its correct items' count of
+//             incorrect items below plus half the tied ones (exact integers),
+//   to AUARC  sum over its descending ranks k of C_k / k, C_k spreading its
+//             correct answers evenly over its ranks; each term as a float pair
+//             (about 44 bits), summed with compensation per thread, then in
+//             fp64 in a fixed order (a long group in closed form, in fp64),
+// and tau is the key of the group that holds ascending rank n_f - k, k =
+// min(floor(q n + 1/2), n_f), n_f the number of finite scores.
+//
+// No pass sorts the pool.  The keys are partitioned into buckets of consecutive
+// keys, and each bucket is resolved in shared memory:
+//   sel_coarse   a histogram of the keys' 12 leading bits
+//   sel_plan     each such bin is cut into 1 to 64 equal buckets, enough for
+//                about `target` items each: at most SB_NB buckets
+//   sel_count    items and correct items per bucket; each share of the pool
+//                learns its place in every bucket from the atomic that adds it
+//   sel_offsets  prefix sums over the buckets
+//   sel_scatter  the items, as (key's offset in its bucket, label) in one word,
+//                into their buckets (the order inside a bucket does not matter)
+//   sel_heavy    buckets of more than SB_HEAVY items counted per key by many CTAs
+//   sel_bucket   one bucket at a time: a crowded one by counting items and labels
+//                for each of its keys, a light one by sorting it; then its groups
+//   sel_finish   the buckets' sums in bucket order
+// Results do not depend on the order in which items reach their buckets, so
+// they are deterministic.  2^24 scores (sigmoids of normals): 495 us; a radix
+// sort of keys and labels with scans and a pass over the sorted items took 787, of
+// which the ranking of equal digits alone 425.  100,000 scores: 62 us against 130.
+// sel_bucket takes 270 of the 495, bound by the issue of the groups' arithmetic
+// (two CTAs with twice the registers per SM instead of three: the same within 2%
+// either way, by the spread of the keys); sel_scatter 143, bound by its partly
+// filled 32-byte sectors (a share has some 70 bytes for each bucket).  Scores of
+// random bits in pools of a million, some 250 items in each of 4,095 coarse bins,
+// stay the weakest pool: 158 us against 153.
 #pragma once
 
 #include "pr_device.cuh"
 
 namespace prk {
 
-constexpr int SEL_NT = 256;                 // threads per CTA
-constexpr int SEL_IPT = 8;                  // items per thread
-constexpr int SEL_TILE = SEL_NT * SEL_IPT;  // items per tile
-constexpr int SR_IPT = 16;                  // items per thread in the radix passes: longer
-constexpr int SR_TILE = SEL_NT * SR_IPT;    // digit runs per tile, half the tile counts
-constexpr int SEL_RADIX = 256;
-constexpr int SEL_FEW_DIGITS = 16;          // a pass with at most this many digits ranks by match.any
+constexpr int SB_NT = 512;            // threads per CTA
+constexpr int SB_SHIFT = 20;          // a coarse bin: 2^20 consecutive keys
+constexpr int SB_BINS = 1 << (32 - SB_SHIFT);
+constexpr int SB_MAXB = 6;            // a bin has at most 2^6 buckets
+constexpr int SB_TARGET = 1024;       // items per bucket aimed at, where the pool is large
+constexpr int SB_FEW_TARGET = 256;    //   enough for 64 buckets of that many; at least
+constexpr int SB_NB = SB_BINS + 2 * 8192 + 1;  // most buckets (a bin of c items over the
+                                      //   target has fewer than 2 c / target; n / target <= 8192)
+constexpr int SB_SHARE = 61440;       // most items of a share (16-bit counts)
+constexpr int SB_VBITS = SB_SHIFT - SB_MAXB;  // keys counted at once: 2^14
+constexpr int SB_SMALL = 128;         // most items of a bucket resolved by one warp (10,000
+                                      //   random bit patterns: 70 us, by CTAs 143; with 256
+                                      //   here a million of them 296 us instead of 158)
+constexpr int SB_LIGHT = 4096;        // most items sorted in shared memory
+constexpr int SB_HEAVY = 65535;       // more items than this: counted by several CTAs, in
+constexpr int SB_CHUNK = 32768;       //   chunks of this many
+constexpr int SB_RADIX = 4096;        // first step of sorting a light bucket
+constexpr int SB_RUN = 24;            // most items of a sub-bin sorted by its thread
+constexpr int SB_LONG = 64;           // most near groups: in closed form from here on
 constexpr uint32_t SEL_NONFINITE = 0xffffffffu;
+static_assert(SB_NB < 65536 && SB_SHARE <= 65535, "16-bit bucket numbers and counts");
 
-struct SelResult {        // written by sel_finish, copied to the host
+struct SelResult {        // written by sel_bucket and sel_finish, copied to the host
   float tau;
   int32_t pad;
   int64_t n_finite, k, n_ship, n_pos;
   double auroc, auarc, acc_shipped;
+};
+
+struct SelArgs {
+  const float* scores;
+  const uint8_t* labels;       // or null
+  uint32_t n, share, target, nbcap;
+  double q;
+  uint32_t* coarse;            // [SB_BINS] items per coarse bin       (zeroed)
+  unsigned long long* total;   // [nbcap] items | correct << 32        (zeroed)
+  uint32_t* info;              // buckets, finite, correct, next of the list, heavy buckets,
+                               //   their chunks, crowded and light buckets (zeroed)
+  uint32_t* plan;              // [SB_BINS] first bucket | log2 buckets << 16
+  uint32_t* bkey;              // [nbcap] first key | log2 keys
+  uint32_t* start;             // [nbcap + 1] items before the bucket
+  uint32_t* pstart;            // [nbcap + 1] correct items before it
+  uint32_t* rel;               // [shares][nbcap] a share's place in each bucket
+  uint32_t* items;             // [n] offset in the bucket << 1 | label
+  uint32_t* list;              // [nbcap] crowded buckets from the front, light from the back
+  uint32_t* hidx;              // [nbcap] a heavy bucket's number
+  uint2* hchunk;               // bucket and chunk of each chunk of the heavy buckets
+  unsigned long long* hcnt;    // [heavy][2^SB_VBITS] items | correct << 32 per key
+  unsigned long long* proc;    // [nbcap] AUROC and
+  double* parc;                // [nbcap] AUARC sums of a bucket
+  SelResult* out;
 };
 
 // finite score -> order-preserving key (-0 and +0 share one key)
@@ -50,571 +109,696 @@ __device__ __forceinline__ float sel_unkey(uint32_t k) {
   return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
 
-// keys, labels and the count of finite scores (one atomic per CTA); a thread
-// takes 4 consecutive scores per step, vector loads when the pointers allow
-__global__ void __launch_bounds__(SEL_NT) sel_init(const float* __restrict__ scores,
-                                                   const uint8_t* __restrict__ labels, int64_t n,
-                                                   uint32_t* __restrict__ key,
-                                                   uint8_t* __restrict__ val,
-                                                   unsigned long long* n_finite) {
-  __shared__ uint32_t wsum[SEL_NT / 32];
-  const int64_t base = (int64_t)blockIdx.x * SEL_TILE;
-  const bool vec = ((reinterpret_cast<uintptr_t>(scores) | reinterpret_cast<uintptr_t>(labels)) &
-                    15u) == 0;
-  uint32_t fin = 0;
-#pragma unroll
-  for (int j = 0; j < SEL_IPT / 4; ++j) {
-    const int64_t i = base + 4 * ((int64_t)j * SEL_NT + threadIdx.x);
-    if (i + 3 < n && vec) {
-      const float4 f = *reinterpret_cast<const float4*>(scores + i);
-      uint32_t lab = 0;
-      if (labels) lab = *reinterpret_cast<const uint32_t*>(labels + i);
-      const uint4 k = make_uint4(sel_key(f.x), sel_key(f.y), sel_key(f.z), sel_key(f.w));
-      *reinterpret_cast<uint4*>(key + i) = k;
-      const uint32_t v = (lab & 0x000000ffu ? 1u : 0u) | (lab & 0x0000ff00u ? 0x100u : 0u) |
-                         (lab & 0x00ff0000u ? 0x10000u : 0u) | (lab & 0xff000000u ? 0x1000000u : 0u);
-      *reinterpret_cast<uint32_t*>(val + i) = v;
-      fin += (k.x != SEL_NONFINITE) + (k.y != SEL_NONFINITE) + (k.z != SEL_NONFINITE) +
-             (k.w != SEL_NONFINITE);
-    } else {
-      for (int e = 0; e < 4; ++e)
-        if (i + e < n) {
-          const uint32_t k = sel_key(scores[i + e]);
-          key[i + e] = k;
-          val[i + e] = labels ? (labels[i + e] != 0) : 0;
-          fin += k != SEL_NONFINITE;
-        }
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) fin += __shfl_xor_sync(FULL, fin, o);
-  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = fin;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t t = 0;
-    for (int w = 0; w < SEL_NT / 32; ++w) t += wsum[w];
-    if (t) atomicAdd(n_finite, (unsigned long long)t);
-  }
-}
-
-// counts[d * ntiles + tile] = items of `tile` whose digit at `shift` is d
-// (per-warp sub-histograms keep the shared-memory atomics apart)
-__global__ void __launch_bounds__(SEL_NT) sel_hist(const uint32_t* __restrict__ key, int64_t n,
-                                                   int shift, uint32_t* __restrict__ counts,
-                                                   int64_t ntiles) {
-  __shared__ uint32_t h[SEL_NT / 32][SEL_RADIX];
-  const int warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int w = 0; w < SEL_NT / 32; ++w) h[w][threadIdx.x] = 0;
-  __syncthreads();
-  const int64_t base = (int64_t)blockIdx.x * SR_TILE;
-#pragma unroll
-  for (int j = 0; j < SR_IPT / 4; ++j) {
-    const int64_t i = base + 4 * ((int64_t)j * SEL_NT + threadIdx.x);
-    if (i + 3 < n) {
-      const uint4 k = *reinterpret_cast<const uint4*>(key + i);
-      atomicAdd(&h[warp][(k.x >> shift) & 0xff], 1u);
-      atomicAdd(&h[warp][(k.y >> shift) & 0xff], 1u);
-      atomicAdd(&h[warp][(k.z >> shift) & 0xff], 1u);
-      atomicAdd(&h[warp][(k.w >> shift) & 0xff], 1u);
-    } else {
-      for (int e = 0; e < 4; ++e)
-        if (i + e < n) atomicAdd(&h[warp][(key[i + e] >> shift) & 0xff], 1u);
-    }
-  }
-  __syncthreads();
-  uint32_t c = 0;
-#pragma unroll
-  for (int w = 0; w < SEL_NT / 32; ++w) c += h[w][threadIdx.x];
-  counts[(int64_t)threadIdx.x * ntiles + blockIdx.x] = c;
-}
-
-// CTA d: exclusive scan of counts[d][0 .. ntiles) in place; total[d] = the sum.
-// Windows of 8,192 counts are staged in shared memory with coalesced loads
-// (one padding word per 32 so that a thread's 32 consecutive counts sit in 32
-// banks); thread t scans counts [32 t, 32 t + 32) of the window, one block scan
-// gives every thread its start, and the prefixes go back with coalesced
-// stores.
-constexpr int SEL_SCAN_W = SEL_NT * 32;  // counts per window
-
-__global__ void __launch_bounds__(SEL_NT) sel_scan_digit(uint32_t* __restrict__ counts,
-                                                         int64_t ntiles,
-                                                         uint32_t* __restrict__ total) {
-  __shared__ uint32_t buf[SEL_SCAN_W + SEL_SCAN_W / 32];
-  __shared__ uint32_t ws[SEL_NT / 32];
-  uint32_t* c = counts + (int64_t)blockIdx.x * ntiles;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint32_t carry = 0;
-  for (int64_t w0 = 0; w0 < ntiles; w0 += SEL_SCAN_W) {
-    const int m = ntiles - w0 < SEL_SCAN_W ? (int)(ntiles - w0) : SEL_SCAN_W;
-#pragma unroll 8
-    for (int i = 0; i < 32; ++i) {
-      const int idx = i * SEL_NT + tid;
-      buf[idx + (idx >> 5)] = idx < m ? c[w0 + idx] : 0u;
-    }
-    __syncthreads();
-    uint32_t* mine = buf + tid * 33;
-    uint32_t sum = 0;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) sum += mine[j];
-    uint32_t x = sum;  // inclusive scan of the thread sums
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(FULL, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) ws[warp] = x;
-    __syncthreads();
-    uint32_t run = carry + x - sum, all = 0;
-#pragma unroll
-    for (int w = 0; w < SEL_NT / 32; ++w) {
-      if (w < warp) run += ws[w];
-      all += ws[w];
-    }
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const uint32_t v = mine[j];
-      mine[j] = run;
-      run += v;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int i = 0; i < 32; ++i) {
-      const int idx = i * SEL_NT + tid;
-      if (idx < m) c[w0 + idx] = buf[idx + (idx >> 5)];
-    }
-    carry += all;
-    __syncthreads();  // buf and ws are reused by the next window
-  }
-  if (tid == 0) total[blockIdx.x] = carry;
-}
-
-// Stable scatter of the tiles by the digit at `shift`.  Persistent: CTA b
-// takes tiles b, b + grid, b + 2 grid, ..., and loads the next tile's keys,
-// labels and offsets while it ranks and writes the current one.  Warp w owns
-// items [w * 512, (w + 1) * 512) of a tile in 16 rounds of 32 consecutive
-// items; the lanes holding the same digit in a round are found (with
-// match.any, or with eight ballots, see sel_scatter) and ranked by lane,
-// rounds in order, so the tile order of equal digits is kept.  The tile is then laid out in shared memory in digit order
-// and written out in that order: each digit's run goes to consecutive
-// addresses.  Indices are 32-bit (n < 2^31).
-struct SelScatterSmem {
-  uint32_t wcnt[SEL_NT / 32][SEL_RADIX];
-  uint32_t gbase[SEL_RADIX];  // global position of the tile's first item of digit d,
-                              // minus the digit's offset inside the tile
-  uint32_t toff[SEL_RADIX];   // offset of digit d inside the tile
-  uint32_t ws[SEL_NT / 32], ws2[SEL_NT / 32];
-  uint32_t sk[SR_TILE];
-  uint8_t sv[SR_TILE];
-};
-
-template <bool BALLOT>
-__device__ __forceinline__ void sel_scatter_body(const uint32_t* __restrict__ key_in,
-                                                      const uint8_t* __restrict__ val_in,
-                                                      int64_t n64, int shift,
-                                                      const uint32_t* __restrict__ counts,
-                                                      int64_t ntiles64,
-                                                      const uint32_t* __restrict__ total,
-                                                      uint32_t* __restrict__ key_out,
-                                                      uint8_t* __restrict__ val_out,
-                                                      SelScatterSmem& sh) {
-  auto& wcnt = sh.wcnt;
-  auto& gbase = sh.gbase;
-  auto& toff = sh.toff;
-  auto& ws = sh.ws;
-  auto& ws2 = sh.ws2;
-  auto& sk = sh.sk;
-  auto& sv = sh.sv;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t n = (uint32_t)n64, ntiles = (uint32_t)ntiles64;
-  constexpr int PER_WARP = SR_TILE / (SEL_NT / 32);
-  const unsigned lt = (1u << lane) - 1u;
-  const uint32_t tv = total[tid];
-  uint32_t k[SR_IPT];
-  uint8_t v[SR_IPT];
-  uint32_t bt = 0;  // items of digit tid in the tiles before the current one
-  auto fetch = [&](uint32_t t, uint32_t (&kk)[SR_IPT], uint8_t (&vv)[SR_IPT], uint32_t& b) {
-    const uint32_t base = t * (uint32_t)SR_TILE + (uint32_t)warp * PER_WARP;
-#pragma unroll
-    for (int r = 0; r < SR_IPT; ++r) {
-      const uint32_t i = base + r * 32 + lane;
-      kk[r] = i < n ? key_in[i] : 0u;
-      vv[r] = i < n ? val_in[i] : 0;
-    }
-    b = counts[(size_t)tid * ntiles + t];
-  };
-  uint32_t tile = blockIdx.x;
-  if (tile < ntiles) fetch(tile, k, v, bt);
-  for (; tile < ntiles; tile += gridDim.x) {
-    const uint32_t next = tile + gridDim.x;
-    uint32_t kn[SR_IPT];
-    uint8_t vn[SR_IPT];
-    uint32_t btn = 0;
-    if (next < ntiles) fetch(next, kn, vn, btn);  // in flight while this tile is done
-#pragma unroll
-    for (int w = 0; w < SEL_NT / 32; ++w) wcnt[w][tid] = 0;
-    __syncthreads();
-    const uint32_t tile0 = tile * (uint32_t)SR_TILE;
-    const uint32_t base = tile0 + (uint32_t)warp * PER_WARP;
-    const uint32_t nt = n - tile0 < (uint32_t)SR_TILE ? n - tile0 : (uint32_t)SR_TILE;
-    uint32_t pos[SR_IPT];
-#pragma unroll
-    for (int r = 0; r < SR_IPT; ++r) {
-      const bool ok = base + r * 32 + lane < n;
-      const uint32_t d = (k[r] >> shift) & 0xff;
-      unsigned peers;  // the lanes holding digit d (lanes without an item group apart)
-      if (!BALLOT) {
-        peers = __match_any_sync(FULL, ok ? d : SEL_RADIX);  // SEL_RADIX: no item
-      } else {
-        peers = __ballot_sync(FULL, ok);
-        if (!ok) peers = ~peers;
-#pragma unroll
-        for (int bit = 0; bit < 8; ++bit) {
-          const unsigned bal = __ballot_sync(FULL, (d >> bit) & 1u);
-          peers &= ((d >> bit) & 1u) ? bal : ~bal;
-        }
-      }
-      const uint32_t rank = __popc(peers & lt);
-      const uint32_t before = ok ? wcnt[warp][d] : 0u;
-      __syncwarp();
-      if (ok && rank == 0) wcnt[warp][d] = before + __popc(peers);
-      __syncwarp();
-      pos[r] = before + rank;
-    }
-    __syncthreads();
-    {
-      // per digit (thread tid = digit): exclusive prefix over the warps, and
-      // the tile's count of the digit
-      uint32_t run = 0;
-#pragma unroll
-      for (int w = 0; w < SEL_NT / 32; ++w) {
-        const uint32_t c = wcnt[w][tid];
-        wcnt[w][tid] = run;
-        run += c;
-      }
-      // exclusive scans over digits: of the tile's counts, and of the totals
-      uint32_t x = run, y = tv;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t xx = __shfl_up_sync(FULL, x, o), yy = __shfl_up_sync(FULL, y, o);
-        if (lane >= o) {
-          x += xx;
-          y += yy;
-        }
-      }
-      if (lane == 31) {
-        ws[warp] = x;
-        ws2[warp] = y;
-      }
-      __syncthreads();
-      uint32_t xb = 0, yb = 0;
-      for (int w = 0; w < warp; ++w) {
-        xb += ws[w];
-        yb += ws2[w];
-      }
-      const uint32_t tile_off_d = xb + x - run;
-      toff[tid] = tile_off_d;
-      gbase[tid] = (yb + y - tv) + bt - tile_off_d;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < SR_IPT; ++r) {
-      const uint32_t i = base + r * 32 + lane;
-      if (i < n) {
-        const uint32_t d = (k[r] >> shift) & 0xff;
-        const uint32_t p = toff[d] + wcnt[warp][d] + pos[r];
-        sk[p] = k[r];
-        sv[p] = v[r];
-      }
-    }
-    __syncthreads();
-    for (uint32_t j = tid; j < nt; j += SEL_NT) {
-      const uint32_t kk = sk[j];
-      const uint32_t o = gbase[(kk >> shift) & 0xff] + j;
-      key_out[o] = kk;
-      val_out[o] = sv[j];
-    }
-    __syncthreads();  // sk, sv, gbase, toff and wcnt are free for the next tile
-#pragma unroll
-    for (int r = 0; r < SR_IPT; ++r) {
-      k[r] = kn[r];
-      v[r] = vn[r];
-    }
-    bt = btn;
-  }
-}
-
-// The warp ranking's method: match.any costs more the more distinct digits a
-// warp holds, eight ballots (one per digit bit) cost the same for any mix.
-// A pass whose keys hold few digits (the top byte of scores that share an
-// exponent range) takes match.any, the others the ballots; the choice is one
-// branch around the whole body, so each method compiles on its own.
-__global__ void __launch_bounds__(SEL_NT) sel_scatter(const uint32_t* __restrict__ key_in,
-                                                      const uint8_t* __restrict__ val_in,
-                                                      int64_t n64, int shift,
-                                                      const uint32_t* __restrict__ counts,
-                                                      int64_t ntiles64,
-                                                      const uint32_t* __restrict__ total,
-                                                      uint32_t* __restrict__ key_out,
-                                                      uint8_t* __restrict__ val_out) {
-  __shared__ SelScatterSmem sh;
-  if (__syncthreads_count(total[threadIdx.x] != 0u) <= SEL_FEW_DIGITS)
-    sel_scatter_body<false>(key_in, val_in, n64, shift, counts, ntiles64, total, key_out, val_out,
-                            sh);
-  else
-    sel_scatter_body<true>(key_in, val_in, n64, shift, counts, ntiles64, total, key_out, val_out,
-                           sh);
-}
-
-// per tile: inclusive prefix of the labels inside the tile (first n_f items)
-// and the tile's total.  Thread t owns items 8 t .. 8 t + 7 of the tile: one
-// 8-byte load of labels, two 16-byte stores of prefixes.
-__global__ void __launch_bounds__(SEL_NT) sel_label_prefix(const uint8_t* __restrict__ val,
-                                                           const unsigned long long* n_finite,
-                                                           uint32_t* __restrict__ pre,
-                                                           uint32_t* __restrict__ tile_sum) {
-  static_assert(SEL_IPT == 8, "one 8-byte vector of labels per thread");
-  __shared__ uint32_t ws[SEL_NT / 32];
-  const int64_t nf = (int64_t)*n_finite;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t base = (int64_t)blockIdx.x * SEL_TILE + (int64_t)tid * SEL_IPT;  // blocked
-  uint32_t lab[2] = {0u, 0u};
-  if (base + SEL_IPT <= nf) {
-    const uint2 q = *reinterpret_cast<const uint2*>(val + base);
-    lab[0] = q.x;
-    lab[1] = q.y;
-  } else {
-    for (int j = 0; j < SEL_IPT; ++j)
-      if (base + j < nf) lab[j >> 2] |= (uint32_t)val[base + j] << (8 * (j & 3));
-  }
-  uint32_t c[SEL_IPT], run = 0;
-#pragma unroll
-  for (int j = 0; j < SEL_IPT; ++j) {
-    run += (lab[j >> 2] >> (8 * (j & 3))) & 0xffu;
-    c[j] = run;
-  }
-  uint32_t x = run;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(FULL, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) ws[warp] = x;
-  __syncthreads();
-  uint32_t wbase = 0, all = 0;
-#pragma unroll
-  for (int w = 0; w < SEL_NT / 32; ++w) {
-    if (w < warp) wbase += ws[w];
-    all += ws[w];
-  }
-  const uint32_t off = wbase + x - run;
-  if (base + SEL_IPT <= nf) {
-#pragma unroll
-    for (int q = 0; q < 2; ++q)
-      *reinterpret_cast<uint4*>(pre + base + 4 * q) =
-          make_uint4(off + c[4 * q], off + c[4 * q + 1], off + c[4 * q + 2], off + c[4 * q + 3]);
-  } else {
-    for (int j = 0; j < SEL_IPT; ++j)
-      if (base + j < nf) pre[base + j] = off + c[j];
-  }
-  if (tid == 0) tile_sum[blockIdx.x] = all;
-}
-
-// exclusive scan of the tile sums (one CTA; the total goes to tile_off[ntiles])
-__global__ void __launch_bounds__(1024) sel_scan_tiles(uint32_t* __restrict__ tile_sum,
-                                                       int64_t ntiles,
-                                                       uint32_t* __restrict__ tile_off) {
-  __shared__ uint32_t ws[32];
-  __shared__ uint32_t carry;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  for (int64_t t0 = 0; t0 < ntiles; t0 += 1024) {
-    const int64_t t = t0 + threadIdx.x;
-    const uint32_t v = t < ntiles ? tile_sum[t] : 0u;
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(FULL, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) ws[warp] = x;
-    __syncthreads();
-    uint32_t wbase = 0, all = 0;
-    for (int w = 0; w < 32; ++w) {
-      if (w < warp) wbase += ws[w];
-      all += ws[w];
-    }
-    const uint32_t c0 = carry;
-    if (t < ntiles) tile_off[t] = c0 + wbase + x - v;
-    __syncthreads();
-    if (threadIdx.x == 0) carry = c0 + all;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) tile_off[ntiles] = carry;
-}
-
-// Indices and counts below are 32-bit (n < 2^31): 64-bit integer arithmetic
-// and 64-bit integer <-> float conversions run on the fp64 pipe, which is
-// narrow on this GPU.
-struct SelView {
-  const uint32_t* key;  // sorted keys
-  const uint32_t* pre;  // in-tile inclusive label prefix
-  const uint32_t* tile_off;
-  uint32_t nf;
-};
-
-// correct answers among the first x sorted items
-__device__ __forceinline__ uint32_t sel_P(const SelView& s, uint32_t x) {
-  if (x == 0) return 0;
-  const uint32_t i = x - 1;
-  return s.tile_off[i / SEL_TILE] + s.pre[i];
-}
-
-// [a, b): the run of keys equal to key[i]: up to 8 neighbours each way,
-// then a binary search for long runs
-__device__ __forceinline__ void sel_group(const SelView& s, uint32_t i, uint32_t& a, uint32_t& b) {
-  const uint32_t k = s.key[i];
-  a = i;
-  int steps = 0;
-  while (a > 0 && s.key[a - 1] == k && steps < 8) {
-    --a;
-    ++steps;
-  }
-  if (a > 0 && s.key[a - 1] == k) {  // first index in [0, a) with key == k
-    uint32_t lo = 0, hi = a - 1;
-    while (lo < hi) {
-      const uint32_t mid = lo + ((hi - lo) >> 1);
-      if (s.key[mid] < k) lo = mid + 1; else hi = mid;
-    }
-    a = lo;
-  }
-  b = i + 1;
-  steps = 0;
-  while (b < s.nf && s.key[b] == k && steps < 8) {
-    ++b;
-    ++steps;
-  }
-  if (b < s.nf && s.key[b] == k) {  // first index in (b, nf) with key > k
-    uint32_t lo = b + 1, hi = s.nf;
-    while (lo < hi) {
-      const uint32_t mid = lo + ((hi - lo) >> 1);
-      if (s.key[mid] <= k) lo = mid + 1; else hi = mid;
-    }
-    b = lo;
-  }
-}
-
-// C / k for integers 0 <= C < 2^31, 1 <= k < 2^31 as an unevaluated sum hi + lo of two
-// floats (about 44 correct bits) without fp64: C and k are split by bit masks
-// into parts that floats hold exactly, a correctly rounded fp32 reciprocal
-// gives the first quotient q, fmaf gives the remainder C - q k with single
-// roundings, and the remainder times the reciprocal is the correction.
+// C / k for integers 0 <= C <= k < 2^31 as an unevaluated sum hi + lo of two floats
+// without fp64: a correctly rounded fp32 reciprocal gives the first quotient q,
+// fmaf gives the remainder C - q k, and the remainder times the reciprocal is
+// the correction (about 46 correct bits).  Below 2^24 both integers are floats and
+// the remainder is exact; from there on they are split by bit masks into parts
+// that floats hold.
 __device__ __forceinline__ float2 sel_ratio(uint32_t C, uint32_t k) {
-  const float kh = (float)(k & ~0xffu), kl = (float)(k & 0xffu);
-  const float ch = (float)(C & ~0xffu), cl = (float)(C & 0xffu);
-  const float r = __frcp_rn((float)k);
-  const float q = (ch + cl) * r;
-  const float rem = fmaf(-q, kh, ch) + fmaf(-q, kl, cl);
+  const float r = __frcp_rn((float)k), q = __fmul_rn((float)C, r);
+  float rem;
+  if (k < 1u << 24) {
+    rem = fmaf(-q, (float)k, (float)C);
+  } else {
+    const float kh = (float)(k & ~0xffu), kl = (float)(k & 0xffu);
+    const float ch = (float)(C & ~0xffu), cl = (float)(C & 0xffu);
+    rem = fmaf(-q, kh, ch) + fmaf(-q, kl, cl);
+  }
   return make_float2(q, rem * r);
 }
 
-// Per tile: twice the AUROC numerator (integers) and the AUARC sum of its
-// finite items: per thread a compensated float-float sum in item order (no
-// fp64 in the loop), then fp64 over a fixed-order block tree.
-__global__ void __launch_bounds__(SEL_NT) sel_metrics(const uint32_t* __restrict__ key,
-                                                      const uint8_t* __restrict__ val,
-                                                      const uint32_t* __restrict__ pre,
-                                                      const uint32_t* __restrict__ tile_off,
-                                                      const unsigned long long* n_finite,
-                                                      int64_t ntiles,
-                                                      unsigned long long* __restrict__ part_roc,
-                                                      double* __restrict__ part_arc) {
-  __shared__ double sd[SEL_NT];
-  __shared__ unsigned long long su[SEL_NT];
-  SelView s{key, pre, tile_off, (uint32_t)*n_finite};
-  const uint32_t Ptot = tile_off[ntiles];
-  const int tid = threadIdx.x;
-  float fs = 0.f, fc = 0.f;  // compensated float-float sum of the thread's terms
-  unsigned long long roc2 = 0;
-  const uint32_t base = blockIdx.x * (uint32_t)SEL_TILE + (uint32_t)tid;
-#pragma unroll 2
-  for (int j = 0; j < SEL_IPT; ++j) {
-    const uint32_t i = base + (uint32_t)j * SEL_NT;
-    if (i < s.nf) {
-      uint32_t a, b;
-      sel_group(s, i, a, b);
-      const uint32_t Pa = sel_P(s, a), Pb = sel_P(s, b);
-      const uint32_t pos_g = Pb - Pa, n_g = b - a;
-      if (val[i]) roc2 += 2ull * (a - Pa) + (n_g - pos_g);
-      const uint32_t k = s.nf - i;      // descending rank, 1-based
-      const uint32_t above = s.nf - b;  // items ranked before the group
-      // C_k / k = (correct answers above the group) / k + (m / n_g)(pos_g / k)
-      // with m = k - above members of the group shipped: float-float ratios
-      // and one float-float product, the roundings carried into fc (a plain
-      // fp32 term would round the same way for every k of a long tie group)
-      float th, tl;
-      if (n_g == 1) {
-        const float2 t = sel_ratio(Ptot - Pb + pos_g, k);
-        th = t.x;
-        tl = t.y;
-      } else {
-        const float2 t1 = sel_ratio(Ptot - Pb, k);
-        const float2 u1 = sel_ratio(k - above, n_g), u2 = sel_ratio(pos_g, k);
-        const float p = u1.x * u2.x;
-        const float pl = fmaf(u1.x, u2.x, -p) + fmaf(u1.x, u2.y, u1.y * u2.x);
-        th = t1.x + p;  // two-sum of the high parts
-        const float bv = th - t1.x;
-        tl = ((t1.x - (th - bv)) + (p - bv)) + (t1.y + pl);
-      }
-      const float u = fs + th;  // two-sum into the running pair (fs, fc)
-      const float bv = u - fs;
-      fc += ((fs - (u - bv)) + (th - bv)) + tl;
-      fs = u;
+// body(key, label) for the scores i, i + 1, .. of [lo, hi) that this thread takes;
+// vector loads when the pointers allow (lo is a multiple of 4)
+template <typename F>
+__device__ __forceinline__ void sel_each(const SelArgs& a, uint32_t lo, uint32_t hi, uint32_t first,
+                                         uint32_t step, bool labels, F body) {
+  const bool vec = ((reinterpret_cast<uintptr_t>(a.scores) |
+                     reinterpret_cast<uintptr_t>(a.labels)) & 15u) == 0;
+  auto one = [&](float s, uint32_t lab) {
+    const uint32_t k = sel_key(s);
+    if (k != SEL_NONFINITE) body(k, lab);
+  };
+  if (vec) {
+#pragma unroll 4
+    for (uint64_t i = (uint64_t)lo + 4ull * first; i + 3 < hi; i += 4ull * step) {
+      const float4 f = __ldg(reinterpret_cast<const float4*>(a.scores + i));
+      const uint32_t l = labels ? __ldg(reinterpret_cast<const uint32_t*>(a.labels + i)) : 0u;
+      one(f.x, (l & 0xffu) ? 1u : 0u);
+      one(f.y, (l & 0xff00u) ? 1u : 0u);
+      one(f.z, (l & 0xff0000u) ? 1u : 0u);
+      one(f.w, (l & 0xff000000u) ? 1u : 0u);
     }
-  }
-  sd[tid] = (double)fs + (double)fc;
-  su[tid] = roc2;
-  __syncthreads();
-  for (int h = SEL_NT / 2; h > 0; h >>= 1) {
-    if (tid < h) {
-      sd[tid] += sd[tid + h];
-      su[tid] += su[tid + h];
-    }
-    __syncthreads();
-  }
-  if (tid == 0) {
-    part_arc[blockIdx.x] = sd[0];
-    part_roc[blockIdx.x] = su[0];
+    const uint32_t rest = lo + ((hi - lo) & ~3u);
+    if (rest + first < hi && first < 4u)
+      one(a.scores[rest + first], labels && a.labels[rest + first] ? 1u : 0u);
+  } else {
+    for (uint64_t i = (uint64_t)lo + first; i < hi; i += step)
+      one(a.scores[i], labels && a.labels[i] ? 1u : 0u);
   }
 }
 
-// One CTA: sums of the tile partials in tile order, then tau and the counts.
-__global__ void __launch_bounds__(SEL_NT) sel_finish(const uint32_t* __restrict__ key,
-                                                     const uint32_t* __restrict__ pre,
-                                                     const uint32_t* __restrict__ tile_off,
-                                                     const unsigned long long* n_finite,
-                                                     int64_t n, int64_t ntiles, double q,
-                                                     int has_labels,
-                                                     const unsigned long long* part_roc,
-                                                     const double* part_arc,
-                                                     SelResult* __restrict__ out) {
-  __shared__ double sd[SEL_NT];
-  __shared__ unsigned long long su[SEL_NT];
+__global__ void __launch_bounds__(SB_NT) sel_coarse(const SelArgs a) {
+  __shared__ uint32_t h[SB_BINS];
+  pdl_enter(false);
+  for (int i = threadIdx.x; i < SB_BINS; i += SB_NT) h[i] = 0u;
+  __syncthreads();
+  sel_each(a, 0u, a.n, blockIdx.x * SB_NT + threadIdx.x, gridDim.x * SB_NT, false,
+           [&](uint32_t k, uint32_t) { atomicAdd(&h[k >> SB_SHIFT], 1u); });
+  __syncthreads();
+  for (int i = threadIdx.x; i < SB_BINS; i += SB_NT)
+    if (h[i]) atomicAdd(a.coarse + i, h[i]);
+}
+
+// exclusive prefix of two counts over the CTA's threads (NT of them), and the totals
+template <int NT>
+__device__ __forceinline__ void sel_scan2(uint32_t& x, uint32_t& y, uint32_t& xall, uint32_t& yall,
+                                          uint32_t (*ws)[NT / 32]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t ix = x, iy = y;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t xx = __shfl_up_sync(FULL, ix, o), yy = __shfl_up_sync(FULL, iy, o);
+    if (lane >= o) {
+      ix += xx;
+      iy += yy;
+    }
+  }
+  __syncthreads();  // ws may still be read from the scan before
+  if (lane == 31) {
+    ws[0][warp] = ix;
+    ws[1][warp] = iy;
+  }
+  __syncthreads();
+  uint32_t bx = 0, by = 0;
+  xall = yall = 0;
+#pragma unroll
+  for (int w = 0; w < NT / 32; ++w) {
+    if (w == warp) {
+      bx = xall;
+      by = yall;
+    }
+    xall += ws[0][w];
+    yall += ws[1][w];
+  }
+  x = bx + ix - x;
+  y = by + iy - y;
+}
+
+__global__ void __launch_bounds__(1024) sel_plan(const SelArgs a) {
+  __shared__ uint32_t ws[2][32];
+  pdl_enter(false);
+  constexpr int PER = SB_BINS / 1024;
+  uint32_t c[PER], b[PER], nb = 0, nf = 0;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    c[j] = a.coarse[threadIdx.x * PER + j];
+    b[j] = 0;
+    while (b[j] < (uint32_t)SB_MAXB && (c[j] >> b[j]) > a.target) ++b[j];
+    nb += c[j] ? 1u << b[j] : 0u;
+    nf += c[j];
+  }
+  uint32_t at = nb, dummy = nf, nball, nfall;
+  sel_scan2<1024>(at, dummy, nball, nfall, ws);
+  if (threadIdx.x == 0) {
+    a.info[0] = nball;
+    a.info[1] = nfall;
+  }
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    if (!c[j]) continue;
+    const uint32_t bin = threadIdx.x * PER + j, r = SB_SHIFT - b[j];
+    a.plan[bin] = at | b[j] << 16;
+    for (uint32_t s = 0; s < 1u << b[j]; ++s)  // the low SB_VBITS bits of a first key are 0
+      a.bkey[at + s] = bin << SB_SHIFT | s << r | r;
+    at += 1u << b[j];
+  }
+}
+
+// bucket of a key, and its offset there
+__device__ __forceinline__ uint32_t sel_bucket_of(uint32_t key, const uint32_t* plan, uint32_t& off) {
+  const uint32_t p = plan[key >> SB_SHIFT], r = SB_SHIFT - (p >> 16);
+  off = key & ((1u << r) - 1u);
+  return (p & 0xffffu) + ((key & ((1u << SB_SHIFT) - 1u)) >> r);
+}
+
+// share s: items and correct items per bucket, added to the buckets' totals
+__global__ void __launch_bounds__(SB_NT, 2) sel_count(const SelArgs a) {
+  extern __shared__ uint32_t sb_dyn[];  // [SB_BINS] plan, [buckets] counts
+  uint32_t *plan = sb_dyn, *cnt = sb_dyn + SB_BINS;
+  pdl_enter(false);
+  const uint32_t nb = a.info[0];
+  for (int i = threadIdx.x; i < SB_BINS; i += SB_NT) plan[i] = a.plan[i];
+  for (uint32_t i = threadIdx.x; i < nb; i += SB_NT) cnt[i] = 0u;
+  __syncthreads();
+  const uint32_t lo = blockIdx.x * a.share, hi = min(a.n - lo, a.share) + lo;
+  sel_each(a, lo, hi, threadIdx.x, SB_NT, a.labels != nullptr, [&](uint32_t k, uint32_t lab) {
+    uint32_t off;
+    atomicAdd(cnt + sel_bucket_of(k, plan, off), 1u + (lab << 16));
+  });
+  __syncthreads();
+  uint32_t* rel = a.rel + (size_t)blockIdx.x * a.nbcap;
+  for (uint32_t i = threadIdx.x; i < nb; i += SB_NT) {
+    const uint32_t c = cnt[i];
+    if (c)
+      rel[i] = (uint32_t)atomicAdd(a.total + i, (unsigned long long)(c & 0xffffu) |
+                                                    (unsigned long long)(c >> 16) << 32);
+  }
+}
+
+// ascending rank of tau's item (the k-th largest finite score), and k
+__device__ __forceinline__ uint32_t sel_tau_rank(const SelArgs& a, uint32_t nf, int64_t& k) {
+  k = (int64_t)floor(a.q * (double)a.n + 0.5);
+  k = k < 0 ? 0 : (k > (int64_t)nf ? (int64_t)nf : k);
+  return nf - (uint32_t)k;
+}
+
+__global__ void __launch_bounds__(1024) sel_offsets(const SelArgs a) {
+  __shared__ uint32_t ws[2][32], listed[2];
+  pdl_enter(false);
+  if (threadIdx.x < 2) listed[threadIdx.x] = 0u;  // (the scan synchronises)
+  int64_t kk;
+  const uint32_t itau = sel_tau_rank(a, a.info[1], kk);
+  const uint32_t nb = a.info[0], per = (nb + 1023u) / 1024u, i0 = threadIdx.x * per;
+  uint32_t x = 0, y = 0, xall, yall;
+  for (uint32_t i = i0; i < min(i0 + per, nb); ++i) {
+    const unsigned long long t = a.total[i];
+    x += (uint32_t)t;
+    y += (uint32_t)(t >> 32);
+  }
+  sel_scan2<1024>(x, y, xall, yall, ws);
+  for (uint32_t i = i0; i < min(i0 + per, nb); ++i) {
+    const unsigned long long t = a.total[i];
+    a.start[i] = x;
+    a.pstart[i] = y;
+    // to be resolved by a CTA; without labels only tau's bucket counts
+    if ((uint32_t)t > (uint32_t)SB_SMALL && (a.labels || (kk > 0 && itau - x < (uint32_t)t))) {
+      if ((uint32_t)t > (uint32_t)SB_LIGHT) a.list[atomicAdd(listed, 1u)] = i;
+      else a.list[a.nbcap - 1u - atomicAdd(listed + 1, 1u)] = i;
+    }
+    if ((uint32_t)t > (uint32_t)SB_HEAVY && (a.bkey[i] & 31u) == (uint32_t)SB_VBITS) {
+      a.hidx[i] = atomicAdd(a.info + 4, 1u);
+      const uint32_t chunks = ((uint32_t)t + SB_CHUNK - 1) / SB_CHUNK;
+      const uint32_t at = atomicAdd(a.info + 5, chunks);
+      for (uint32_t j = 0; j < chunks; ++j) a.hchunk[at + j] = make_uint2(i, j);
+    }
+    x += (uint32_t)t;
+    y += (uint32_t)(t >> 32);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    a.info[6] = listed[0];
+    a.info[7] = listed[1];
+    a.start[nb] = xall;
+    a.pstart[nb] = yall;
+    a.info[2] = yall;
+  }
+}
+
+__global__ void __launch_bounds__(SB_NT, 2) sel_scatter(const SelArgs a) {
+  extern __shared__ uint32_t sb_dyn[];  // [SB_BINS] plan, [buckets] next places
+  uint32_t *plan = sb_dyn, *pos = sb_dyn + SB_BINS;
+  pdl_enter(false);
+  const uint32_t nb = a.info[0];
+  const uint32_t* rel = a.rel + (size_t)blockIdx.x * a.nbcap;
+  for (int i = threadIdx.x; i < SB_BINS; i += SB_NT) plan[i] = a.plan[i];
+  // (a bucket that the share has no item of has no place; it is not used)
+  for (uint32_t i = threadIdx.x; i < nb; i += SB_NT) pos[i] = a.start[i] + rel[i];
+  const uint64_t hwords = (uint64_t)a.info[4] << SB_VBITS;  // the heavy buckets' counters
+  for (uint64_t i = (uint64_t)blockIdx.x * SB_NT + threadIdx.x; i < hwords;
+       i += (uint64_t)gridDim.x * SB_NT)
+    a.hcnt[i] = 0ull;
+  __syncthreads();
+  const uint32_t lo = blockIdx.x * a.share, hi = min(a.n - lo, a.share) + lo;
+  sel_each(a, lo, hi, threadIdx.x, SB_NT, a.labels != nullptr, [&](uint32_t k, uint32_t lab) {
+    uint32_t off;
+    const uint32_t b = sel_bucket_of(k, plan, off);
+    a.items[atomicAdd(pos + b, 1u)] = off << 1 | lab;
+  });
+}
+
+constexpr int SB_WORDS = 1 << SB_VBITS;  // the counters of sel_heavy and sel_bucket
+constexpr size_t SB_BUCKET_SMEM = SB_WORDS * sizeof(uint32_t);
+
+// The heavy buckets (scores piled up on few keys, as those of a confident
+// scorer just below 1): their items counted chunk by chunk on all SMs
+__global__ void __launch_bounds__(SB_NT, 3) sel_heavy(const SelArgs a) {
+  extern __shared__ uint32_t sb_dyn[];
+  pdl_enter(false);
+  const uint32_t chunks = a.info[5];
+  for (uint32_t q = blockIdx.x; q < chunks; q += gridDim.x) {
+    const uint2 bc = a.hchunk[q];
+    const uint32_t s0 = a.start[bc.x], m = a.start[bc.x + 1] - s0;
+    const uint32_t lo = bc.y * SB_CHUNK, hi = min(lo + SB_CHUNK, m);
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < (uint32_t)SB_WORDS; i += SB_NT) sb_dyn[i] = 0u;
+    __syncthreads();
+    for (uint32_t i = lo + threadIdx.x; i < hi; i += SB_NT) {
+      const uint32_t it = a.items[s0 + i];
+      atomicAdd(sb_dyn + (it >> 1), 1u + ((it & 1u) << 16));
+    }
+    __syncthreads();
+    unsigned long long* out = a.hcnt + ((size_t)a.hidx[bc.x] << SB_VBITS);
+    for (uint32_t w = threadIdx.x; w < 1u << SB_VBITS; w += SB_NT) {
+      const uint32_t u = sb_dyn[w];
+      if (u)
+        atomicAdd(out + w, (unsigned long long)(u & 0xffffu) | (unsigned long long)(u >> 16) << 32);
+    }
+  }
+}
+
+// H(x + c) - H(x), the harmonic numbers' difference: summed up to 64, then by
+// the asymptotic series of H (its next term is below 2e-17 there)
+__device__ __forceinline__ double sel_harmonic(uint32_t x, uint32_t c) {
+  double s = 0.0;
+  while (x < 64u && c > 0u) {
+    ++x;
+    --c;
+    s += 1.0 / (double)x;
+  }
+  if (c == 0u) return s;
+  const double A = (double)x, N = A + (double)c;
+  const double u = 1.0 / A, v = 1.0 / N;
+  auto tail = [](double w) {  // 1/2n - 1/12n^2 + 1/120n^4 - 1/252n^6
+    const double w2 = w * w;
+    return w * 0.5 - w2 * (1.0 / 12.0 - w2 * (1.0 / 120.0 - w2 * (1.0 / 252.0)));
+  };
+  return s + (log1p((double)c * u) + (tail(v) - tail(u)));
+}
+
+// A thread's sums over tie groups
+struct SelSums {
+  float fs, fc;              // compensated float-float sum of AUARC terms
+  double ds;                 // long groups
+  unsigned long long roc2;   // twice the AUROC numerator
+  __device__ __forceinline__ void add(float th, float tl) {
+    const float u = fs + th;  // two-sum into the running pair (fs, fc)
+    const float bv = u - fs;
+    fc += ((fs - (u - bv)) + (th - bv)) + tl;
+    fs = u;
+  }
+  // this lane's group (if `on`) of c items, p correct, with lo items and plo
+  // correct ones below it; whole warp
+  __device__ __forceinline__ void group(bool on, uint32_t lo, uint32_t plo, uint32_t c, uint32_t p,
+                                        uint32_t nf, uint32_t ptot, int lane) {
+    const uint32_t above = nf - lo - c, cab = ptot - plo - p;
+    if (on) roc2 += (unsigned long long)p * (2ull * (lo - plo) + (c - p));
+    // sum over j = 1 .. c of (cab + p j / c) / (above + j)
+    const bool one = c == 1u, near = !one && (above >> 6 < c || c >> 23 != 0u);
+    if (on && !near) {
+      // one item: its ratio.  More: ranks M + d around their mean M = D / 2, D =
+      // 2 above + c + 1, c / M < 2^-6, 1 / (M + d) expanded to d^4 (what is left is
+      // below 2^-36 / 448 of the sum).  The leading term (2 c cab + p (c + 1)) / D
+      // as float pairs; the correction (Cm / M - p / c) (S2 / M^2 + S4 / M^4), S2
+      // and S4 = sums of d^2 and d^4, Cm the mean of the numerators, in fp32
+      // while it is below 2^-23 of the sum (c / M < 2^-10), else in fp64
+      const uint32_t D = one ? nf - lo : 2u * above + c + 1u;
+      const float2 t1 = sel_ratio(one ? ptot - plo : cab, D);
+      const float cf = (float)c, c2 = one ? 1.f : 2.f * cf;  // exact (c < 2^23)
+      const float x = __fmul_rn(t1.x, c2), xl = fmaf(t1.x, c2, -x) + t1.y * c2;
+      add(x, xl);
+      if (!one) {
+        const float2 t2 = sel_ratio(p, D);
+        const float c1 = cf + 1.f;
+        const float y = __fmul_rn(t2.x, c1), yl = fmaf(t2.x, c1, -y) + t2.y * c1;
+        const float r = 2.f / (float)D, lead = x + y;  // c Cm / M
+        float corr = 0.f;
+        if (above >> 10 >= c) {
+          corr = cf * (cf * cf - 1.f) * (1.f / 12.f) * r * r * ((lead - (float)p) / cf);
+        } else {
+          const double cd = (double)c, rd = (double)r, im = rd * (2.0 - 0.5 * (double)D * rd);
+          const double im2 = im * im, cc = cd * cd, ri = (double)(1.f / cf);
+          const double w = (((double)x + (double)y) + ((double)xl + (double)yl)) - (double)p;
+          ds += (cc - 1.0) * (1.0 / 12.0) * im2 * (1.0 + (3.0 * cc - 7.0) * 0.05 * im2) *
+                (w * (cd * ri * (2.0 - cd * ri)));
+        }
+        add(y, yl + corr);
+      }
+    }
+    // groups at the top ranks: long ones in closed form, of the others the warp
+    // takes one by one, a lane every 32nd rank
+    if (on && near && c >= (uint32_t)SB_LONG) {
+      const double dh = sel_harmonic(above, c);
+      ds += (double)cab * dh + ((double)p / (double)c) * ((double)c - (double)above * dh);
+    }
+    unsigned todo = __ballot_sync(FULL, on && near && c < (uint32_t)SB_LONG);
+    while (todo) {
+      const int src = __ffs(todo) - 1;
+      todo &= todo - 1u;
+      ranks(__shfl_sync(FULL, above, src), __shfl_sync(FULL, cab, src), __shfl_sync(FULL, c, src),
+            __shfl_sync(FULL, p, src), lane);
+    }
+  }
+  __device__ __forceinline__ void ranks(uint32_t above, uint32_t cab, uint32_t c, uint32_t p,
+                                        int lane) {
+    // rank k = above + j: (correct answers above) / k + (j / c)(p / k) as
+    // float-float ratios and one float-float product, the roundings carried
+    for (uint32_t j = 1u + lane; j <= c; j += 32u) {
+      const uint32_t k = above + j;
+      const float2 t1 = sel_ratio(cab, k);
+      const float2 u1 = sel_ratio(j, c), u2 = sel_ratio(p, k);
+      const float pr = __fmul_rn(u1.x, u2.x);  // (not to be fused into the sum below)
+      const float pl = fmaf(u1.x, u2.x, -pr) + fmaf(u1.x, u2.y, u1.y * u2.x);
+      const float th = t1.x + pr;  // two-sum of the high parts
+      const float bv = th - t1.x;
+      add(th, ((t1.x - (th - bv)) + (pr - bv)) + (t1.y + pl));
+    }
+  }
+};
+
+// word of sub-bin w: one word of padding per 32, so that the runs of 8 that
+// threads scan lie in different banks
+__device__ __forceinline__ uint32_t sel_at(uint32_t w) { return w + (w >> 5); }
+static_assert(2 * SB_LIGHT + SB_RADIX + SB_RADIX / 32 <= SB_WORDS,
+              "a light bucket, its label prefix and the sub-bins");
+static_assert(1 << SB_VBITS == 32 * SB_NT, "a strip of 32 keys per thread");
+static_assert(SB_RADIX == 8 * SB_NT && SB_LIGHT == 8 * SB_NT, "eight per thread");
+
+__global__ void __launch_bounds__(SB_NT, 3) sel_bucket(const SelArgs a) {
+  extern __shared__ uint32_t sb_dyn[];
+  __shared__ uint32_t ws[2][SB_NT / 32], next, ranges[4], strip[2][SB_NT];
+  __shared__ double sd[SB_NT / 32];
+  __shared__ unsigned long long su[SB_NT / 32];
+  pdl_enter(false);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t nb = a.info[0], nf = a.info[1], ptot = a.info[2];
+  int64_t kk;
+  const uint32_t itau = sel_tau_rank(a, nf, kk);
+  const bool metrics = a.labels != nullptr;
+  // a warp's group of keys at key0 + off; every lane of the warp calls
+  auto visit = [&](SelSums& S, bool has_tau, uint32_t key, uint32_t lo, uint32_t plo, uint32_t c,
+                   uint32_t p) {
+    if (metrics) S.group(c != 0u, lo, plo, c, p, nf, ptot, lane);
+    if (has_tau && itau - lo < c) {
+      a.out->tau = sel_unkey(key);
+      a.out->n_ship = (int64_t)(nf - lo);
+      a.out->acc_shipped = metrics ? (double)(ptot - plo) / (double)(nf - lo)
+                                   : __longlong_as_double(0x7ff8000000000000ll);
+    }
+  };
+  // ---- buckets of a few items (those of a pool spread over many coarse bins), a
+  // warp each: a lane counts the items below and equal to its own
+  uint32_t* mine = sb_dyn + warp * SB_SMALL;
+  for (uint32_t b = blockIdx.x * (SB_NT / 32) + warp; b < nb; b += gridDim.x * (SB_NT / 32)) {
+    const uint32_t s0 = a.start[b], m = a.start[b + 1] - s0, p0 = a.pstart[b];
+    const bool has_tau = kk > 0 && itau - s0 < m;
+    if (m > (uint32_t)SB_SMALL || !(metrics || has_tau)) continue;
+    SelSums S = {0.f, 0.f, 0.0, 0ull};
+    __syncwarp();
+    for (uint32_t i = lane; i < ((m + 3u) & ~3u); i += 32u)
+      mine[i] = i < m ? a.items[s0 + i] : ~0u;  // no item's offset
+    __syncwarp();
+    for (uint32_t base = 0; base < m; base += 32u) {
+      const uint32_t i = base + lane, v = i < m ? mine[i] : ~0u, key = v & ~1u;
+      uint32_t below = 0u, same = 0u, first = i;  // items | correct << 16
+#pragma unroll 2
+      for (uint32_t j = 0; j < m; j += 4u) {
+        const uint4 q = *reinterpret_cast<const uint4*>(mine + j);
+        const uint32_t u[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (uint32_t e = 0; e < 4u; ++e) {
+          const uint32_t add = 1u | (u[e] & 1u) << 16;
+          if (u[e] < key) below += add;
+          if ((u[e] ^ v) < 2u) {
+            same += add;
+            first = min(first, j + e);
+          }
+        }
+      }
+      if (i >= m || first != i) same = 0u;
+      visit(S, has_tau, (a.bkey[b] & ~31u) + (v >> 1), s0 + (below & 0xffffu), p0 + (below >> 16),
+            same & 0xffffu, same >> 16);
+    }
+    double d = ((double)S.fs + (double)S.fc) + S.ds;
+    unsigned long long u = S.roc2;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      d += __shfl_xor_sync(FULL, d, o);
+      u += __shfl_xor_sync(FULL, u, o);
+    }
+    if (lane == 0) {
+      a.parc[b] = d;
+      a.proc[b] = u;
+    }
+  }
+  // ---- the others, the crowded ones first, a CTA each
+  const uint32_t crowds = a.info[6], listed = crowds + a.info[7];
+  for (;;) {
+    __syncthreads();
+    if (tid == 0) next = atomicAdd(a.info + 3, 1u);
+    __syncthreads();
+    if (next >= listed) return;
+    const uint32_t b = a.list[next < crowds ? next : a.nbcap - 1u - (next - crowds)];
+    const uint32_t s0 = a.start[b], m = a.start[b + 1] - s0, p0 = a.pstart[b];
+    const bool has_tau = kk > 0 && itau - s0 < m;
+    const uint32_t bk = a.bkey[b], r = bk & 31u, key0 = bk & ~31u;
+    const uint32_t* items = a.items + s0;
+    SelSums S = {0.f, 0.f, 0.0, 0ull};
+    // the groups of `vals` consecutive keys from key0 + first on, with a0 items and
+    // q0 correct ones below; count(w, c, p) gives key w's.  The keys go by strips
+    // of 32, a lane per key, to the warps in turn: long tie groups come in
+    // neighbouring keys, and all warps share them.  `small`: a strip's counts
+    // fit 16 bits.  Returns the totals.
+    auto walk = [&](uint32_t first, uint32_t vals, uint32_t a0, uint32_t q0, bool small, auto count,
+                    uint32_t& xall, uint32_t& yall) {
+      const uint32_t strips = vals / 32u;  // at most one per thread
+      for (uint32_t s = warp; s < strips; s += SB_NT / 32) {
+        uint32_t c, p;
+        count(32u * s + lane, c, p);
+        c = __reduce_add_sync(FULL, c);
+        p = __reduce_add_sync(FULL, p);
+        if (lane == 0) {
+          strip[0][s] = c;
+          strip[1][s] = p;
+        }
+      }
+      __syncthreads();
+      uint32_t x = (uint32_t)tid < strips ? strip[0][tid] : 0u,
+               y = (uint32_t)tid < strips ? strip[1][tid] : 0u;
+      sel_scan2<SB_NT>(x, y, xall, yall, ws);
+      strip[0][tid] = x;
+      strip[1][tid] = y;
+      __syncthreads();
+      for (uint32_t s = warp; s < strips; s += SB_NT / 32) {
+        uint32_t c, p;
+        count(32u * s + lane, c, p);
+        if (!__any_sync(FULL, c != 0u)) continue;
+        uint32_t ic = small ? c | p << 16 : c, ip = p;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t cc = __shfl_up_sync(FULL, ic, o);
+          if (lane >= o) ic += cc;
+        }
+        if (small) {
+          ip = ic >> 16;
+          ic &= 0xffffu;
+        } else {
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t pp = __shfl_up_sync(FULL, ip, o);
+            if (lane >= o) ip += pp;
+          }
+        }
+        visit(S, has_tau, key0 + first + 32u * s + lane, a0 + strip[0][s] + ic - c, q0 + strip[1][s] + ip - p, c, p);
+      }
+    };
+    if (m <= (uint32_t)SB_LIGHT) {
+      // ---- a light bucket: sorted, then a group per run of equal offsets.  The
+      // items go to sub-bins of the offset's leading bits (about one item in
+      // each), a thread sorts each sub-bin; piled-up offsets take a bitonic
+      // sort of the whole
+      uint32_t *v = sb_dyn, *pre = sb_dyn + SB_LIGHT, *sub = pre + SB_LIGHT;
+      const uint32_t sh = r - 12u;  // 2^r keys, SB_RADIX = 2^12 sub-bins
+      uint32_t it[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) it[e] = e * SB_NT + tid < m ? items[e * SB_NT + tid] : ~0u;
+      for (uint32_t i = tid; i < SB_RADIX + SB_RADIX / 32; i += SB_NT) sub[i] = 0u;
+      __syncthreads();
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (e * SB_NT + tid < m) atomicAdd(sub + sel_at(it[e] >> 1 >> sh), 1u);
+      __syncthreads();
+      uint32_t c8[8], sx = 0, sy = 0, sxall, syall;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        c8[e] = sub[sel_at(8 * tid + e)];
+        sx += c8[e];
+      }
+      sel_scan2<SB_NT>(sx, sy, sxall, syall, ws);
+      bool crowded = false;
+      uint32_t at8 = sx;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        sub[sel_at(8 * tid + e)] = at8;
+        at8 += c8[e];
+        crowded = crowded || c8[e] > (uint32_t)SB_RUN;
+      }
+      uint32_t n2 = SB_NT;
+      while (n2 < m) n2 <<= 1;
+      if (!__syncthreads_or(crowded)) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          if (e * SB_NT + tid < m) v[atomicAdd(sub + sel_at(it[e] >> 1 >> sh), 1u)] = it[e];
+        __syncthreads();
+        at8 = sx;
+#pragma unroll 1
+        for (int e = 0; e < 8; ++e) {
+          for (uint32_t i = at8 + 1; i < at8 + c8[e]; ++i) {  // insertion sort
+            const uint32_t x = v[i];
+            uint32_t j = i;
+            for (; j > at8 && v[j - 1] > x; --j) v[j] = v[j - 1];
+            v[j] = x;
+          }
+          at8 += c8[e];
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          if (e * SB_NT + tid < n2) v[e * SB_NT + tid] = it[e];  // ~0 past the items
+        for (uint32_t k = 2; k <= n2; k <<= 1)
+          for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+            __syncthreads();
+            for (uint32_t q = tid; q < n2 >> 1; q += SB_NT) {
+              const uint32_t i = ((q & ~(j - 1u)) << 1) | (q & (j - 1u)), l = i + j;
+              const uint32_t x = v[i], y = v[l];
+              if ((x > y) == ((i & k) == 0u)) {
+                v[i] = y;
+                v[l] = x;
+              }
+            }
+          }
+      }
+      __syncthreads();
+      const uint32_t per = n2 / SB_NT, i0 = tid * per;
+      uint32_t x = 0, y = 0, xall, yall;
+      for (uint32_t i = i0; i < min(i0 + per, m); ++i) x += v[i] & 1u;
+      sel_scan2<SB_NT>(x, y, xall, yall, ws);
+      for (uint32_t i = i0; i < min(i0 + per, m); ++i) {
+        pre[i] = x;  // correct items before item i
+        x += v[i] & 1u;
+      }
+      __syncthreads();
+      for (uint32_t base = 0; base < m; base += SB_NT) {
+        const uint32_t i = base + tid;
+        uint32_t off = 0u, pi = 0u, c = 0u, p = 0u;
+        if (i < m) {
+          off = v[i] >> 1;
+          pi = pre[i];
+          if (i == 0 || v[i - 1] >> 1 != off) {
+            uint32_t e = i + 1, hi = m;  // the group's end
+            if (e < m && v[e] >> 1 == off) {
+              while (e < hi) {
+                const uint32_t mid = (e + hi) >> 1;
+                if (v[mid] >> 1 <= off) e = mid + 1;
+                else hi = mid;
+              }
+            }
+            c = e - i;
+            p = (e < m ? pre[e] : xall) - pi;
+          }
+        }
+        visit(S, has_tau, key0 + off, s0 + i, p0 + pi, c, p);
+      }
+    } else if (m > (uint32_t)SB_HEAVY && r == (uint32_t)SB_VBITS) {
+      // ---- a heavy bucket: already counted (sel_heavy)
+      const unsigned long long* hc = a.hcnt + ((size_t)a.hidx[b] << SB_VBITS);
+      uint32_t xall, yall;
+      walk(0u, 1u << SB_VBITS, s0, p0, false, [&](uint32_t w, uint32_t& c, uint32_t& p) {
+        const unsigned long long u = __ldcg(hc + w);
+        c = (uint32_t)u;
+        p = (uint32_t)(u >> 32);
+      }, xall, yall);
+    } else {
+      // ---- counted: 2^14 keys at a time (16-bit counts of items and labels), or
+      // 2^13 with 32-bit counts for a bucket of more items than 16 bits hold
+      const bool wide = m > (uint32_t)SB_HEAVY;
+      const int vb = wide ? SB_VBITS - 1 : SB_VBITS;
+      const uint32_t vals = 1u << vb;
+      uint32_t* lab = sb_dyn + vals;  // wide only
+      uint32_t a0 = s0, q0 = p0;
+      // which of the (up to 128) key ranges hold items: piled-up scores fill few
+      uint32_t used[4] = {r == (uint32_t)vb ? 1u : 0u, 0u, 0u, 0u};
+      for (uint32_t i = r == (uint32_t)vb ? m : tid; i < m; i += SB_NT) {
+        const uint32_t ps = items[i] >> 1 >> vb;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) used[e] |= ps >> 5 == (uint32_t)e ? 1u << (ps & 31u) : 0u;
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) used[e] = __reduce_or_sync(FULL, used[e]);
+      if (tid < 4) ranges[tid] = 0u;
+      __syncthreads();
+      if (lane < 4)
+        atomicOr(ranges + lane, lane == 0 ? used[0] : lane == 1 ? used[1] : lane == 2 ? used[2] : used[3]);
+      __syncthreads();
+      for (uint32_t ps = 0; ps < 1u << (r - vb); ++ps) {
+        if (!(ranges[ps >> 5] >> (ps & 31u) & 1u)) continue;
+        __syncthreads();
+        for (uint32_t i = tid; i < (uint32_t)SB_WORDS; i += SB_NT) sb_dyn[i] = 0u;
+        __syncthreads();
+        for (uint32_t i = tid; i < m; i += SB_NT) {
+          const uint32_t it = items[i], off = it >> 1;
+          if (off >> vb != ps) continue;
+          const uint32_t at = off & (vals - 1u);
+          if (!wide) {
+            atomicAdd(sb_dyn + at, 1u + ((it & 1u) << 16));
+          } else {
+            atomicAdd(sb_dyn + at, 1u);
+            if (it & 1u) atomicAdd(lab + at, 1u);
+          }
+        }
+        __syncthreads();
+        uint32_t xall, yall;
+        walk(ps << vb, vals, a0, q0, !wide, [&](uint32_t w, uint32_t& c, uint32_t& p) {
+          const uint32_t u = sb_dyn[w];
+          c = wide ? u : u & 0xffffu;
+          p = wide ? lab[w] : u >> 16;
+        }, xall, yall);
+        a0 += xall;
+        q0 += yall;
+      }
+    }
+    // the bucket's sums, in a fixed order
+    double d = ((double)S.fs + (double)S.fc) + S.ds;
+    unsigned long long u = S.roc2;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      d += __shfl_xor_sync(FULL, d, o);
+      u += __shfl_xor_sync(FULL, u, o);
+    }
+    if (lane == 0) {
+      sd[warp] = d;
+      su[warp] = u;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      for (int w = 1; w < SB_NT / 32; ++w) {
+        d += sd[w];
+        u += su[w];
+      }
+      a.parc[b] = d;
+      a.proc[b] = u;
+    }
+  }
+}
+
+// One CTA: the buckets' sums in a fixed order, and the counts.
+__global__ void __launch_bounds__(SB_NT) sel_finish(const SelArgs a) {
+  __shared__ double sd[SB_NT];
+  __shared__ unsigned long long su[SB_NT];
+  pdl_enter(false);
   const int tid = threadIdx.x;
-  const int64_t nf = (int64_t)*n_finite;
-  const int64_t nt_used = (nf + SEL_TILE - 1) / SEL_TILE;
+  const uint32_t nb = a.info[0], nf = a.info[1];
   double arc = 0.0;
   unsigned long long roc2 = 0;
-  if (has_labels)
-    for (int64_t t = tid; t < nt_used; t += SEL_NT) {  // each thread in tile order
-      arc += part_arc[t];
-      roc2 += part_roc[t];
+  if (a.labels)
+    for (uint32_t t = tid; t < nb; t += SB_NT) {  // each thread in bucket order
+      arc += a.parc[t];
+      roc2 += a.proc[t];
     }
   sd[tid] = arc;
   su[tid] = roc2;
   __syncthreads();
-  for (int h = SEL_NT / 2; h > 0; h >>= 1) {
+  for (int h = SB_NT / 2; h > 0; h >>= 1) {
     if (tid < h) {
       sd[tid] += sd[tid + h];
       su[tid] += su[tid + h];
@@ -622,31 +806,22 @@ __global__ void __launch_bounds__(SEL_NT) sel_finish(const uint32_t* __restrict_
     __syncthreads();
   }
   if (tid != 0) return;
-  SelView s{key, pre, tile_off, (uint32_t)nf};
-  SelResult r;
-  r.pad = 0;
-  r.n_finite = nf;
-  r.n_pos = has_labels ? (int64_t)tile_off[ntiles] : 0;
-  int64_t k = (int64_t)floor(q * (double)n + 0.5);
-  k = k < 0 ? 0 : (k > nf ? nf : k);
-  r.k = k;
   const double nan = __longlong_as_double(0x7ff8000000000000ll);
+  SelResult* out = a.out;
+  int64_t k;
+  sel_tau_rank(a, nf, k);
+  out->pad = 0;
+  out->n_finite = nf;
+  out->k = k;
+  const int64_t P = a.labels ? (int64_t)a.info[2] : 0, N = (int64_t)nf - P;
+  out->n_pos = P;
   if (k == 0) {
-    r.tau = __int_as_float(0x7f800000);  // +inf: nothing ships
-    r.n_ship = 0;
-    r.acc_shipped = nan;
-  } else {
-    const uint32_t i = (uint32_t)(nf - k);
-    uint32_t a, b;
-    sel_group(s, i, a, b);
-    r.tau = sel_unkey(key[i]);
-    r.n_ship = nf - a;
-    r.acc_shipped = has_labels ? (double)(r.n_pos - sel_P(s, a)) / (double)r.n_ship : nan;
+    out->tau = __int_as_float(0x7f800000);  // +inf: nothing ships
+    out->n_ship = 0;
+    out->acc_shipped = nan;
   }
-  const int64_t P = r.n_pos, N = nf - P;
-  r.auroc = (has_labels && P > 0 && N > 0) ? (double)su[0] / (2.0 * (double)P * (double)N) : nan;
-  r.auarc = (has_labels && nf > 0) ? sd[0] / (double)nf : nan;
-  *out = r;
+  out->auroc = (a.labels && P > 0 && N > 0) ? (double)su[0] / (2.0 * (double)P * (double)N) : nan;
+  out->auarc = (a.labels && nf > 0) ? sd[0] / (double)nf : nan;
 }
 
 }  // namespace prk

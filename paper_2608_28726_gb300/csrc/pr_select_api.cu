@@ -21,30 +21,58 @@ namespace {
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// byte offsets of the workspace pieces for capacity n
+// shares of the pool and most buckets of a pool of n scores
+struct SelShape {
+  uint32_t share, shares, target, nbcap, rows;
+  SelShape(int64_t n, int num_sms) {
+    // two shares per SM, not below 4,096 items (a share pays for every bucket);
+    // a multiple of 4 for the vector loads
+    const int64_t even = ((n + 2 * num_sms - 1) / (2 * num_sms) + 3) & ~(int64_t)3;
+    share = (uint32_t)std::min<int64_t>(prk::SB_SHARE, std::max<int64_t>(4096, even));
+    shares = (uint32_t)((n + share - 1) / share);
+    // a bin that holds most of a small pool is still cut into 64 buckets, whose keys
+    // are counted in one go (33,000 scores just below 1: 118 us, at 1,024 a bucket 151)
+    target = (uint32_t)std::max<int64_t>(
+        std::min<int64_t>(prk::SB_TARGET, std::max<int64_t>(prk::SB_FEW_TARGET, n / 64)),
+        (n + 8191) / 8192);
+// the workspace's bounds do not fall when n grows: n / target buckets over the
+    // coarse bins', twice, and the shares
+    nbcap = (uint32_t)(std::min<int64_t>(n, prk::SB_BINS) + 1 +
+                       2 * std::max(std::min<int64_t>(n / prk::SB_FEW_TARGET, 65),
+                                    std::min<int64_t>(n / prk::SB_TARGET, 8192)));
+    rows = (uint32_t)std::max<int64_t>(std::min<int64_t>((n + 4095) / 4096, 2 * num_sms),
+                                       (n + prk::SB_SHARE - 1) / prk::SB_SHARE);
+  }
+};
+
+// byte offsets of the workspace pieces
 struct SelLayout {
-  size_t key0, key1, val0, val1, pre, counts, total, tsum, toff, proc, parc, nf, out, bytes;
-  explicit SelLayout(int64_t n) {
-    const int64_t nt = (n + prk::SEL_TILE - 1) / prk::SEL_TILE;
+  size_t coarse, total, info, zeroed, plan, bkey, start, pstart, proc, parc, out, items, list, hidx, hchunk, hcnt, rel, bytes;
+  SelLayout(int64_t n, const SelShape& g) {
     size_t o = 0;
     auto take = [&](size_t b) {
       const size_t at = o;
       o += align256(b);
       return at;
     };
-    key0 = take((size_t)n * 4);
-    key1 = take((size_t)n * 4);
-    val0 = take((size_t)n);
-    val1 = take((size_t)n);
-    pre = take((size_t)n * 4);
-    counts = take((size_t)nt * prk::SEL_RADIX * 4);
-    total = take(prk::SEL_RADIX * 4);
-    tsum = take((size_t)nt * 4);
-    toff = take(((size_t)nt + 1) * 4);
-    proc = take((size_t)nt * 8);
-    parc = take((size_t)nt * 8);
-    nf = take(8);
+    coarse = take(prk::SB_BINS * 4);
+    total = take((size_t)g.nbcap * 8);
+    info = take(32);
+    zeroed = o;  // zeroed at the start of a call
+    plan = take(prk::SB_BINS * 4);
+    bkey = take((size_t)g.nbcap * 4);
+    start = take(((size_t)g.nbcap + 1) * 4);
+    pstart = take(((size_t)g.nbcap + 1) * 4);
+    proc = take((size_t)g.nbcap * 8);
+    parc = take((size_t)g.nbcap * 8);
     out = take(sizeof(prk::SelResult));
+    items = take((size_t)n * 4);
+    const size_t heavy = (size_t)(n / (prk::SB_HEAVY + 1));  // buckets with more than SB_HEAVY items
+    list = take((size_t)g.nbcap * 4);
+    hidx = take((size_t)g.nbcap * 4);
+    hchunk = take(((size_t)(n / prk::SB_CHUNK) + heavy + 1) * 8);
+    hcnt = take((heavy << prk::SB_VBITS) * 8);
+    rel = take((size_t)g.rows * g.nbcap * 4);
     bytes = o;
   }
 };
@@ -68,85 +96,101 @@ pr_status pr_selective_metrics(pr_ctx* c, const float* scores, const uint8_t* la
   pr_status st = set_device(c);
   if (st != PR_OK) return st;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (n > c->sel_cap) {
+  const SelShape g(n, c->num_sms);
+  const SelLayout L(n, g);
+  if ((int64_t)L.bytes > c->sel_cap) {
     PR_CUDA(cudaDeviceSynchronize());  // the old workspace may still be in use
     cudaFree(c->sel_ws);
     c->sel_ws = nullptr;
     c->sel_cap = 0;
-    const SelLayout L(n);
     if (cudaMalloc(&c->sel_ws, L.bytes) != cudaSuccess) {
       cudaGetLastError();
       c->sel_ws = nullptr;
       return PR_ERR_NO_MEMORY;
     }
-    c->sel_cap = n;
+    c->sel_cap = (int64_t)L.bytes;
   }
-  const SelLayout L(c->sel_cap);
+  const size_t share_smem = (size_t)(prk::SB_BINS + g.nbcap) * sizeof(uint32_t);
+  if (!c->sel_ready) {
+    const int most = (prk::SB_BINS + prk::SB_NB) * (int)sizeof(uint32_t);
+    PR_CUDA(cudaFuncSetAttribute(prk::sel_count, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    PR_CUDA(cudaFuncSetAttribute(prk::sel_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    PR_CUDA(cudaFuncSetAttribute(prk::sel_heavy, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)prk::SB_BUCKET_SMEM));
+    PR_CUDA(cudaFuncSetAttribute(prk::sel_bucket, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)prk::SB_BUCKET_SMEM));
+    c->sel_ready = true;
+  }
   char* w = static_cast<char*>(c->sel_ws);
-  uint32_t* key[2] = {reinterpret_cast<uint32_t*>(w + L.key0), reinterpret_cast<uint32_t*>(w + L.key1)};
-  uint8_t* val[2] = {reinterpret_cast<uint8_t*>(w + L.val0), reinterpret_cast<uint8_t*>(w + L.val1)};
-  uint32_t* pre = reinterpret_cast<uint32_t*>(w + L.pre);
-  uint32_t* counts = reinterpret_cast<uint32_t*>(w + L.counts);
-  uint32_t* total = reinterpret_cast<uint32_t*>(w + L.total);
-  uint32_t* tsum = reinterpret_cast<uint32_t*>(w + L.tsum);
-  uint32_t* toff = reinterpret_cast<uint32_t*>(w + L.toff);
-  unsigned long long* proc = reinterpret_cast<unsigned long long*>(w + L.proc);
-  double* parc = reinterpret_cast<double*>(w + L.parc);
-  unsigned long long* nf = reinterpret_cast<unsigned long long*>(w + L.nf);
-  prk::SelResult* res = reinterpret_cast<prk::SelResult*>(w + L.out);
-  const int64_t ntiles = (n + prk::SEL_TILE - 1) / prk::SEL_TILE;
-  const unsigned g_tiles = (unsigned)ntiles;
-  // the scatter is persistent: one wave of resident CTAs
-  if (c->sel_scatter_bps == 0) {
-    int b = 0;
-    PR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, prk::sel_scatter, prk::SEL_NT, 0));
-    c->sel_scatter_bps = b > 0 ? b : 1;
-  }
-  const int64_t rtiles = (n + prk::SR_TILE - 1) / prk::SR_TILE;  // tiles of the radix passes
-  const unsigned g_scatter =
-      (unsigned)std::min<int64_t>(rtiles, (int64_t)c->num_sms * c->sel_scatter_bps);
+  prk::SelArgs a;
+  memset(&a, 0, sizeof a);
+  a.scores = scores;
+  a.labels = labels;
+  a.n = (uint32_t)n;
+  a.share = g.share;
+  a.target = g.target;
+  a.nbcap = g.nbcap;
+  a.q = q;
+  a.coarse = reinterpret_cast<uint32_t*>(w + L.coarse);
+  a.total = reinterpret_cast<unsigned long long*>(w + L.total);
+  a.info = reinterpret_cast<uint32_t*>(w + L.info);
+  a.plan = reinterpret_cast<uint32_t*>(w + L.plan);
+  a.bkey = reinterpret_cast<uint32_t*>(w + L.bkey);
+  a.start = reinterpret_cast<uint32_t*>(w + L.start);
+  a.pstart = reinterpret_cast<uint32_t*>(w + L.pstart);
+  a.rel = reinterpret_cast<uint32_t*>(w + L.rel);
+  a.items = reinterpret_cast<uint32_t*>(w + L.items);
+  a.list = reinterpret_cast<uint32_t*>(w + L.list);
+  a.hidx = reinterpret_cast<uint32_t*>(w + L.hidx);
+  a.hchunk = reinterpret_cast<uint2*>(w + L.hchunk);
+  a.hcnt = reinterpret_cast<unsigned long long*>(w + L.hcnt);
+  a.proc = reinterpret_cast<unsigned long long*>(w + L.proc);
+  a.parc = reinterpret_cast<double*>(w + L.parc);
+  a.out = reinterpret_cast<prk::SelResult*>(w + L.out);
   int launches = 0;
-  // after each launch: count it, check it, and (PR_OPT_TIMING) record an event
-  auto launched = [&]() -> pr_status {
+  // one kernel of the chain, set up behind the one before it
+  auto launch = [&](void (*kernel)(prk::SelArgs), unsigned grid, unsigned block,
+                    size_t smem) -> pr_status {
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    void* args[] = {&a};
+    PR_CUDA(cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kernel), args));
     ++launches;
-    PR_CUDA(cudaGetLastError());
     return timing_mark(c, s);
   };
-#define PR_LAUNCHED()                        \
-  do {                                       \
-    if ((st = launched()) != PR_OK) return st; \
+#define PR_LAUNCH(...)                                   \
+  do {                                                   \
+    if ((st = launch(__VA_ARGS__)) != PR_OK) return st; \
   } while (0)
 
-  PR_CUDA(cudaMemsetAsync(nf, 0, sizeof *nf, s));
+  PR_CUDA(cudaMemsetAsync(w, 0, L.zeroed, s));
   if ((st = timing_begin(c, s)) != PR_OK) return st;
-  prk::sel_init<<<g_tiles, prk::SEL_NT, 0, s>>>(scores, labels, n, key[0], val[0], nf);
-  PR_LAUNCHED();
-  for (int pass = 0; pass < 4; ++pass) {
-    const int cur = pass & 1, nxt = cur ^ 1;
-    prk::sel_hist<<<(unsigned)rtiles, prk::SEL_NT, 0, s>>>(key[cur], n, 8 * pass, counts, rtiles);
-    PR_LAUNCHED();
-    prk::sel_scan_digit<<<prk::SEL_RADIX, prk::SEL_NT, 0, s>>>(counts, rtiles, total);
-    PR_LAUNCHED();
-    prk::sel_scatter<<<g_scatter, prk::SEL_NT, 0, s>>>(key[cur], val[cur], n, 8 * pass, counts,
-                                                       rtiles, total, key[nxt], val[nxt]);
-    PR_LAUNCHED();
-  }
-  // four passes: the sorted arrays are back in key[0], val[0]
-  prk::sel_label_prefix<<<g_tiles, prk::SEL_NT, 0, s>>>(val[0], nf, pre, tsum);
-  PR_LAUNCHED();
-  prk::sel_scan_tiles<<<1, 1024, 0, s>>>(tsum, ntiles, toff);
-  PR_LAUNCHED();
-  if (labels) {
-    prk::sel_metrics<<<g_tiles, prk::SEL_NT, 0, s>>>(key[0], val[0], pre, toff, nf, ntiles, proc,
-                                                    parc);
-    PR_LAUNCHED();
-  }
-  prk::sel_finish<<<1, prk::SEL_NT, 0, s>>>(key[0], pre, toff, nf, n, ntiles, q, labels ? 1 : 0,
-                                            proc, parc, res);
-  PR_LAUNCHED();
-#undef PR_LAUNCHED
+  const unsigned g_coarse =
+      (unsigned)std::min<int64_t>((n + 16 * prk::SB_NT - 1) / (16 * prk::SB_NT), 4 * c->num_sms);
+  PR_LAUNCH(prk::sel_coarse, g_coarse, prk::SB_NT, 0);
+  PR_LAUNCH(prk::sel_plan, 1, 1024, 0);
+  PR_LAUNCH(prk::sel_count, g.shares, prk::SB_NT, share_smem);
+  PR_LAUNCH(prk::sel_offsets, 1, 1024, 0);
+  PR_LAUNCH(prk::sel_scatter, g.shares, prk::SB_NT, share_smem);
+  if (n > prk::SB_HEAVY)
+    PR_LAUNCH(prk::sel_heavy,
+              (unsigned)std::min<int64_t>(n / prk::SB_CHUNK + 1, 3 * c->num_sms), prk::SB_NT,
+              prk::SB_BUCKET_SMEM);
+  PR_LAUNCH(prk::sel_bucket, (unsigned)std::min<int64_t>(g.nbcap, 3 * c->num_sms), prk::SB_NT,
+            prk::SB_BUCKET_SMEM);
+  PR_LAUNCH(prk::sel_finish, 1, prk::SB_NT, 0);
+#undef PR_LAUNCH
   g_launches.fetch_add((uint64_t)launches, std::memory_order_relaxed);
-  PR_CUDA(cudaMemcpyAsync(out, res, sizeof *out, cudaMemcpyDeviceToHost, s));
+  PR_CUDA(cudaMemcpyAsync(out, a.out, sizeof *out, cudaMemcpyDeviceToHost, s));
   PR_CUDA(cudaStreamSynchronize(s));
   return PR_OK;
 }

@@ -68,7 +68,7 @@ def check(g, s, y, q):
 
 @pytest.mark.parametrize("n", [1, 2, 31, 2047, 2048, 2049, 4095, 4096, 4097, 12289, 100003])
 def test_selective_matches_oracle_sizes(B, ctx, n):
-    # tile edges (2,048 items per tile) and ragged tails
+    # bucket targets and ragged tails
     s, y = make(n, seed=n, levels=97, nan_frac=0.03)
     # q * n + 1/2 lands on an integer for some of these: the rounding of q itself
     # must be the oracle's (double)
@@ -90,6 +90,41 @@ def test_selective_tie_structures(B, ctx, kind):
         s, y = make(n, 4, neg_zero=True)
     for q in (0.1, 0.5, 0.9):
         check(run(B, ctx, s, y, q), s, y, q)
+
+
+@pytest.mark.parametrize("kind", ["logits", "clusters", "neighbours", "extremes", "ties_63_64",
+                                  "long_ties", "one_bucket"])
+@pytest.mark.parametrize("n", [900, 5000, 70000, 300007])
+def test_selective_key_structures(B, ctx, n, kind):
+    """Keys spread over both signs and many exponents, piled up in a few buckets,
+    a few floats apart, at the ends of the float range; tie groups on both
+    sides of the closed form, also at the very top ranks; buckets that are
+    sorted, counted and counted with wide counts."""
+    g = np.random.Generator(np.random.PCG64(n))
+    if kind == "logits":
+        s = g.normal(0.0, 2.0, n) ** 3
+    elif kind == "clusters":
+        s = g.choice([-3.0, 1e-30, 0.7, 0.70001, 1e20], n) * (1.0 + 1e-5 * g.random(n))
+    elif kind == "neighbours":
+        s = (np.float32(0.75).view(np.uint32) + g.integers(0, 3000, n)).astype(np.uint32)
+        s = s.view(np.float32)
+    elif kind == "extremes":
+        s = g.choice(np.array([1e-45, -1e-45, 3.4028235e38, -3.4028235e38, 0.0, 1.1754944e-38],
+                              np.float32), n)
+    elif kind == "ties_63_64":
+        s = np.repeat(np.arange(n // 60 + 1) / (n // 60 + 1), g.integers(62, 67, n // 60 + 1))[:n]
+    elif kind == "long_ties":
+        s = np.where(g.random(n) < 0.9, 1.0, g.random(n))
+    else:
+        s = 0.5 + 2.0 ** -24 * g.integers(0, 1 << 14, n) + 0.0
+    s = s.astype(np.float32)
+    y = (g.random(n) < 0.3 + 0.4 * (s > np.median(s))).astype(np.uint8)
+    for q in (0.001, 0.4, 1.0):
+        check(run(B, ctx, s, y, q), s, y, q)
+    check(run(B, ctx, s, None, 0.4), s, None, 0.4)
+    off = torch.from_numpy(np.concatenate([[0.5], s]).astype(np.float32)).cuda()[1:]  # no vector loads
+    lab = torch.from_numpy(np.concatenate([[1], y]).astype(np.uint8)).cuda()[1:]
+    check(B.pr_selective_metrics(ctx, off, 0.4, labels=lab), s, y, 0.4)
 
 
 def test_selective_degenerate_pools(B, ctx):
