@@ -142,13 +142,15 @@ static pr_status launch_lm_fused(pr_ctx* c, const void* hidden, const void* weig
   cfg.blockDim = dim3(prk::LM_NT);
   cfg.dynamicSmemBytes = prk::LM_SMEM;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;  // a CTA pair lies along x
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   void* kargs[] = {&ma, &mb, &la};
   PR_CUDA(cudaLaunchKernelExC(&cfg, kern, kargs));
   *nparts_out = nparts;
@@ -156,16 +158,28 @@ static pr_status launch_lm_fused(pr_ctx* c, const void* hidden, const void* weig
 }
 
 // The merge launch: wpr warps per row, more for rows with many parts.
-static void launch_lm_merge(const prk::Args& a, pr_ctx* c, int64_t nparts, int mode,
-                            cudaStream_t s) {
-  const int wpr = nparts >= 64 ? 8 : nparts >= 32 ? 4 : 1;
+static pr_status launch_lm_merge(prk::Args a, pr_ctx* c, int64_t nparts, int mode,
+                                 cudaStream_t s) {
+  int wpr = nparts >= 64 ? 8 : nparts >= 32 ? 4 : 1, np = (int)nparts;
   const int64_t rows_per_cta = 8 / wpr;
-  const unsigned grid = (unsigned)((a.n_rows + rows_per_cta - 1) / rows_per_cta);
   const prk::LmPart* parts = static_cast<const prk::LmPart*>(c->lm_parts);
-  if (mode == prk::MODE_DECODE)
-    prk::lm_merge<prk::MODE_DECODE><<<grid, 256, 0, s>>>(a, parts, (int)nparts, wpr);
-  else
-    prk::lm_merge<prk::MODE_FEATURES><<<grid, 256, 0, s>>>(a, parts, (int)nparts, wpr);
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof cfg);
+  cfg.gridDim = dim3((unsigned)((a.n_rows + rows_per_cta - 1) / rows_per_cta));
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  void* args[] = {&a, &parts, &np, &wpr};
+  PR_CUDA(cudaLaunchKernelExC(
+      &cfg,
+      mode == prk::MODE_DECODE ? reinterpret_cast<const void*>(&prk::lm_merge<prk::MODE_DECODE>)
+                               : reinterpret_cast<const void*>(&prk::lm_merge<prk::MODE_FEATURES>),
+      args));
+  return PR_OK;
 }
 
 extern "C" {
@@ -205,8 +219,7 @@ pr_status pr_lmhead_features(pr_ctx* c, const void* hidden, const void* weight, 
   a.top2 = top2;
   a.row_flags = row_flags;
   a.ctx_flags = c->flags;
-  launch_lm_merge(a, c, nparts, prk::MODE_FEATURES, s);
-  PR_CUDA(cudaGetLastError());
+  if ((st = launch_lm_merge(a, c, nparts, prk::MODE_FEATURES, s)) != PR_OK) return st;
   g_launches.fetch_add(2, std::memory_order_relaxed);
   return timing_mark(c, s);
 }
@@ -253,8 +266,7 @@ pr_status pr_lmhead_decode_step(pr_ctx* c, const void* hidden, const void* weigh
   a.req_flags = slot_flags;
   a.agg = agg_out;
   a.ctx_flags = c->flags;
-  launch_lm_merge(a, c, nparts, prk::MODE_DECODE, s);
-  PR_CUDA(cudaGetLastError());
+  if ((st = launch_lm_merge(a, c, nparts, prk::MODE_DECODE, s)) != PR_OK) return st;
   g_launches.fetch_add(2, std::memory_order_relaxed);
   return timing_mark(c, s);
 }
