@@ -31,15 +31,15 @@
 //                for each of its keys, a light one by sorting it; then its groups
 //   sel_finish   the buckets' sums in bucket order
 // Results do not depend on the order in which items reach their buckets, so
-// they are deterministic.  2^24 scores (sigmoids of normals): 495 us; a radix
+// they are deterministic.  2^24 scores (sigmoids of normals): 468 us; a radix
 // sort of keys and labels with scans and a pass over the sorted items took 787, of
 // which the ranking of equal digits alone 425.  100,000 scores: 62 us against 130.
-// sel_bucket takes 270 of the 495, bound by the issue of the groups' arithmetic
+// sel_bucket takes 246 of the 468, bound by the issue of the groups' arithmetic
 // (two CTAs with twice the registers per SM instead of three: the same within 2%
 // either way, by the spread of the keys); sel_scatter 143, bound by its partly
 // filled 32-byte sectors (a share has some 70 bytes for each bucket).  Scores of
 // random bits in pools of a million, some 250 items in each of 4,095 coarse bins,
-// stay the weakest pool: 158 us against 153.
+// stay the weakest pool: 157 us against 153.
 #pragma once
 
 #include "pr_device.cuh"
@@ -115,8 +115,8 @@ __device__ __forceinline__ float sel_unkey(uint32_t k) {
 // the correction (about 46 correct bits).  Below 2^24 both integers are floats and
 // the remainder is exact; from there on they are split by bit masks into parts
 // that floats hold.
-__device__ __forceinline__ float2 sel_ratio(uint32_t C, uint32_t k) {
-  const float r = __frcp_rn((float)k), q = __fmul_rn((float)C, r);
+__device__ __forceinline__ float2 sel_ratio(uint32_t C, uint32_t k, float r) {  // r = 1 / k
+  const float q = __fmul_rn((float)C, r);
   float rem;
   if (k < 1u << 24) {
     rem = fmaf(-q, (float)k, (float)C);
@@ -126,6 +126,9 @@ __device__ __forceinline__ float2 sel_ratio(uint32_t C, uint32_t k) {
     rem = fmaf(-q, kh, ch) + fmaf(-q, kl, cl);
   }
   return make_float2(q, rem * r);
+}
+__device__ __forceinline__ float2 sel_ratio(uint32_t C, uint32_t k) {
+  return sel_ratio(C, k, __frcp_rn((float)k));
 }
 
 // body(key, label) for the scores i, i + 1, .. of [lo, hi) that this thread takes;
@@ -402,7 +405,7 @@ struct SelSums {
   __device__ __forceinline__ void group(bool on, uint32_t lo, uint32_t plo, uint32_t c, uint32_t p,
                                         uint32_t nf, uint32_t ptot, int lane) {
     const uint32_t above = nf - lo - c, cab = ptot - plo - p;
-    if (on) roc2 += (unsigned long long)p * (2ull * (lo - plo) + (c - p));
+    if (on) roc2 += (unsigned long long)p * (2u * (lo - plo) + (c - p));  // (below 2^32)
     // sum over j = 1 .. c of (cab + p j / c) / (above + j)
     const bool one = c == 1u, near = !one && (above >> 6 < c || c >> 23 != 0u);
     if (on && !near) {
@@ -413,21 +416,22 @@ struct SelSums {
       // and S4 = sums of d^2 and d^4, Cm the mean of the numerators, in fp32
       // while it is below 2^-23 of the sum (c / M < 2^-10), else in fp64
       const uint32_t D = one ? nf - lo : 2u * above + c + 1u;
-      const float2 t1 = sel_ratio(one ? ptot - plo : cab, D);
+      const float rD = __frcp_rn((float)D);
+      const float2 t1 = sel_ratio(one ? ptot - plo : cab, D, rD);
       const float cf = (float)c, c2 = one ? 1.f : 2.f * cf;  // exact (c < 2^23)
       const float x = __fmul_rn(t1.x, c2), xl = fmaf(t1.x, c2, -x) + t1.y * c2;
       add(x, xl);
       if (!one) {
-        const float2 t2 = sel_ratio(p, D);
+        const float2 t2 = sel_ratio(p, D, rD);
         const float c1 = cf + 1.f;
         const float y = __fmul_rn(t2.x, c1), yl = fmaf(t2.x, c1, -y) + t2.y * c1;
-        const float r = 2.f / (float)D, lead = x + y;  // c Cm / M
+        const float r = 2.f * rD, lead = x + y;  // c Cm / M
         float corr = 0.f;
         if (above >> 10 >= c) {
-          corr = cf * (cf * cf - 1.f) * (1.f / 12.f) * r * r * ((lead - (float)p) / cf);
+          corr = cf * (cf * cf - 1.f) * (1.f / 12.f) * r * r * __fdividef(lead - (float)p, cf);
         } else {
           const double cd = (double)c, rd = (double)r, im = rd * (2.0 - 0.5 * (double)D * rd);
-          const double im2 = im * im, cc = cd * cd, ri = (double)(1.f / cf);
+          const double im2 = im * im, cc = cd * cd, ri = (double)__frcp_rn(cf);
           const double w = (((double)x + (double)y) + ((double)xl + (double)yl)) - (double)p;
           ds += (cc - 1.0) * (1.0 / 12.0) * im2 * (1.0 + (3.0 * cc - 7.0) * 0.05 * im2) *
                 (w * (cd * ri * (2.0 - cd * ri)));
@@ -557,21 +561,33 @@ __global__ void __launch_bounds__(SB_NT, 3) sel_bucket(const SelArgs a) {
     // the groups of `vals` consecutive keys from key0 + first on, with a0 items and
     // q0 correct ones below; count(w, c, p) gives key w's.  The keys go by strips
     // of 32, a lane per key, to the warps in turn: long tie groups come in
-    // neighbouring keys, and all warps share them.  `small`: a strip's counts
-    // fit 16 bits.  Returns the totals.
+    // neighbouring keys, and all warps share them.  `small`: the counts are the
+    // 16-bit halves of sb_dyn's words.  Returns the totals.
     auto walk = [&](uint32_t first, uint32_t vals, uint32_t a0, uint32_t q0, bool small, auto count,
                     uint32_t& xall, uint32_t& yall) {
       const uint32_t strips = vals / 32u;  // at most one per thread
-      for (uint32_t s = warp; s < strips; s += SB_NT / 32) {
-        uint32_t c, p;
-        count(32u * s + lane, c, p);
-        c = __reduce_add_sync(FULL, c);
-        p = __reduce_add_sync(FULL, p);
-        if (lane == 0) {
-          strip[0][s] = c;
-          strip[1][s] = p;
+      if (small)  // four strips at a time, both counts in one sum
+        for (uint32_t s = 4u * warp; s < strips; s += SB_NT / 8) {
+          const uint4 u = *reinterpret_cast<const uint4*>(sb_dyn + 32u * s + 4u * lane);
+          uint32_t c = (u.x + u.y) + (u.z + u.w);
+#pragma unroll
+          for (int o = 1; o < 8; o <<= 1) c += __shfl_xor_sync(FULL, c, o);
+          if ((lane & 7) == 0) {
+            strip[0][s + (lane >> 3)] = c & 0xffffu;
+            strip[1][s + (lane >> 3)] = c >> 16;
+          }
         }
-      }
+      else
+        for (uint32_t s = warp; s < strips; s += SB_NT / 32) {
+          uint32_t c, p;
+          count(32u * s + lane, c, p);
+          c = __reduce_add_sync(FULL, c);
+          p = __reduce_add_sync(FULL, p);
+          if (lane == 0) {
+            strip[0][s] = c;
+            strip[1][s] = p;
+          }
+        }
       __syncthreads();
       uint32_t x = (uint32_t)tid < strips ? strip[0][tid] : 0u,
                y = (uint32_t)tid < strips ? strip[1][tid] : 0u;
