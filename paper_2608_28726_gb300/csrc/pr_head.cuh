@@ -647,6 +647,12 @@ __global__ void __launch_bounds__(HA_M, HA_CTAS_PER_SM) head_attn(const HeadArgs
 // columns; W_2: 64; W_qkv: 192) and 384 (W_o: 64); H1 kept at 448-511 for
 // the second residual.  One elected thread issues the MMAs; every wait is
 // bounded.
+// LAST and QKV keep their weights, so with more tiles than SMs each CTA takes several
+// tiles in turn (QKV loads the next one during its GEMM and stages its output
+// behind the weights, half a tile at a time): staging the weights was a third of a
+// tile's time.  1,000 tiles: QKV 62 -> 43 us, LAST 94 -> 65; two layers over 1,024
+// lognormal requests of 8 to 1,024 rows 1,065 -> 991 us.  MID's weights do not fit
+// side by side.
 constexpr int HT_M = 128;                           // rows per tile = TMEM lanes
 constexpr int HT_NT = 2 * HT_M;                     // threads: two per row (column halves)
 constexpr uint32_t HT_TMEM_COLS = 512;
@@ -671,6 +677,8 @@ constexpr int HT_X = HT_VEC + HT_VEC_N * 4;
 constexpr int HT_LDQ = 3 * HD + 4;
 constexpr int HT_Q = 0;
 static_assert(HT_Q + HT_M * HT_LDQ * 4 <= HT_VEC, "the QKV tile fits over the weights");
+constexpr int HT_Q2 = HT_WQKV + 2 * 3 * HD * HD * 4;  // or half of it behind W_qkv (mode QKV)
+static_assert(HT_Q2 + HT_M / 2 * HT_LDQ * 4 <= HT_VEC, "half a QKV tile fits behind W_qkv");
 constexpr int HT_XCH = HT_X + HT_M * HT_LDX * 4;    // row sums of the two halves [2][2][128]
 constexpr int HT_BAR = HT_XCH + 4 * HT_M * 4;       // mbarrier: MMA completion
 constexpr int HT_TSLOT = HT_BAR + 8;
@@ -821,7 +829,7 @@ __global__ void __launch_bounds__(HT_NT, 1) head_rows(const HeadArgs a) {
   float* xch = reinterpret_cast<float*>(ht_sm + HT_XCH);
   // this thread's half of its row in the staging tile (8 pieces of 16 bytes)
   float4* xrow = reinterpret_cast<float4*>(ht_sm + HT_X) + r * (HT_LDX / 4) + 8 * hf;
-  const int64_t row0 = (int64_t)blockIdx.x * HT_M;
+  int64_t row0 = (int64_t)blockIdx.x * HT_M;
 
   // the weights and vectors are inputs of the call: staged before the wait,
   // their copies in flight while the CTA takes its TMEM
@@ -890,11 +898,6 @@ __global__ void __launch_bounds__(HT_NT, 1) head_rows(const HeadArgs a) {
   pdl_trigger();
   pdl_wait();
 
-  // the tile's input rows (the attention output over Q for MID / LAST, H for
-  // QKV), then this thread's half row as the first GEMM's A operand
-  ht_load_rows(ht_sm, a.scratch, row0, a.n_rows, MODE == HR_QKV ? 0 : HD);
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  __syncthreads();
   auto read_half = [&](float (&x)[32]) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -905,12 +908,6 @@ __global__ void __launch_bounds__(HT_NT, 1) head_rows(const HeadArgs a) {
       x[4 * j + 3] = v.w;
     }
   };
-  {
-    float x[32];
-    read_half(x);
-    ht_put_split(tq + HT_A_HI + c32, tq + HT_A_LO + c32, x);
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-  }
   uint32_t phase = 0;
   bool ok = true;
   // all threads' operands written -> one thread issues the MMAs -> every
@@ -932,112 +929,143 @@ __global__ void __launch_bounds__(HT_NT, 1) head_rows(const HeadArgs a) {
   };
   auto nothing = [] {};
 
-  if (MODE != HR_QKV) {
-    float h[32];
-    // O = A W_o^T, while the residual H comes into the staging tile
-    ok = mma_step(
-        [&] { ht_gemm<HD, HD>(tmem + HT_DO, tmem + HT_A_HI, tmem + HT_A_LO, sb + HT_WO); },
-        [&] { ht_load_rows(ht_sm, a.scratch, row0, a.n_rows, 0); });
+  // the tile's input rows (the attention output over Q for MID / LAST, H for
+  // QKV), then this thread's half row as the first GEMM's A operand
+  const int64_t step = (int64_t)gridDim.x * HT_M;
+  ht_load_rows(ht_sm, a.scratch, row0, a.n_rows, MODE == HR_QKV ? 0 : HD);
+  for (;;) {
+    const bool more = MODE != HR_MID && row0 + step < a.n_rows;  // another tile for this CTA
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    if (ok) {
-      // H1 = LN1(H + O + b_o): kept in TMEM for the second residual and split
-      // as the A operand of W_1
-      read_half(h);
-      {
-        float d[32];
-        ha_ld32(tq + HT_DO + c32, d);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) h[j] += d[j] + sV[HV_BO + c32 + j];
-      }
-      ht_layer_norm(h, sV + HV_G1, sV + HV_BE1, xch, r, hf);
-      ha_st32(tq + HT_H1 + c32, h);
-      ht_put_split(tq + HT_A_HI + c32, tq + HT_A_LO + c32, h);
+    {
+      float x[32];
+      read_half(x);
+      ht_put_split(tq + HT_A_HI + c32, tq + HT_A_LO + c32, x);
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-      ok = mma_step(
-          [&] { ht_gemm<HFF, HD>(tmem + HT_D, tmem + HT_A_HI, tmem + HT_A_LO, sb + HT_W1); },
-          nothing);
     }
-    if (ok) {
-      if (MODE == HR_MID) {  // W_o and W_1 are done: W_qkv over them
+    if (MODE != HR_QKV) {
+      float h[32];
+      // O = A W_o^T, while the residual H comes into the staging tile
+      ok = mma_step(
+          [&] { ht_gemm<HD, HD>(tmem + HT_DO, tmem + HT_A_HI, tmem + HT_A_LO, sb + HT_WO); },
+          [&] { ht_load_rows(ht_sm, a.scratch, row0, a.n_rows, 0); });
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncthreads();
+      if (ok) {
+        // H1 = LN1(H + O + b_o): kept in TMEM for the second residual and split
+        // as the A operand of W_1
+        read_half(h);
+        {
+          float d[32];
+          ha_ld32(tq + HT_DO + c32, d);
 #pragma unroll
-        for (int i = 0; i < WQ_IT; ++i) {
-          float4 hh, ll;
-          ha_split(wq_hold[i], hh, ll);
-          reinterpret_cast<float4*>(ht_sm + HT_WQKV)[tid + i * HT_NT] = hh;
-          reinterpret_cast<float4*>(ht_sm + HT_WQKV + 3 * HD * HD * 4)[tid + i * HT_NT] = ll;
+          for (int j = 0; j < 32; ++j) h[j] += d[j] + sV[HV_BO + c32 + j];
         }
-      }
-      // F = ReLU(H1 W_1^T + b_1), split as the A operand of W_2 (64 columns a half)
-#pragma unroll
-      for (int c = 0; c < HFF / 64; ++c) {
-        const uint32_t col = 64u * hf + 32u * c;
-        float d[32];
-        ha_ld32(tq + HT_D + col, d);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) d[j] = fmaxf(d[j] + sV[HV_B1 + col + j], 0.f);
-        ht_put_split(tq + HT_F_HI + col, tq + HT_F_LO + col, d);
-      }
-      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-      ok = mma_step(
-          [&] { ht_gemm<HD, HFF>(tmem + HT_D, tmem + HT_F_HI, tmem + HT_F_LO, sb + HT_W2); },
-          nothing);
-    }
-    if (ok) {
-      // H2 = LN2(H1 + F W_2^T + b_2) -> H, through the staging tile
-      {
-        float d[32], rr[32];
-        ha_ld32(tq + HT_D + c32, d);
-        ha_ld32(tq + HT_H1 + c32, rr);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) h[j] = rr[j] + (d[j] + sV[HV_B2 + c32 + j]);
-      }
-      ht_layer_norm(h, sV + HV_G2, sV + HV_BE2, xch, r, hf);
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        xrow[j] = make_float4(h[4 * j], h[4 * j + 1], h[4 * j + 2], h[4 * j + 3]);
-      if (MODE == HR_MID) {
+        ht_layer_norm(h, sV + HV_G1, sV + HV_BE1, xch, r, hf);
+        ha_st32(tq + HT_H1 + c32, h);
         ht_put_split(tq + HT_A_HI + c32, tq + HT_A_LO + c32, h);
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        ok = mma_step(
+            [&] { ht_gemm<HFF, HD>(tmem + HT_D, tmem + HT_A_HI, tmem + HT_A_LO, sb + HT_W1); },
+            nothing);
       }
-      __syncthreads();
-      ht_store_rows(ht_sm, a.scratch, row0, a.n_rows, 0);
-    }
-  }
-  if (MODE != HR_LAST && ok) {
-    // QKV = H W_qkv^T + b_qkv -> scratch columns [64, 256), through a
-    // staging tile over the weights (their MMAs are done); 96 columns a half
-    ok = mma_step(
-        [&] { ht_gemm<3 * HD, HD>(tmem + HT_D, tmem + HT_A_HI, tmem + HT_A_LO, sb + HT_WQKV); },
-        nothing);
-    if (ok) {
-      float4* qrow = reinterpret_cast<float4*>(ht_sm + HT_Q) + r * (HT_LDQ / 4);
+      if (ok) {
+        if (MODE == HR_MID) {  // W_o and W_1 are done: W_qkv over them
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const uint32_t col = 96u * hf + 32u * c;
-        float d[32];
-        ha_ld32(tq + HT_D + col, d);
+          for (int i = 0; i < WQ_IT; ++i) {
+            float4 hh, ll;
+            ha_split(wq_hold[i], hh, ll);
+            reinterpret_cast<float4*>(ht_sm + HT_WQKV)[tid + i * HT_NT] = hh;
+            reinterpret_cast<float4*>(ht_sm + HT_WQKV + 3 * HD * HD * 4)[tid + i * HT_NT] = ll;
+          }
+        }
+        // F = ReLU(H1 W_1^T + b_1), split as the A operand of W_2 (64 columns a half)
+#pragma unroll
+        for (int c = 0; c < HFF / 64; ++c) {
+          const uint32_t col = 64u * hf + 32u * c;
+          float d[32];
+          ha_ld32(tq + HT_D + col, d);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) d[j] = fmaxf(d[j] + sV[HV_B1 + col + j], 0.f);
+          ht_put_split(tq + HT_F_HI + col, tq + HT_F_LO + col, d);
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        ok = mma_step(
+            [&] { ht_gemm<HD, HFF>(tmem + HT_D, tmem + HT_F_HI, tmem + HT_F_LO, sb + HT_W2); },
+            nothing);
+      }
+      if (ok) {
+        // H2 = LN2(H1 + F W_2^T + b_2) -> H, through the staging tile
+        {
+          float d[32], rr[32];
+          ha_ld32(tq + HT_D + c32, d);
+          ha_ld32(tq + HT_H1 + c32, rr);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) h[j] = rr[j] + (d[j] + sV[HV_B2 + c32 + j]);
+        }
+        ht_layer_norm(h, sV + HV_G2, sV + HV_BE2, xch, r, hf);
 #pragma unroll
         for (int j = 0; j < 8; ++j)
-          qrow[col / 4 + j] = make_float4(d[4 * j] + sV[HV_BQKV + col + 4 * j],
-                                          d[4 * j + 1] + sV[HV_BQKV + col + 4 * j + 1],
-                                          d[4 * j + 2] + sV[HV_BQKV + col + 4 * j + 2],
-                                          d[4 * j + 3] + sV[HV_BQKV + col + 4 * j + 3]);
+          xrow[j] = make_float4(h[4 * j], h[4 * j + 1], h[4 * j + 2], h[4 * j + 3]);
+        if (MODE == HR_MID) {
+          ht_put_split(tq + HT_A_HI + c32, tq + HT_A_LO + c32, h);
+          asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        }
+        __syncthreads();
+        ht_store_rows(ht_sm, a.scratch, row0, a.n_rows, 0);
       }
-      __syncthreads();
+    }
+    if (MODE != HR_LAST && ok) {
+      // QKV = H W_qkv^T + b_qkv -> scratch columns [64, 256), through a
+      // staging tile over the weights (their MMAs are done); 96 columns a half
+      ok = mma_step(
+          [&] { ht_gemm<3 * HD, HD>(tmem + HT_D, tmem + HT_A_HI, tmem + HT_A_LO, sb + HT_WQKV); },
+          [&] {  // (its first barrier: every thread has read the staging tile)
+            if (more) ht_load_rows(ht_sm, a.scratch, row0 + step, a.n_rows, 0);
+          });
+      // the weights stay for another tile: 64 rows at a time go through the room
+      // behind them
+      const int passes = more ? 2 : 1, rows = HT_M / passes;
+      for (int p = 0; p < passes && ok; ++p) {
+        uint8_t* stage = ht_sm + (more ? HT_Q2 : HT_Q);
+        if (p) __syncthreads();
+        float4* qrow = reinterpret_cast<float4*>(stage) + (r - p * rows) * (HT_LDQ / 4);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          if (r / rows != p) break;  // warp-uniform
+          const uint32_t col = 96u * hf + 32u * c;
+          float d[32];
+          ha_ld32(tq + HT_D + col, d);
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            qrow[col / 4 + j] = make_float4(d[4 * j] + sV[HV_BQKV + col + 4 * j],
+                                            d[4 * j + 1] + sV[HV_BQKV + col + 4 * j + 1],
+                                            d[4 * j + 2] + sV[HV_BQKV + col + 4 * j + 2],
+                                            d[4 * j + 3] + sV[HV_BQKV + col + 4 * j + 3]);
+        }
+        __syncthreads();
 #pragma unroll 4
-      for (int i = 0; i < HT_M * (3 * HD / 4) / HT_NT; ++i) {  // 48 pieces of 16 bytes a row
-        const int f = tid + i * HT_NT;
-        const int rw = f / (3 * HD / 4), q = f - rw * (3 * HD / 4);
-        if (row0 + rw < a.n_rows)
-          *reinterpret_cast<float4*>(a.scratch + (row0 + rw) * HSCR + HD + 4 * q) =
-              reinterpret_cast<const float4*>(ht_sm + HT_Q)[rw * (HT_LDQ / 4) + q];
+        for (int i = 0; i < rows * (3 * HD / 4) / HT_NT; ++i) {  // 48 pieces of 16 bytes a row
+          const int f = tid + i * HT_NT;
+          const int rw = f / (3 * HD / 4), q = f - rw * (3 * HD / 4);
+          const int64_t row = row0 + p * rows + rw;
+          if (row < a.n_rows)
+            *reinterpret_cast<float4*>(a.scratch + row * HSCR + HD + 4 * q) =
+                reinterpret_cast<const float4*>(stage)[rw * (HT_LDQ / 4) + q];
+        }
       }
+    }
+    if (!ok || !more) break;
+    row0 += step;
+    if (MODE == HR_LAST) {  // (QKV: already on their way)
+      __syncthreads();      // the staging tile has been stored
+      ht_load_rows(ht_sm, a.scratch, row0, a.n_rows, HD);
     }
   }
   if (!ok) {
     if (tid == 0) atomicOr(a.ctx_flags, HA_ERR_TIMEOUT);
     ha_wait(bar, phase);  // the MMAs still pending, bounded as well
+    asm volatile("cp.async.wait_all;" ::: "memory");
   }
   ha_fence_before();
   __syncthreads();

@@ -107,12 +107,14 @@ pr_status pr_head_score(pr_ctx* c, const float* feat, const uint32_t* row_flags,
                    dim3((unsigned)n_req, prk::HES), blk, 0, s, a);
   if (st != PR_OK) return st;
   if (n_rows > 0) {
-    // one CTA per 128-row tile (the row kernels hold all 512 TMEM columns of an SM)
+    // one CTA per 128-row tile (the row kernels hold all 512 TMEM columns of an
+    // SM); those that keep their weights in shared memory take several tiles
     const unsigned ntiles = (unsigned)((n_rows + prk::HT_M - 1) / prk::HT_M);
+    const unsigned nkeep = std::min(ntiles, (unsigned)c->num_sms);
     const dim3 rblk(prk::HT_NT);
     a.lcur = nullptr;
     a.lnext = layer(0);
-    st = launch_head(c, reinterpret_cast<const void*>(&prk::head_rows<prk::HR_QKV>), dim3(ntiles),
+    st = launch_head(c, reinterpret_cast<const void*>(&prk::head_rows<prk::HR_QKV>), dim3(nkeep),
                      rblk, prk::HT_SMEM, s, a);
     if (st != PR_OK) return st;
     // CTAs per (request, head): one per query block of a request of the mean
@@ -134,7 +136,7 @@ pr_status pr_head_score(pr_ctx* c, const float* feat, const uint32_t* row_flags,
       a.lnext = last ? nullptr : layer(l + 1);
       const void* k = last ? reinterpret_cast<const void*>(&prk::head_rows<prk::HR_LAST>)
                            : reinterpret_cast<const void*>(&prk::head_rows<prk::HR_MID>);
-      st = launch_head(c, k, dim3(ntiles), rblk, prk::HT_SMEM, s, a);
+      st = launch_head(c, k, dim3(last ? nkeep : ntiles), rblk, prk::HT_SMEM, s, a);
       if (st != PR_OK) return st;
     }
   }

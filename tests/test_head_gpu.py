@@ -100,6 +100,23 @@ def test_head_more_row_tiles_than_sms(B, ctx):
     check(B, ctx, lengths, 2, seed=4401)
 
 
+@pytest.mark.parametrize("tiles,extra", [(1.0, -1), (1.0, 0), (1.0, 1), (2.0, 5), (2.5, 64)])
+def test_head_row_tiles_taken_in_turn(B, ctx, tiles, extra):
+    """Row kernels whose CTAs keep their weights for several 128-row tiles: the
+    same requests in batches of one tile per CTA give the same bits."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = int(tiles * sms) * 128 + extra
+    lengths = [61] * (n // 61) + ([n % 61] if n % 61 else [])
+    feat, offsets = workloads.head_features(lengths, 4300)
+    w = workloads.head_weights(2, seed=3003)
+    got = run_head(B, ctx, feat, offsets, w, 2)[0]
+    per = 9000 // 61
+    for r0 in range(0, len(lengths), per):
+        o = offsets[r0:r0 + per + 1]
+        want = run_head(B, ctx, feat[o[0]:o[-1]], o - o[0], w, 2)[0]
+        assert (got[r0:r0 + per].view(np.uint32) == want.view(np.uint32)).all()
+
+
 def test_head_thresholds(B, ctx):
     g = np.random.Generator(np.random.PCG64(7))
     lengths = g.integers(1, 80, size=40, endpoint=True)
