@@ -160,8 +160,9 @@ pr_status pr_last_error(pr_ctx* ctx, uint32_t* flags);
 /*
  * Per-kernel device times (milliseconds, launch order) of the last call made
  * with PR_OPT_TIMING = 1: for pr_head_score the embedding, the first QKV
- * projection, then per layer the attention and the row-local block, then the
- * pool; for pr_selective_metrics the histogram of leading bits, the plan of
+ * projection, then per layer the attention and the row-local block (followed
+ * by the next layer's projection on its own when the batch has more 128-row tiles
+ * than the device has SMs), then the pool; for pr_selective_metrics the histogram of leading bits, the plan of
  * the buckets, their counts, their offsets, the scatter into them, the counts of
  * crowded ones (above 65,535 scores), the buckets' groups and the final
  * reduction.  Waits for the call's last event.  Writes min(count, cap) values to

@@ -108,7 +108,7 @@ pr_status pr_head_score(pr_ctx* c, const float* feat, const uint32_t* row_flags,
   if (st != PR_OK) return st;
   if (n_rows > 0) {
     // one CTA per 128-row tile (the row kernels hold all 512 TMEM columns of an
-    // SM); those that keep their weights in shared memory take several tiles
+    // SM); with more tiles than SMs a CTA keeps its weights for several tiles
     const unsigned ntiles = (unsigned)((n_rows + prk::HT_M - 1) / prk::HT_M);
     const unsigned nkeep = std::min(ntiles, (unsigned)c->num_sms);
     const dim3 rblk(prk::HT_NT);
@@ -134,9 +134,18 @@ pr_status pr_head_score(pr_ctx* c, const float* feat, const uint32_t* row_flags,
       a.lcur = layer(l);
       const bool last = l + 1 == n_layers;
       a.lnext = last ? nullptr : layer(l + 1);
-      const void* k = last ? reinterpret_cast<const void*>(&prk::head_rows<prk::HR_LAST>)
-                           : reinterpret_cast<const void*>(&prk::head_rows<prk::HR_MID>);
-      st = launch_head(c, k, dim3(last ? nkeep : ntiles), rblk, prk::HT_SMEM, s, a);
+      // with more tiles than SMs the middle layers' projection goes apart: two
+      // kernels that keep their weights instead of one that stages both sets for
+      // every tile (153 tiles: 25 + 18 us against 37; 310: 31 + 23 against 55;
+      // 1,000: 64 + 43 against 130.  Up to one tile per SM one kernel is faster,
+      // 152 tiles: 25 against 20 + 14)
+      const bool alone = last || ntiles > nkeep;
+      const void* k = alone ? reinterpret_cast<const void*>(&prk::head_rows<prk::HR_LAST>)
+                            : reinterpret_cast<const void*>(&prk::head_rows<prk::HR_MID>);
+      st = launch_head(c, k, dim3(nkeep), rblk, prk::HT_SMEM, s, a);
+      if (st == PR_OK && alone && !last)
+        st = launch_head(c, reinterpret_cast<const void*>(&prk::head_rows<prk::HR_QKV>),
+                         dim3(nkeep), rblk, prk::HT_SMEM, s, a);
       if (st != PR_OK) return st;
     }
   }
