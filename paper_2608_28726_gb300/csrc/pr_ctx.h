@@ -9,7 +9,7 @@
 
 #include "pro_router.h"
 
-#define PR_MAX_TIMED 24  // kernels one call can time under PR_OPT_TIMING
+#define PR_MAX_TIMED 32  // kernels one call can time under PR_OPT_TIMING
 
 struct pr_ctx {
   int device = 0;
