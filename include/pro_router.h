@@ -30,7 +30,7 @@
  *   - Logits are row-major [n_rows][row_stride] elements, bf16 or fp32;
  *     only the first `vocab` entries of a row count.  Any element alignment is
  *     accepted; rows whose start is 16-byte aligned (base pointer and
- *     row_stride * element size multiples of 16) take the vector path.
+ *     row_stride * element size multiples of 16) are read fastest.
  *   - Token ids are int32 (V < 2^31); request offsets are int64 CSR: request r
  *     owns rows [offsets[r], offsets[r+1]).
  *   - Features are written as PR_NFEAT floats per row, in the order of the
@@ -108,7 +108,7 @@ typedef enum { PR_DTYPE_F32 = 0, PR_DTYPE_BF16 = 1 } pr_dtype;
 #define PR_OPT_OVERLAP 3     /* 1: a call may start while the previous kernel on its stream is
                                 still running (programmatic dependent launch): it reads its
                                 inputs at once and waits for that kernel before writing
-                                anything.  Only for callers whose inputs are complete before
+                                anything (0: it waits before reading as well).  Only for callers whose inputs are complete before
                                 the preceding kernel starts (e.g. back-to-back verifier calls
                                 on resident logits).  Default 0. */
 #define PR_OPT_TIMING 4      /* 1: the calls after the verifier's (pr_head_score,
