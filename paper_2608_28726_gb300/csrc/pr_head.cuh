@@ -406,6 +406,10 @@ __global__ void __launch_bounds__(HA_M, HA_CTAS_PER_SM) head_attn(const HeadArgs
   const int nqb = (T + HA_M - 1) / HA_M;
   if ((int)blockIdx.z >= nqb) {
     pdl_trigger();
+    // one CTA of the grid always waits: a grid whose requests are all empty or
+    // rejected must not end before the row kernel that it follows, on whose end
+    // everything after it relies
+    if ((blockIdx.x | blockIdx.y | blockIdx.z) == 0) pdl_wait();
     return;
   }
   const int hh = blockIdx.y;

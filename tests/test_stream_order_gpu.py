@@ -82,3 +82,35 @@ def test_inputs_written_just_before_a_call(B, n, V):
         torch.cuda.synchronize()
         assert same()
     B.pr_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("layers", [1, 2])
+def test_head_call_of_rejected_requests_before_a_good_one(B, layers):
+    """A head call whose requests are all empty or inconsistent leaves its attention
+    grid without work; the calls behind it still wait for its row kernels, which
+    write the shared scratch."""
+    lengths = [200, 1, 130, 77, 300]
+    feat_np, off_np = W.head_features(lengths, 11)
+    feat, off = torch.from_numpy(feat_np).cuda(), torch.from_numpy(off_np).cuda()
+    n, r = int(off_np[-1]), len(lengths)
+    hw = torch.from_numpy(W.head_weights(layers)).cuda()
+    empty = torch.full((r + 1,), n, dtype=torch.int64, device="cuda")
+    wrong = torch.arange(r + 1, dtype=torch.int64, device="cuda") + n + 1
+    ctx = B.pr_ctx_create(0, n, r)
+    out = [torch.zeros(r, dtype=d, device="cuda") for d in (torch.float32, torch.uint8, torch.int32)]
+    junk = [t.clone() for t in out]
+    B.pr_head_score(ctx, feat, off, hw, layers, 0.5, None, *out)
+    torch.cuda.synchronize()
+    ref = [t.clone() for t in out]
+
+    def calls():
+        B.pr_head_score(ctx, feat, off, hw, layers, 0.5, None, *out)
+        B.pr_head_score(ctx, -feat, empty, hw, layers, 0.5, None, *junk)
+        B.pr_head_score(ctx, feat, wrong, hw, layers, 0.5, None, *junk)
+        B.pr_head_score(ctx, feat, off, hw, layers, 0.5, None, *out)
+
+    for _ in range(20):
+        calls()
+        assert all(torch.equal(a, b) for a, b in zip(out, ref))
+    assert (junk[2] == B.PR_FLAG_BAD_OFFSETS).all()
+    B.pr_ctx_destroy(ctx)
