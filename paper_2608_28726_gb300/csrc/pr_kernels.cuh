@@ -693,8 +693,9 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T, ALIGNED>()) verify_rows
           for (int k = 0; k < UNR; ++k) dst[k] = tile_pos(tid, k) < rem ? load(k) : NEG;
         }
       } else {
-        const bool rim = (row == 0 && rank == 0 && t == 0) ||
-                         (row == a.n_rows - 1 && rank == C - 1 && t == ntiles - 1);
+        // (a row of fewer groups than CTAs has its first group in a later CTA)
+        const bool rim = (row == 0 && g0 + nb == 0) ||
+                         (row == a.n_rows - 1 && g1 == geo.gfull && t == ntiles - 1);
         ld_tile_off_grid(rowt, g0 + nb, g1, rim, tid, dst, ext, NEG);
       }
     };

@@ -161,6 +161,31 @@ def test_row_alignment_does_not_change_the_bits(ctx, dtype, V, split):
     _set(ctx)
 
 
+@pytest.mark.parametrize("n", [12, 300])
+@pytest.mark.parametrize("dtype,V", [(torch.bfloat16, 9), (torch.bfloat16, 21),
+                                     (torch.bfloat16, 63), (torch.bfloat16, 40009),
+                                     (torch.float32, 7), (torch.float32, 31),
+                                     (torch.float32, 20003)])
+def test_split_rows_off_the_grid(ctx, dtype, V, n):
+    """The split kernel off the 16-byte grid, against the oracle and the same rows
+    on the grid: clusters of 8 (12 rows), among them rows of fewer groups than
+    CTAs, whose first group is not the first CTA's, and one CTA per row (300)."""
+    _set(ctx)
+    step = 16 // dtype.itemsize
+    src, ch = random_rows(n, V, dtype, seed=V + n)
+    grid = torch.zeros(n, (V + step - 1) // step * step, dtype=dtype, device="cuda")
+    grid[:, :V] = src
+    ref = B.pr_token_features(ctx, grid, ch, topk=20, vocab=V)
+    of, oi, ofl = _oracle_rows(src[::11], ch[::11])
+    _check_features(ref[0][::11], ref[1][::11], ref[2][::11], of, oi, ofl, "on the grid")
+    for shift in range(1, step):
+        flat = torch.zeros(shift + n * V, dtype=dtype, device="cuda")
+        x = flat[shift:].view(n, V)
+        x.copy_(src)
+        for a, b in zip(B.pr_token_features(ctx, x, ch, topk=20), ref):
+            assert torch.equal(a, b), shift
+
+
 def test_features_vocab_narrower_than_stride(ctx):
     x, ch = random_rows(10, 5000, torch.float32, seed=3)
     V = 4321
