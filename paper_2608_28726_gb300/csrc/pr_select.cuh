@@ -247,7 +247,7 @@ __device__ __forceinline__ uint32_t sel_bucket_of(uint32_t key, const uint32_t* 
 
 // share s: items and correct items per bucket, added to the buckets' totals
 __global__ void __launch_bounds__(SB_NT, 2) sel_count(const SelArgs a) {
-  extern __shared__ uint32_t sb_dyn[];  // [SB_BINS] plan, [buckets] counts
+  extern __shared__ __align__(16) uint32_t sb_dyn[];  // [SB_BINS] plan, [buckets] counts
   uint32_t *plan = sb_dyn, *cnt = sb_dyn + SB_BINS;
   pdl_enter(false);
   const uint32_t nb = a.info[0];
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(1024) sel_offsets(const SelArgs a) {
 }
 
 __global__ void __launch_bounds__(SB_NT, 2) sel_scatter(const SelArgs a) {
-  extern __shared__ uint32_t sb_dyn[];  // [SB_BINS] plan, [buckets] next places
+  extern __shared__ __align__(16) uint32_t sb_dyn[];  // [SB_BINS] plan, [buckets] next places
   uint32_t *plan = sb_dyn, *pos = sb_dyn + SB_BINS;
   pdl_enter(false);
   const uint32_t nb = a.info[0];
@@ -346,7 +346,7 @@ constexpr size_t SB_BUCKET_SMEM = SB_WORDS * sizeof(uint32_t);
 // The heavy buckets (scores piled up on few keys, as those of a confident
 // scorer just below 1): their items counted chunk by chunk on all SMs
 __global__ void __launch_bounds__(SB_NT, 3) sel_heavy(const SelArgs a) {
-  extern __shared__ uint32_t sb_dyn[];
+  extern __shared__ __align__(16) uint32_t sb_dyn[];
   pdl_enter(false);
   const uint32_t chunks = a.info[5];
   for (uint32_t q = blockIdx.x; q < chunks; q += gridDim.x) {
@@ -479,7 +479,7 @@ static_assert(1 << SB_VBITS == 32 * SB_NT, "a strip of 32 keys per thread");
 static_assert(SB_RADIX == 8 * SB_NT && SB_LIGHT == 8 * SB_NT, "eight per thread");
 
 __global__ void __launch_bounds__(SB_NT, 3) sel_bucket(const SelArgs a) {
-  extern __shared__ uint32_t sb_dyn[];
+  extern __shared__ __align__(16) uint32_t sb_dyn[];
   __shared__ uint32_t ws[2][SB_NT / 32], next, ranges[4], strip[2][SB_NT];
   __shared__ double sd[SB_NT / 32];
   __shared__ unsigned long long su[SB_NT / 32];
