@@ -110,7 +110,7 @@ __device__ __forceinline__ float ex2(float x) {
 
 __device__ __forceinline__ uint4 ld_stream(const void* p) {
   uint4 r;
-  asm volatile("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"
                : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
                : "l"(p));
   return r;
@@ -424,7 +424,11 @@ struct WarpTopK {
 // holds as with a plain launch; only the launch's own latency is hidden (16
 // decode steps of 256 rows 347 us without, 306 us with it).  It lets its own
 // dependents be set up after that wait, so that whatever they read early is
-// older than the previous kernel too.
+// older than the previous kernel too.  What a caller's kernel may have written
+// just before the call (logits, records, offsets, weights of the linear scorers)
+// is never read through the read-only path (ld.global.nc, __ldg, __restrict__):
+// that path is for memory that nothing writes while the kernel is resident, and a
+// kernel is resident before its wait.
 // With PR_OPT_OVERLAP (`early`) the order is loosened: every CTA allows its
 // dependents at once, reads only its inputs before pdl_wait(), and waits there
 // before its first global write and before any read of context state

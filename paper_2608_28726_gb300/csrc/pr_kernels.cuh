@@ -16,7 +16,7 @@ namespace prk {
 // from DRAM instead of a 256-byte block.
 __device__ __forceinline__ uint4 ld_reread(const void* p) {
   uint4 r;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
                : "l"(p));
   return r;
@@ -109,7 +109,7 @@ __device__ __forceinline__ Pooled pool_rows(const float* feat, const uint32_t* f
   p.agg[10] = (float)(T + 1) / (float)(2 * T);  // mean of t/T over t = 1..T
   float z = b;
 #pragma unroll
-  for (int j = 0; j < NAGG; ++j) z = fmaf(__ldg(w + j), p.agg[j], z);
+  for (int j = 0; j < NAGG; ++j) z = fmaf(w[j], p.agg[j], z);
   p.score = 1.f / (1.f + expf(-z));
   p.ship = (z >= zthr) ? 1 : 0;
   return p;
@@ -150,14 +150,14 @@ __device__ __forceinline__ int32_t find_request(const int64_t* off, int32_t n_re
   while (hi > lo) {
     const int64_t step = (hi - lo + 32) / 32;
     const int64_t pos = lo + (int64_t)lane * step;
-    const bool ok = pos <= hi && __ldg(off + pos) <= gr;
+    const bool ok = pos <= hi && off[pos] <= gr;
     const unsigned bal = __ballot_sync(FULL, ok);
     if (bal == 0) return -1;
     const int L = 31 - __clz(bal);
     lo = lo + (int64_t)L * step;
     hi = min(hi, lo + step - 1);
   }
-  const int64_t a = __ldg(off + lo), c = __ldg(off + lo + 1);
+  const int64_t a = off[lo], c = off[lo + 1];
   return (a <= gr && gr < c) ? (int32_t)lo : -1;
 }
 
@@ -285,15 +285,15 @@ __device__ __forceinline__ int32_t tile_pos(int tid, int k) {
 // with every group loaded by its elements.
 __device__ __forceinline__ uint32_t ld_l1_32(const char* p) {
   uint32_t r;
-  asm volatile("ld.global.nc.L2::256B.u32 %0, [%1];" : "=r"(r) : "l"(p));
+  asm volatile("ld.global.L2::256B.u32 %0, [%1];" : "=r"(r) : "l"(p));
   return r;
 }
 __device__ __forceinline__ void ld_l1_64(const char* p, uint32_t& x, uint32_t& y) {
-  asm volatile("ld.global.nc.L2::256B.v2.u32 {%0,%1}, [%2];" : "=r"(x), "=r"(y) : "l"(p));
+  asm volatile("ld.global.L2::256B.v2.u32 {%0,%1}, [%2];" : "=r"(x), "=r"(y) : "l"(p));
 }
 __device__ __forceinline__ void ld_l1_128(const char* p, uint32_t& x, uint32_t& y, uint32_t& z,
                                           uint32_t& w) {
-  asm volatile("ld.global.nc.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"
                : "=r"(x), "=r"(y), "=r"(z), "=r"(w)
                : "l"(p));
 }
@@ -412,8 +412,8 @@ __device__ __forceinline__ RowPre load_pre(const Args& a, int64_t row, int32_t y
     p.eos = a.eos[row];
   }
   if (MODE != MODE_DECODE && p.r >= 0) {
-    p.lo = __ldg(a.offsets + p.r);
-    p.hi = __ldg(a.offsets + p.r + 1);
+    p.lo = a.offsets[p.r];
+    p.hi = a.offsets[p.r + 1];
   }
   return p;
 }
@@ -569,7 +569,7 @@ __device__ __forceinline__ void row_finish(const Args& a, int64_t row, float m, 
       ag[10] = (float)(n + 1) / (float)(2 * n);
 #pragma unroll
       for (int j = 0; j < NAGG; ++j) {
-        z = fmaf(__ldg(a.w + j), ag[j], z);
+        z = fmaf(a.w[j], ag[j], z);
         if (lane == j) mine = ag[j];
       }
       sc = 1.f / (1.f + expf(-z));

@@ -586,7 +586,7 @@ __global__ void lm_wait_probe(uint32_t* err, uint64_t limit_ns, int32_t* complet
 // products had ended: 1,640 rows of 70,001 logits from 1,024 features took 470 us
 // with lm_fused, now 422; 33 rows of 4,000 from 256: 52, now 44).
 template <int MODE>
-__global__ void __launch_bounds__(256) lm_merge(const Args a, const LmPart* __restrict__ parts,
+__global__ void __launch_bounds__(256) lm_merge(const Args a, const LmPart* parts,
                                                 int nparts, int wpr) {
   __shared__ float s_m[8], s_S[8], s_U[8], s_xy[8];
   __shared__ uint32_t s_fl[8];  // bit 0: a non-finite logit, bit 1: holds the chosen token
@@ -662,8 +662,8 @@ __global__ void __launch_bounds__(256) lm_merge(const Args a, const LmPart* __re
   } else if (a.offsets) {
     pre.r = find_request(a.offsets, a.n_req, row, lane);
     if (pre.r >= 0) {
-      pre.lo = __ldg(a.offsets + pre.r);
-      pre.hi = __ldg(a.offsets + pre.r + 1);
+      pre.lo = a.offsets[pre.r];
+      pre.hi = a.offsets[pre.r + 1];
     }
   }
   row_finish<float, MODE>(a, row, m, S, U, bad, lane < a.kc ? E : 0ull, pre, lane);

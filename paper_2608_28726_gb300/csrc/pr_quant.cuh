@@ -241,7 +241,7 @@ __device__ __forceinline__ uint32_t q_step(uint32_t d, uint32_t mul) {
 // Bound by the latency of this chain and, for long requests, of the passes.
 // `idle` runs before the sort (loads that the caller wants in flight).
 template <typename F>
-__device__ __forceinline__ void q_select(const float* __restrict__ feat, int64_t lo, int T,
+__device__ __forceinline__ void q_select(const float* feat, int64_t lo, int T,
                                          uint32_t* dyn, uint32_t (*qx)[Q_SMALL], float* out,
                                          F idle) {
   __shared__ uint32_t s_red[8][Q_NT / 32], s_rank[Q_NR], s_pre[4][64], s_half[4], s_n[4];
@@ -264,7 +264,7 @@ __device__ __forceinline__ void q_select(const float* __restrict__ feat, int64_t
       const uint32_t t = c0 + (uint32_t)(i * Q_NT + tid);
       if (t < (uint32_t)T) {
         const float4* rec = reinterpret_cast<const float4*>(feat + (lo + t) * NFEAT);
-        const float4 r0 = __ldg(rec), r1 = __ldg(rec + 1);
+        const float4 r0 = rec[0], r1 = rec[1];
         k[i][0] = q_key(r0.x);  // l
         k[i][1] = q_key(r0.y);  // m
         k[i][2] = q_key(r1.x);  // h
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(Q_NT, 3) qmlp_requests(const QArgs a) {
 #pragma unroll
     for (int i = 0; i < QW_PER_T; ++i) {
       const int g = tid + i * Q_NT;
-      wr[i] = g < QW_SIZE ? __ldg(a.w + g) : 0.f;
+      wr[i] = g < QW_SIZE ? a.w[g] : 0.f;
     }
   };
   if (T <= Q_MID) fetch_w();
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(Q_NT, 3) qmlp_requests(const QArgs a) {
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const int t = half * 128 + lane * 4 + e;
-        v[e] = t < T ? q_key(__ldg(a.feat + (lo + t) * NFEAT + slot)) : 0xffffffffu;
+        v[e] = t < T ? q_key(a.feat[(lo + t) * NFEAT + slot]) : 0xffffffffu;
       }
       q_sort256_pair(v, half, lane, qx[f], 1 + f);
 #pragma unroll
@@ -620,7 +620,7 @@ __global__ void __launch_bounds__(Q_NT, 3) qmlp_requests(const QArgs a) {
       uint32_t k0 = 0xffffffffu, k1 = 0xffffffffu, k2 = 0xffffffffu, k3 = 0xffffffffu;
       if (t < T) {
         const float4* rec = reinterpret_cast<const float4*>(a.feat + (lo + t) * NFEAT);
-        const float4 r0 = __ldg(rec), r1 = __ldg(rec + 1);
+        const float4 r0 = rec[0], r1 = rec[1];
         k0 = q_key(r0.x);  // l
         k1 = q_key(r0.y);  // m
         k2 = q_key(r1.x);  // h

@@ -145,8 +145,8 @@ __device__ __forceinline__ void sel_each(const SelArgs& a, uint32_t lo, uint32_t
   if (vec) {
 #pragma unroll 4
     for (uint64_t i = (uint64_t)lo + 4ull * first; i + 3 < hi; i += 4ull * step) {
-      const float4 f = __ldg(reinterpret_cast<const float4*>(a.scores + i));
-      const uint32_t l = labels ? __ldg(reinterpret_cast<const uint32_t*>(a.labels + i)) : 0u;
+      const float4 f = *reinterpret_cast<const float4*>(a.scores + i);
+      const uint32_t l = labels ? *reinterpret_cast<const uint32_t*>(a.labels + i) : 0u;
       one(f.x, (l & 0xffu) ? 1u : 0u);
       one(f.y, (l & 0xff00u) ? 1u : 0u);
       one(f.z, (l & 0xff0000u) ? 1u : 0u);

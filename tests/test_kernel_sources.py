@@ -21,3 +21,16 @@ def test_dynamic_shared_memory_declares_its_alignment(name):
     it starts wherever the static part ends.  (head_attn aligns its base itself.)"""
     for decl in re.findall(r"extern\s+__shared__[^;]*;", code(name)):
         assert "__align__(16)" in decl or "ha_raw" in decl, decl
+
+
+@pytest.mark.parametrize("name", FILES)
+def test_no_read_only_loads_of_the_callers_data(name):
+    """Kernels are resident before the kernel ahead of them has ended, so what that
+    one may write is not read through the path for read-only memory.  The scorer
+    head's weights may be: its row kernels start once what precedes the call is
+    complete."""
+    found = re.findall(r"[^\n]*(?:__ldg\s*\(|ld\.global\.nc|__restrict__)[^\n]*", code(name))
+    if name == "pr_head.cuh":
+        found = [f for f in found
+                 if not re.search(r"a\.lnext|\bL \+ H|__ldg\(wout|ht_copy_w", f)]
+    assert not found, found
