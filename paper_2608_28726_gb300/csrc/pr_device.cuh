@@ -17,15 +17,13 @@
 //   * exact top-K (and the first two tokens, lower index first on ties) at
 //     almost no streaming cost: each thread only stores the maximum of each of
 //     its tiles in shared memory.  After the stream, theta1 = the K-th largest
-//     of (some of) the per-thread maxima is a lower bound of the K-th largest
-//     element (K distinct elements reach it); the stored tile maxima >= theta1 are the
-//     candidate "super-groups"; theta = the K-th largest candidate value is a
-//     tighter bound, and every element >= theta lies in a candidate >= theta
-//     (an element below theta has K strictly larger elements, the maxima of K
-//     candidates).  Those few super-groups are re-read and their elements
-//     >= theta sorted by (value, lower index first) with warp bitonic networks.
-//     Ties never lose an element; rows whose ties swamp the buffers fall back
-//     to an exact scan of the whole row.
+//     of some of the per-thread maxima is a lower bound of the K-th largest
+//     element (K distinct elements reach it); where those let too much through
+//     (values side by side in few warps' shares) a bound from all of them takes
+//     its place.  The stored tile maxima >= theta1 are the candidate
+//     "super-groups"; those few are re-read and their elements >= theta1 ranked by
+//     (value, lower index first).  Ties never lose an element; rows whose ties
+//     swamp the buffers fall back to an exact scan of the whole row.
 //   * rows with -inf (masked tokens), NaN or +inf make the fast accumulators
 //     non-finite; such rows are re-streamed with per-element guards, which
 //     classify them exactly.
@@ -363,15 +361,12 @@ struct RowPre {
 struct Smem {
   float tm[MAX_SLOTS][NT];    // per-thread tile (super-group) maxima
   uint32_t pub[NWARP * PUB];  // every warp's largest thread maxima, ord() encoded
-  union {
-    uint32_t all_max[NT];     // all thread maxima, when the published ones do not suffice
-    uint32_t cand_id[CCAP];   // candidate super-groups: slot << 8 | thread
-  };
+  uint32_t all_max[NT];       // all thread maxima, for where the published ones do not suffice
+  uint32_t cand_id[CCAP];     // candidate super-groups: slot << 8 | thread
   uint64_t ebuf[ECAP];        // candidate element keys
   float pm[NWARP], pS[NWARP], pU[NWARP];
   int pbad[NWARP];
-  int ncand, nelem, careful;
-  float theta1;
+  int ncand[2], nelem[2], careful;
   uint64_t top[32];           // the CTA's top-32 keys, ranked by counting
   RowPre pre;
   // cluster rank 0: the other CTAs' states (m, S, U, bad) and top-32 lists

@@ -585,13 +585,19 @@ __device__ __forceinline__ void row_finish(const Args& a, int64_t row, float m, 
   }
 }
 
-// 32 of a CTA's largest thread maxima into pub[0 .. 31], from which theta1 comes:
-// every warp's PUB largest ones; of a range of less than a tile, whose first
-// warps hold all of it, the 32 / A largest ones of A warps, A the largest power
-// of two up to the number of warps with a group in every lane.
-__device__ __forceinline__ void publish_max(uint32_t cur, uint32_t* pub, int32_t groups, int warp,
-                                            int lane) {
+// What theta1 comes from.  pub[0 .. 31]: 32 of a CTA's largest thread maxima, every
+// warp's PUB largest ones; of a range of less than a tile, whose first warps hold
+// all of it, the 32 / A largest ones of A warps, A the largest power of two up to the
+// number of warps with a group in every lane.  low[warp] (unless null): a code that
+// at least kc of the warp's maxima reach, for rows whose largest values lie side by
+// side in one warp's share (a range of allowed tokens, sorted logits).
+__device__ __forceinline__ void publish_max(uint32_t cur, uint32_t* pub, uint32_t* low,
+                                            int32_t groups, int kc, int warp, int lane) {
   if (groups >= TILE) {
+    if (low) {
+      const uint32_t least = __reduce_min_sync(FULL, cur);
+      if (lane == 0) low[warp] = least;
+    }
 #pragma unroll
     for (int i = 0; i < PUB; ++i) {
       const uint32_t w = __reduce_max_sync(FULL, cur);
@@ -603,10 +609,66 @@ __device__ __forceinline__ void publish_max(uint32_t cur, uint32_t* pub, int32_t
   }
   const int full = max(1, (groups + 32 * (UNR - 1)) / (32 * UNR));  // warps with 32 groups or more
   const int A = full >= 8 ? 8 : full >= 4 ? 4 : full >= 2 ? 2 : 1, n = 32 / A;
-  if (warp >= A) return;
+  if (warp >= A) {
+    if (low && lane == 0) low[warp] = 0u;
+    return;
+  }
   cur = warp_sort_desc<uint32_t>(cur, lane);
   if (lane < n) pub[warp * n + lane] = cur;
+  if (low && lane == kc - 1) low[warp] = cur;
 }
+
+// A better bound where theta1 lets too many tiles or elements pass (values side by
+// side in the shares of few warps), by bisection of the ord() codes of all thread
+// maxima (code(j): this lane's j-th, N per lane) from th1, which at least kc of them
+// reach, to the smallest of kc to kc + 4 of them (of more where they tie).
+// With 1,000 neighbouring tokens 10 above the others: 256 rows of V = 151,936 bf16
+// 781 us when the published maxima alone decided and such rows went on to the scan,
+// 21 now; 1,500 rows 3,594 us, 95 now.
+template <int N, typename F>
+__device__ __forceinline__ float raise_bound(F code, float th1, int kc) {
+  uint32_t v[N], lo = ord(th1);
+#pragma unroll
+  for (int j = 0; j < N; ++j) v[j] = code(j);
+  auto reach = [&](uint32_t from) {
+    int c = 0;
+#pragma unroll
+    for (int j = 0; j < N; ++j) c += v[j] >= from ? 1 : 0;
+    return __reduce_add_sync(FULL, c);
+  };
+  if (reach(lo + 1u) < kc) return th1;  // ties, or too few unmasked tokens
+  uint32_t hi = v[0];
+#pragma unroll
+  for (int j = 1; j < N; ++j) hi = max(hi, v[j]);
+  hi = __reduce_max_sync(FULL, hi) + 1u;
+#pragma unroll 1
+  while (hi - lo > 1u) {
+    const uint32_t mid = lo + ((hi - lo) >> 1);
+    const int c = reach(mid);
+    if (c < kc) {
+      hi = mid;
+    } else {
+      lo = mid;
+      if (c <= kc + 4) break;
+    }
+  }
+  uint32_t least = 0xffffffffu;  // the least of those that reach lo: nothing lies between
+#pragma unroll
+  for (int j = 0; j < N; ++j) least = v[j] >= lo ? min(least, v[j]) : least;
+  return unord(__reduce_min_sync(FULL, least));
+}
+static __device__ __noinline__ float raise_cta(const uint32_t* all, float th1, int kc, int lane) {
+  return raise_bound<NWARP>([&](int j) { return all[32 * j + lane]; }, th1, kc);
+}
+__device__ __forceinline__ float raise_ws(const float4* tinfo, uint32_t edge, float th1, int kc,
+                                              int lane) {
+  return raise_bound<NWARP + 1>(
+      [&](int j) { return j < NWARP ? ord(tinfo[j * 32 + lane].x) : edge; }, th1, kc);
+}
+// Candidate tiles from which on it is tried.  Of values in no order about kc + 3 reach
+// theta1, up to twice as many in a range of less than a tile (of which not every
+// warp publishes) or where kc is most of what is published.
+__device__ __forceinline__ int many_tiles(int kc) { return 2 * kc + 24; }
 
 // ---- the row kernel for split rows: one thread-block cluster of C CTAs per row ----------------
 
@@ -621,59 +683,71 @@ constexpr int rows_min_blocks() {
   return sizeof(T) == 4 && ALIGNED ? 5 : 4;
 }
 
+// What a CTA of the split kernel works on.  Read from the special registers each time
+// it is built: the stream and the selection after it build their own, so that
+// nothing of the latter takes registers from the former (kept alive together, fp32
+// batches of V = 151,936 took up to 9% longer).
+template <typename T>
+struct SplitPlace {
+  uint32_t C, rank, cid;  // CTAs of the row, this one's, the row
+  int32_t gfull, g0, g1, ng, ntiles, shift;
+  __device__ __forceinline__ explicit SplitPlace(const Args& a) {
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(cid));
+    gfull = (int32_t)((uint32_t)a.vocab / Traits<T>::VEC);
+    const int lc = __ffs(C) - 1;  // C is 1, 2, 4 or 8
+    g0 = (int32_t)(((int64_t)gfull * rank) >> lc);
+    g1 = (int32_t)(((int64_t)gfull * (rank + 1)) >> lc);
+    ng = g1 - g0;
+    ntiles = (int32_t)((uint32_t)(ng + TILE - 1) / TILE);
+    shift = 0;
+    while (((ntiles + (1 << shift) - 1) >> shift) > MAX_SLOTS) ++shift;
+  }
+  __device__ __forceinline__ const T* row(const Args& a) const {
+    return reinterpret_cast<const T*>(a.logits) + (int64_t)cid * a.row_stride;
+  }
+};
+
 template <typename T, int MODE, bool ALIGNED>
 __global__ void __launch_bounds__(NT, rows_min_blocks<T, ALIGNED>()) verify_rows(const Args a) {
   __shared__ Smem sm;
   using Tr = Traits<T>;
   constexpr int VEC = Tr::VEC;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint32_t C, rank, cid;
-  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
-  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-  asm("mov.u32 %0, %%clusterid.x;" : "=r"(cid));
-  const int64_t row = cid;
-
-  pdl_enter(a.early);
-  if (C > 1) cluster_arrive();  // every CTA of the cluster has started (waited for below)
-
-  const char* rowp = reinterpret_cast<const char*>(a.logits) + row * a.row_stride * (int64_t)sizeof(T);
-  const int64_t V = a.vocab;
-  const T* rowt = reinterpret_cast<const T*>(rowp);
-  const uint4* vp = reinterpret_cast<const uint4*>(rowp);
-  const RowGeom geo(V, VEC);
-  const int32_t g0 = (int32_t)((int64_t)geo.gfull * rank / C);
-  const int32_t g1 = (int32_t)((int64_t)geo.gfull * (rank + 1) / C);
-  const int32_t ng = g1 - g0;
-  const int32_t nfull = ng / TILE, rem = ng - nfull * TILE;
-  const int32_t ntiles = nfull + (rem > 0 ? 1 : 0);
-  const int32_t nedge = rank == 0 ? geo.nedge : 0;  // cluster rank 0 takes the last elements
-  int shift = 0;
-  while (((ntiles + (1 << shift) - 1) >> shift) > MAX_SLOTS) ++shift;
-  const int32_t smask = (1 << shift) - 1;
-  const int32_t nslots = (ntiles + smask) >> shift;
   const uint4 NEG = make_uint4(Tr::NEG_WORD, Tr::NEG_WORD, Tr::NEG_WORD, Tr::NEG_WORD);
 
+  pdl_enter(a.early);
+
+  float m = M2_INIT;
+  float2 S2 = make_float2(0.f, 0.f), U2 = make_float2(0.f, 0.f);
+  float thr_max = -INFINITY;
+  bool bad = false;
+
+  // ---- stream the groups [g0, g1): tile t holds groups t*TILE + k*NT + tid ------------
+  {
+    const SplitPlace<T> pl(a);
+    const uint32_t C = pl.C;
+    const int32_t g0 = pl.g0, g1 = pl.g1, ng = pl.ng, ntiles = pl.ntiles, shift = pl.shift;
+    const int32_t nfull = (int32_t)((uint32_t)ng / TILE), rem = ng & (TILE - 1), smask = (1 << shift) - 1;
+    const T* rowt = pl.row(a);
+    const uint4* vp = reinterpret_cast<const uint4*>(rowt);
+    float racc = -INFINITY;
+    if (C > 1) cluster_arrive();  // every CTA of the cluster has started (waited for below)
   if (tid == 0) {
-    sm.ncand = 0;
-    sm.nelem = 0;
+    sm.ncand[0] = sm.ncand[1] = 0;
+    sm.nelem[0] = sm.nelem[1] = 0;
     // the row's inputs beside the logits, on their way into L2 while it streams
-    if (rank == 0) {
-      prefetch_line(a.chosen + row);
+    if (pl.rank == 0) {
+      prefetch_line(a.chosen + pl.cid);
       if (MODE == MODE_DECODE) {
-        prefetch_line(a.slot + row);
-        prefetch_line(a.eos + row);
+        prefetch_line(a.slot + pl.cid);
+        prefetch_line(a.eos + pl.cid);
       }
     }
   }
   if (tid < 32) sm.top[tid] = 0ull;
 
-  float m = M2_INIT;
-  float2 S2 = make_float2(0.f, 0.f), U2 = make_float2(0.f, 0.f);
-  float thr_max = -INFINITY, racc = -INFINITY;
-  bool bad = false;
-
-  // ---- stream the groups [g0, g1): tile t holds groups t*TILE + k*NT + tid ------------
-  {
     // the groups of tile t (off the grid: uncut), nothing past the range
     auto load_tile = [&](uint4 (&dst)[UNR], uint32_t (&ext)[UNR], int32_t t) {
       const int32_t nb = t * TILE;
@@ -694,8 +768,8 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T, ALIGNED>()) verify_rows
         }
       } else {
         // (a row of fewer groups than CTAs has its first group in a later CTA)
-        const bool rim = (row == 0 && g0 + nb == 0) ||
-                         (row == a.n_rows - 1 && g1 == geo.gfull && t == ntiles - 1);
+        const bool rim = (pl.cid == 0 && g0 + nb == 0) ||
+                         (pl.cid == a.n_rows - 1 && g1 == pl.gfull && t == ntiles - 1);
         ld_tile_off_grid(rowt, g0 + nb, g1, rim, tid, dst, ext, NEG);
       }
     };
@@ -755,6 +829,16 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T, ALIGNED>()) verify_rows
   }
   float S = S2.x + S2.y, U = U2.x + U2.y;
 
+  const SplitPlace<T> pl(a);
+  const uint32_t C = pl.C, rank = pl.rank, cid = pl.cid;
+  const int64_t row = cid, V = a.vocab;
+  const int32_t g0 = pl.g0, g1 = pl.g1, ng = pl.ng, ntiles = pl.ntiles, shift = pl.shift;
+  const int32_t nslots = (ntiles + (1 << shift) - 1) >> shift;
+  const char* rowp = reinterpret_cast<const char*>(pl.row(a));
+  const uint4* vp = reinterpret_cast<const uint4*>(rowp);
+  // cluster rank 0 takes the last elements
+  const int32_t nedge = rank == 0 ? (int32_t)V & (VEC - 1) : 0;
+
   // What follows the stream is a chain of latencies that a lone launch cannot
   // hide; it is kept short: four block barriers, no sort, every global load
   // issued as early as its address is known (see the phases' comments).
@@ -764,7 +848,7 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T, ALIGNED>()) verify_rows
 
   // ---- the elements after the last group: warp 0 of cluster rank 0, one per lane
   float xe = -INFINITY;
-  const int64_t ve = (int64_t)geo.gfull * VEC + lane;  // this lane's
+  const int64_t ve = (int64_t)pl.gfull * VEC + lane;  // this lane's
   if (warp == 0 && lane < nedge) {
     const float x = Tr::elem(rowp, ve);
     careful_add(x, m, S, U, bad);
@@ -778,7 +862,8 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T, ALIGNED>()) verify_rows
   // per warp and seven merges, about one candidate more passes it (22 for 21 of
   // 151,936 normal values and kc = 20).
   const int kc = a.kc;
-  publish_max(ord(thr_max), sm.pub, ng, warp, lane);
+  publish_max(ord(thr_max), sm.pub, nullptr, ng, kc, warp, lane);
+  sm.all_max[tid] = ord(thr_max);
   int32_t y = 0;
   if (rank == 0 && warp == 1) y = a.chosen[row];  // used after the next barrier
   __syncthreads();
@@ -793,42 +878,6 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T, ALIGNED>()) verify_rows
     }
     th1 = unord(__shfl_sync(FULL, mine, __ffs(__ballot_sync(FULL, rk == kc - 1)) - 1));
   }
-  if (!(th1 > -INFINITY) && ng > 32 * UNR) {
-    // fewer than kc published maxima (all but a few neighbouring tokens masked;
-    // one warp's share has published all it has): the kc-th largest of all
-    // thread maxima
-    sm.all_max[tid] = ord(thr_max);
-    if (tid == 0) sm.theta1 = -INFINITY;
-    __syncthreads();
-    const uint32_t mine = sm.all_max[tid];
-    int rk = 0;
-#pragma unroll 8
-    for (int j = 0; j < NT; ++j) {
-      const uint32_t q = sm.all_max[j];
-      rk += (q > mine || (q == mine && j < tid)) ? 1 : 0;
-    }
-    if (rk == kc - 1) sm.theta1 = thr_max;
-    __syncthreads();
-    th1 = sm.theta1;
-  }
-  const bool fallback = !(th1 > -INFINITY);
-
-  // ---- candidate super-groups: this thread's stored tile maxima >= theta1
-  if (!fallback && thr_max >= th1) {
-    uint32_t mask = 0u;
-#pragma unroll
-    for (int32_t s = 0; s < MAX_SLOTS; ++s)
-      if (s < nslots) mask |= sm.tm[s][tid] >= th1 ? 1u << s : 0u;
-    if (mask) {
-      int i = atomicAdd(&sm.ncand, __popc(mask));
-      for (; mask; mask &= mask - 1u, ++i)
-        if (i < CCAP) sm.cand_id[i] = ((uint32_t)(__ffs(mask) - 1) << 8) | (uint32_t)tid;
-    }
-    if (xe >= th1) {  // an edge element is a candidate by itself
-      const int e = atomicAdd(&sm.nelem, 1);
-      if (e < ECAP) sm.ebuf[e] = make_key(xe, (uint32_t)ve);
-    }
-  }
   // the warp's state
   lse_warp(m, S, U);
   bad = __any_sync(FULL, bad);
@@ -838,69 +887,100 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T, ALIGNED>()) verify_rows
     sm.pU[warp] = U;
     sm.pbad[warp] = bad;
   }
-  __syncthreads();
 
-  // ---- re-read the candidates (a 16-byte group per thread, all in flight at
-  // once); their elements >= theta1 become keys: kc distinct elements reach
-  // theta1, so the CTA's top kc are among them
-  const int ncand = sm.ncand;
-  const bool fb_cand = fallback || ncand > CCAP;
-  const int total = fb_cand ? 0 : ncand * (UNR << shift);  // groups of the super-groups
-  int32_t g = -1;
-  uint4 wv = NEG;
-  auto fetch = [&](int i) {
-    const int c = i / UNR >> shift, j = i - (c << shift) * UNR;
-    const uint32_t id = sm.cand_id[c];
-    const int32_t t = (int32_t)((id >> 8) << shift) + j / UNR;
-    const int32_t gi = t * TILE + tile_pos((int)(id & 255u), j % UNR);
-    g = t < ntiles && gi < ng ? g0 + gi : -1;
-    if (g >= 0) wv = ALIGNED ? ld_reread(vp + g) : Tr::load_elems(rowp, g);
-  };
-  if (tid < total) fetch(tid);
-  // while they arrive: warp 0 merges the CTA's state, warp 1 of cluster rank 0
-  // finds what the row's epilogue needs besides the reduction
-  if (warp == 0) {
-    m = lane < NWARP ? sm.pm[lane] : M2_INIT;
-    S = lane < NWARP ? sm.pS[lane] : 0.f;
-    U = lane < NWARP ? sm.pU[lane] : 0.f;
-    bad = __any_sync(FULL, lane < NWARP && sm.pbad[lane] != 0);
+  // ---- candidates and their elements by theta1; once more by a bound from all
+  // thread maxima if too many reach theta1, or fewer than kc maxima are published (all
+  // but a few neighbouring tokens masked; one warp's share has published all it has)
+  bool more = ng > 32 * UNR, merged = false;
+  int ncand, at = 0;  // counters of this attempt
+#pragma unroll 1
+  for (;;) {
+    // candidate super-groups: this thread's stored tile maxima >= theta1
+    if (th1 > -INFINITY && thr_max >= th1) {
+      uint32_t mask = 0u;
 #pragma unroll
-    for (int o = NWARP / 2; o > 0; o >>= 1) {
-      const float mo = __shfl_xor_sync(FULL, m, o);
-      const float So = __shfl_xor_sync(FULL, S, o);
-      const float Uo = __shfl_xor_sync(FULL, U, o);
-      lse_merge(m, S, U, mo, So, Uo);
-    }
-    // only lanes 0..NWARP-1 took part in the last butterfly: give every lane the total
-    m = __shfl_sync(FULL, m, 0);
-    S = __shfl_sync(FULL, S, 0);
-    U = __shfl_sync(FULL, U, 0);
-    // a masked (-inf), NaN or infinite logit made the CTA's fast accumulators
-    // non-finite: it re-streams its range with guards (the row's merged state
-    // is non-finite exactly when a CTA's is)
-    if (lane == 0) sm.careful = (!bad && !(isfinite(S) && isfinite(U))) ? 1 : 0;
-  } else if (warp == 1 && rank == 0) {
-    const RowPre p = load_pre<T, MODE>(a, row, y, rowp, lane);
-    if (lane == 0) sm.pre = p;
-  }
-  for (int i = tid; i < total;) {
-    if (g >= 0) {
-      uint32_t hits = 0u;
-#pragma unroll
-      for (int e = 0; e < VEC; ++e) hits |= Tr::at(wv, e) >= th1 ? 1u << e : 0u;
-      if (hits) {
-        int at = atomicAdd(&sm.nelem, __popc(hits));
-        for (; hits; hits &= hits - 1u, ++at) {
-          const int e = __ffs(hits) - 1;
-          if (at < ECAP)
-            sm.ebuf[at] = make_key(Tr::at(wv, e), (uint32_t)(g * VEC + e));
-        }
+      for (int32_t s = 0; s < MAX_SLOTS; ++s)
+        if (s < nslots) mask |= sm.tm[s][tid] >= th1 ? 1u << s : 0u;
+      if (mask) {
+        int i = atomicAdd(&sm.ncand[at], __popc(mask));
+        for (; mask; mask &= mask - 1u, ++i)
+          if (i < CCAP) sm.cand_id[i] = ((uint32_t)(__ffs(mask) - 1) << 8) | (uint32_t)tid;
+      }
+      if (xe >= th1) {  // an edge element is a candidate by itself
+        const int e = atomicAdd(&sm.nelem[at], 1);
+        if (e < ECAP) sm.ebuf[e] = make_key(xe, (uint32_t)ve);
       }
     }
-    i += NT;
-    if (i < total) fetch(i);
+    __syncthreads();
+    ncand = sm.ncand[at];
+    if (!more || (th1 > -INFINITY && ncand <= many_tiles(kc))) {
+      // re-read the candidates (a 16-byte group per thread, all in flight at
+      // once); their elements >= theta1 become keys: kc distinct elements reach
+      // theta1, so the CTA's top kc are among them
+      const int total = ncand <= CCAP ? ncand * (UNR << shift) : 0;  // the super-groups' groups
+      int32_t g = -1;
+      uint4 wv = NEG;
+      auto fetch = [&](int i) {
+        const int c = i / UNR >> shift, j = i - (c << shift) * UNR;
+        const uint32_t id = sm.cand_id[c];
+        const int32_t t = (int32_t)((id >> 8) << shift) + j / UNR;
+        const int32_t gi = t * TILE + tile_pos((int)(id & 255u), j % UNR);
+        g = t < ntiles && gi < ng ? g0 + gi : -1;
+        if (g >= 0) wv = ALIGNED ? ld_reread(vp + g) : Tr::load_elems(rowp, g);
+      };
+      if (tid < total) fetch(tid);
+      // while they arrive: warp 0 merges the CTA's state, warp 1 of cluster rank 0
+      // finds what the row's epilogue needs besides the reduction
+      if (warp == 0 && !merged) {
+        m = lane < NWARP ? sm.pm[lane] : M2_INIT;
+        S = lane < NWARP ? sm.pS[lane] : 0.f;
+        U = lane < NWARP ? sm.pU[lane] : 0.f;
+        bad = __any_sync(FULL, lane < NWARP && sm.pbad[lane] != 0);
+#pragma unroll
+        for (int o = NWARP / 2; o > 0; o >>= 1) {
+          const float mo = __shfl_xor_sync(FULL, m, o);
+          const float So = __shfl_xor_sync(FULL, S, o);
+          const float Uo = __shfl_xor_sync(FULL, U, o);
+          lse_merge(m, S, U, mo, So, Uo);
+        }
+        // only lanes 0..NWARP-1 took part in the last butterfly: give every lane the total
+        m = __shfl_sync(FULL, m, 0);
+        S = __shfl_sync(FULL, S, 0);
+        U = __shfl_sync(FULL, U, 0);
+        // a masked (-inf), NaN or infinite logit made the CTA's fast accumulators
+        // non-finite: it re-streams its range with guards (the row's merged state
+        // is non-finite exactly when a CTA's is)
+        if (lane == 0) sm.careful = (!bad && !(isfinite(S) && isfinite(U))) ? 1 : 0;
+      } else if (warp == 1 && rank == 0 && !merged) {
+        const RowPre p = load_pre<T, MODE>(a, row, y, rowp, lane);
+        if (lane == 0) sm.pre = p;
+      }
+      merged = true;
+      for (int i = tid; i < total;) {
+        if (g >= 0) {
+          uint32_t hits = 0u;
+#pragma unroll
+          for (int e = 0; e < VEC; ++e) hits |= Tr::at(wv, e) >= th1 ? 1u << e : 0u;
+          if (hits) {
+            int k = atomicAdd(&sm.nelem[at], __popc(hits));
+            for (; hits; hits &= hits - 1u, ++k) {
+              const int e = __ffs(hits) - 1;
+              if (k < ECAP)
+                sm.ebuf[k] = make_key(Tr::at(wv, e), (uint32_t)(g * VEC + e));
+            }
+          }
+        }
+        i += NT;
+        if (i < total) fetch(i);
+      }
+      __syncthreads();
+      if (!more || sm.nelem[at] <= NT) break;
+    }
+    more = false;
+    at = 1;
+    th1 = raise_cta(sm.all_max, th1, kc, lane);
   }
-  __syncthreads();
+  const bool fb_cand = !(th1 > -INFINITY) || ncand > CCAP;
   if (sm.careful) {
     float cm = M2_INIT, cS = 0.f, cU = 0.f;
     bool cbad = false;
@@ -920,7 +1000,7 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T, ALIGNED>()) verify_rows
   // keys with two threads each), more by warp 0's sorting network; the exact
   // scan when the buffers overflowed
   uint64_t E = 0ull;
-  const int ne = sm.nelem;
+  const int ne = sm.nelem[at];
   const bool fb = fb_cand || ne > ECAP;
   if (!fb && ne <= NT) {
     if (ne <= NT / 2) {
@@ -1042,7 +1122,8 @@ __device__ __forceinline__ void named_bar_arrive(int id, int n) {
 struct SmemWS {
   float4 tinfo[2][NT];          // per thread: best, second and third tile maxima, and
                                 //   (best tile | second tile << 16); two row buffers
-  uint32_t pub[2][NWARP * PUB]; // every warp's largest thread maxima, ord() encoded
+  uint32_t pub[2][NWARP * PUB]; // every warp's largest thread maxima, ord() encoded, and
+  uint32_t low[2][NWARP];       //   what kc of its maxima reach (publish_max)
   float pm[2][NWARP], pS[2][NWARP], pU[2][NWARP];
   uint32_t cand_id[CCAP];       // finaliser: candidate tiles (tile << 8 | thread, | BEST_BIT
                                 //   for a thread's best tile)
@@ -1141,30 +1222,16 @@ __device__ __noinline__ void finalize_ws(const Args& a, SmemWS& sm, int b, int64
     const unsigned hite = __ballot_sync(FULL, edge && re == kc - 1);
     const uint32_t v = hit ? __shfl_sync(FULL, mine, __ffs(hit) - 1)
                            : __shfl_sync(FULL, em, (__ffs(hite) - 1) & 31);
-    th1 = unord(v);
+    th1 = unord(max(v, __reduce_max_sync(FULL, sm.low[b][lane & (NWARP - 1)])));
   }
-  if (!(th1 > -INFINITY)) {
-    // fewer than kc published maxima (all but a few neighbouring tokens
-    // masked): the kc-th largest of all thread maxima, bit by bit
-    uint32_t v[NT / 32 + 1], kth = 0u;
-#pragma unroll
-    for (int j = 0; j < NT / 32; ++j) v[j] = ord(sm.tinfo[b][j * 32 + lane].x);
-    v[NT / 32] = edge ? ord(xe) : 0u;
-#pragma unroll 1
-    for (uint32_t bit = 0x80000000u; bit; bit >>= 1) {
-      int c = 0;
-#pragma unroll
-      for (int j = 0; j <= NT / 32; ++j) c += __popc(__ballot_sync(FULL, v[j] >= (kth | bit)));
-      if (c >= kc) kth |= bit;
-    }
-    th1 = unord(kth);
-  }
-  bool fb = !(th1 > -INFINITY);
-
-  // ---- candidate tiles: lane l looks at the reports of threads l, 32 + l, ...
-  int n = 0;  // candidate tiles
-  if (!fb) {
-    uint32_t m1 = 0u, m2 = 0u, m3 = 0u;  // bit j: best, second, third tile >= theta1
+  // ---- candidate tiles: lane l looks at the reports of threads l, 32 + l, ...  Once
+  // more by a bound from all thread maxima if too many reach theta1, or fewer than
+  // kc maxima are published (all but a few neighbouring tokens masked; rows of up
+  // to 32 x UNR groups have published all they have)
+  uint32_t m1, m2, m3;  // bit j: best, second, third tile >= theta1
+  int x, n;
+  auto count = [&]() {
+    m1 = m2 = m3 = 0u;
 #pragma unroll
     for (int j = 0; j < NT / 32; ++j) {
       const float4 inf = sm.tinfo[b][j * 32 + lane];
@@ -1173,15 +1240,24 @@ __device__ __noinline__ void finalize_ws(const Args& a, SmemWS& sm, int b, int64
       m3 |= inf.z >= th1 ? 1u << j : 0u;
     }
     m2 &= ~m3;
-    int x = __popc(m1) + __popc(m2);
-    const int own = x;
+    x = __popc(m1) + __popc(m2);
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(FULL, x, o);
       if (lane >= o) x += y;
     }
-    n = __shfl_sync(FULL, x, 31);
-    int pos = x - own;
+    n = __shfl_sync(FULL, x, 31);  // candidate tiles
+  };
+  count();
+  // (32 candidates are read at once: where theta1 is sharp, more are already too many)
+  const int many = kc <= 24 && geo.gfull >= TILE ? kc + 12 : many_tiles(kc);
+  if (geo.gfull > 32 * UNR && (n > many || !(th1 > -INFINITY))) {
+    th1 = raise_ws(sm.tinfo[b], edge ? ord(xe) : 0u, th1, kc, lane);
+    count();
+  }
+  bool fb = !(th1 > -INFINITY);
+  if (!fb) {
+    int pos = x - __popc(m1) - __popc(m2);
     for (uint32_t q = m1; q; q &= q - 1u, ++pos) {
       const uint32_t t = (uint32_t)((__ffs(q) - 1) * 32 + lane);
       if (pos < CCAP)
@@ -1266,6 +1342,7 @@ __device__ __noinline__ void finalize_ws(const Args& a, SmemWS& sm, int b, int64
     }
     if (ne > ECAP) fb = true;
   }
+  // (the scan below is the shorter, the higher its bound)
   __syncwarp();
 
   // ---- the row's exact top-32 elements: up to 64 keys are ranked by counting
@@ -1632,7 +1709,7 @@ __global__ void __launch_bounds__(NT_WS, 3) verify_rows_ws(const Args a) {
       sm.pS[b][warp] = S;
       sm.pU[b][warp] = U;
     }
-    publish_max(ord(v1), sm.pub[b], geo.gfull, warp, lane);
+    publish_max(ord(v1), sm.pub[b], sm.low[b], geo.gfull, a.kc, warp, lane);
     sm.tinfo[b][tid] = make_float4(v1, v2, v3, __uint_as_float(i1 | (i2 << 16)));
     __syncwarp();
     __threadfence_block();
