@@ -373,6 +373,7 @@ struct Smem {
   uint32_t peer_state[MAXC][4];
   uint64_t peer_list[MAXC][32];
 };
+static_assert(ECAP / NWARP >= 64, "a buffer of WarpTopK per warp");
 static_assert(NWARP * PUB == 32 && PUB * NWARP >= 32, "one published maximum per lane; kc <= 32");
 
 // ---- warp-level top-32 of pushed keys ---------------------------------------------

@@ -670,6 +670,47 @@ __device__ __forceinline__ float raise_ws(const float4* tinfo, uint32_t edge, fl
 // warp publishes) or where kc is most of what is published.
 __device__ __forceinline__ int many_tiles(int kc) { return 2 * kc + 24; }
 
+// The exact scan, of groups [ga, gb) by one warp: rows whose ties overflow the
+// buffers, or with fewer than kc unmasked tokens.  Elements from thr on go to the
+// list; once that is full, only those that beat its last entry: an element of a
+// later round has a higher index, so that its equals no longer count.  (A round's
+// elements come by their place in the group, not by index: the bound moves
+// between rounds.)  AHEAD rounds' loads are in flight.
+template <typename T, bool ALIGNED, int AHEAD>
+__device__ __forceinline__ void scan_groups(const char* rowp, int32_t ga, int32_t gb, float thr,
+                                            WarpTopK& ek, int lane) {
+  using Tr = Traits<T>;
+  const uint4 NEG = make_uint4(Tr::NEG_WORD, Tr::NEG_WORD, Tr::NEG_WORD, Tr::NEG_WORD);
+  uint32_t least = 0u;  // ord() code
+#pragma unroll 1
+  for (int32_t g0 = ga; g0 < gb; g0 += 32 * AHEAD) {
+    uint4 w[AHEAD];
+#pragma unroll
+    for (int k = 0; k < AHEAD; ++k) {
+      const int32_t g = g0 + 32 * k + lane;
+      w[k] = NEG;
+      if (g < gb)
+        w[k] = ALIGNED ? ld_stream(reinterpret_cast<const uint4*>(rowp) + g)
+                       : Tr::load_elems(rowp, g);
+    }
+#pragma unroll
+    for (int k = 0; k < AHEAD; ++k) {
+      const int32_t g = g0 + 32 * k + lane;
+      const float most = Tr::gmax(w[k]);
+      if (!__any_sync(FULL, g < gb && most >= thr && ord(most) >= least)) continue;
+#pragma unroll 1
+      for (int e = 0; e < Tr::VEC; ++e) {
+        const float x = Tr::at(w[k], e);
+        const bool c = g < gb && x >= thr && ord(x) >= least;
+        ek.push(c, c ? make_key(x, (uint32_t)(g * Tr::VEC + e)) : 0ull, lane);
+        ek.drain(lane);
+      }
+      const uint64_t last = shfl64(ek.list, 31);
+      if (last != 0ull) least = (uint32_t)(last >> 32) + 1u;
+    }
+  }
+}
+
 // ---- the row kernel for split rows: one thread-block cluster of C CTAs per row ----------------
 
 // Resident CTAs per SM the compiler sizes registers for: five for fp32 rows
@@ -1021,41 +1062,35 @@ __global__ void __launch_bounds__(NT, rows_min_blocks<T, ALIGNED>()) verify_rows
     }
     __syncthreads();
     if (warp == 0) E = sm.top[lane];
-  } else if (warp == 0) {
-    const int n = ne;
-    if (!fb) {
-      for (int b0 = 0; b0 < n; b0 += 32) {
-        uint64_t k = b0 + lane < n ? sm.ebuf[b0 + lane] : 0ull;
+  } else if (!fb) {
+    if (warp == 0)
+      for (int b0 = 0; b0 < ne; b0 += 32) {
+        uint64_t k = b0 + lane < ne ? sm.ebuf[b0 + lane] : 0ull;
         k = warp_sort_desc<uint64_t>(k, lane);
         E = warp_merge_desc<uint64_t>(E, k, lane);
       }
-    } else {
-      // exact scan of the whole range (rows whose ties overflow the buffers)
-      const float thr = th1;
-      WarpTopK ek;
-      ek.buf = sm.ebuf;
-      ek.cnt = 0;
-      ek.list = 0ull;
-      for (int32_t gb = 0; gb < ng; gb += 32) {
-        const int32_t gi = gb + lane;
-        const bool in = gi < ng;
-        uint4 w4 = NEG;
-        if (in) w4 = ALIGNED ? ld_stream(vp + g0 + gi) : Tr::load_elems(rowp, (int64_t)(g0 + gi));
-#pragma unroll 1
-        for (int e2 = 0; e2 < VEC; ++e2) {
-          const float x = Tr::at(w4, e2);
-          const bool c = in && x >= thr;
-          ek.push(c, c ? make_key(x, (uint32_t)((g0 + gi) * VEC + e2)) : 0ull, lane);
-          ek.drain(lane);
-        }
-      }
-      if (nedge > 0) {
-        const bool c = lane < nedge && xe >= thr;
-        ek.push(c, c ? make_key(xe, (uint32_t)ve) : 0ull, lane);
-        ek.drain(lane);
-      }
-      ek.drain_all(lane);
+  } else {
+    // exact scan of the whole range, an eighth of it per warp (256 equal rows of
+    // V = 151,936 bf16: 3,760 us with one warp and no rising bound, 50 now)
+    WarpTopK ek;
+    ek.buf = sm.ebuf + warp * (ECAP / NWARP);
+    ek.cnt = 0;
+    ek.list = 0ull;
+    scan_groups<T, ALIGNED, 2>(rowp, g0 + (int32_t)((int64_t)ng * warp / NWARP),
+                               g0 + (int32_t)((int64_t)ng * (warp + 1) / NWARP), th1, ek, lane);
+    if (warp == 0 && nedge > 0) {
+      const bool c = lane < nedge && xe >= th1;
+      ek.push(c, c ? make_key(xe, (uint32_t)ve) : 0ull, lane);
+      ek.drain(lane);
+    }
+    ek.drain_all(lane);
+    __syncthreads();
+    sm.ebuf[32 * warp + lane] = ek.list;
+    __syncthreads();
+    if (warp == 0) {
       E = ek.list;
+      for (int w = 1; w < NWARP; ++w)
+        E = warp_merge_desc<uint64_t>(E, sm.ebuf[32 * w + lane], lane);
     }
   }
 
@@ -1372,25 +1407,13 @@ __device__ __noinline__ void finalize_ws(const Args& a, SmemWS& sm, int b, int64
       E = warp_merge_desc<uint64_t>(E, k, lane);
     }
   } else {
-    // exact scan of the whole row (rows whose ties overflow the buffers)
+    // exact scan of the whole row (1,500 equal rows of V = 151,936 bf16: 14.7 ms
+    // without the rising bound, 0.64 now)
     WarpTopK ek;
     ek.buf = sm.ebuf;
     ek.cnt = 0;
     ek.list = 0ull;
-#pragma unroll 1
-    for (int32_t g0 = 0; g0 < geo.gfull; g0 += 32) {
-      const int32_t g = g0 + lane;
-      const bool in = g < geo.gfull;
-      uint4 w4 = NEG;
-      if (in) w4 = ALIGNED ? ld_stream(vp + g) : Tr::load_elems(rowp, g);
-#pragma unroll 1
-      for (int e2 = 0; e2 < VEC; ++e2) {
-        const float x = Tr::at(w4, e2);
-        const bool c = in && x >= th1;
-        ek.push(c, c ? make_key(x, (uint32_t)(g * VEC + e2)) : 0ull, lane);
-        ek.drain(lane);
-      }
-    }
+    scan_groups<T, ALIGNED, 4>(rowp, 0, geo.gfull, th1, ek, lane);
     if (geo.nedge > 0) {
       const bool c = edge && xe >= th1;
       ek.push(c, c ? make_key(xe, (uint32_t)ve) : 0ull, lane);

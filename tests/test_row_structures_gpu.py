@@ -70,6 +70,13 @@ def test_structured_rows_match_the_oracle(B, dtype, V, K, split):
         x[r:r + 2] = shape_rows(x[r:r + 2], kind, width)
         ch[r:r + 2] = V // 3 + 1
         pick += [r, r + 1]
+    x[120:122] = 1.25                                   # all tied
+    x[122:124] = torch.arange(V, device="cuda") % 7     # many ties at the top
+    x[124:126] = -float("inf")
+    x[124, [5, V - 2]] = x[125, [V // 2, V - 1]] = -1.0  # two tokens left, tied
+    x[126:128] = torch.arange(V, device="cuda") // 8    # climbs by ties of 8, to the last token
+    ch[124:126] = torch.tensor([V - 2, V // 2])
+    pick += list(range(120, 128))
     x = x.to(dtype)
     feat, top2, fl = features(B, ctx, x, ch, K)
     xs, cn = as_oracle(x), ch.cpu().numpy()
@@ -123,5 +130,32 @@ def test_structured_rows_take_about_the_time_of_others(B, n, dtype):
              for k in ("bump", "bump_across", "two_bumps", "trend", "sorted", "sorted_up", "mask_1e4")
              if n > 16 or k != "mask_1e4"}  # (clusters: CTAs that hold only masked tokens scan)
     slow = {k: round(v / base, 2) for k, v in times.items() if v > 2.5 * base}
+    assert not slow, (slow, base)
+    B.pr_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("n", [16, 256, 1200])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_rows_that_are_scanned(B, n, dtype):
+    """Rows of one value, and rows with fewer unmasked tokens than K, take at most 25 times
+    as long as others (one warp scanned them, sorting every element: 44 to 340 times)."""
+    V = 100000 if n < 1000 else 60000
+    ctx = B.pr_ctx_create(0, n, 4)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    x0 = torch.randn(n, V, generator=g, device="cuda") * 2
+    ch = torch.zeros(n, dtype=torch.int32, device="cuda")
+    out = (torch.empty(n, 8, device="cuda"), torch.empty(n, 2, dtype=torch.int32, device="cuda"),
+           torch.empty(n, dtype=torch.int32, device="cuda"))
+
+    def t(x):
+        x = x.to(dtype)
+        return time_us(lambda: B.pr_token_features(ctx, x, ch, 20, None, *out))
+
+    base = t(x0)
+    times = {"one value": t(torch.full_like(x0, 0.5)),
+             "12 tokens left": t(shape_rows(x0.clone(), "mask_1e4", 12)),
+             "range in one CTA": t(shape_rows(x0.clone(), "mask_1e4"))}
+    slow = {k: round(v / base, 1) for k, v in times.items() if v > 25 * base}
     assert not slow, (slow, base)
     B.pr_ctx_destroy(ctx)
