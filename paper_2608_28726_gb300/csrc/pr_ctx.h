@@ -43,6 +43,9 @@ struct pr_ctx {
   int bps[2][3] = {{0, 0, 0}, {0, 0, 0}};
   // split kernel: shared memory opt-in made, per (dtype, mode, aligned)
   bool rows_ready[2][3][2] = {};
+  // and clusters resident at one CTA per SM, also per CTAs per row (2, 4, 8); 0 = not
+  // asked for yet
+  int places[2][3][2][3] = {};
   // persistent kernel: CTAs per SM per (dtype, mode, aligned); 0 = not set up yet
   int ws_bps[2][3][2] = {};
   // scorer head: activation scratch (rows x prk::HSCR floats), grown on demand

@@ -82,6 +82,58 @@ pr_status ws_setup(pr_ctx* c, pr_dtype dt, int mode, bool aligned, int* bps) {
   return PR_OK;
 }
 
+// Unused shared memory that holds every SM to its even share of a split launch's
+// CTAs.  A launch that follows another of these finds its CTAs still on the SMs and
+// would be spread around them, three on one SM and one on the next (16 decode steps
+// of 256 rows then took 306, 388 or 428 us, whichever pattern the launches fell into);
+// with the overlap option launches are meant to run side by side.  The CTAs of a
+// cluster lie within one GPC, whose SMs are no multiple of their number: at one CTA
+// per SM only 15 clusters of eight find a place on 152 SMs, so that the share is
+// counted from those.  V = 151,936 bf16: a step of 16 to 19 rows 9.2 us, 13.1 with a
+// share of rows x CTAs / SMs, 32 to 38 rows 10.5, 13.5 to 14.3.  (What the runtime
+// counts at two or more per SM is more than runs: with that, 32 rows took 12.9.)
+pr_status even_share(pr_ctx* c, pr_dtype dt, int mode, bool aligned, int64_t n_rows, int C,
+                     size_t* smem) {
+  const int bf16 = dt == PR_DTYPE_BF16 ? 1 : 0;
+  const int bps = blocks_per_sm(c, dt, mode);
+  if (n_rows * C > (int64_t)(bps - 1) * c->num_sms) return PR_OK;
+  void* f = row_kernel(dt, mode, aligned);
+  const int fixed = (int)sizeof(prk::Smem) + 1024;  // and what the system takes per CTA
+  auto pad = [&](int share) {
+    return (size_t)std::max(0, c->sm_smem / (share + 1) + 256 - fixed) & ~(size_t)127;
+  };
+  bool& ready = c->rows_ready[bf16][mode][aligned ? 1 : 0];
+  if (!ready) {
+    PR_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pad(1)));
+    ready = true;
+  }
+  int places = c->num_sms;  // rows at one CTA per SM
+  if (C > 1) {
+    int& known = c->places[bf16][mode][aligned ? 1 : 0][C == 2 ? 0 : C == 4 ? 1 : 2];
+    if (known == 0) {
+      cudaLaunchConfig_t cfg;
+      memset(&cfg, 0, sizeof cfg);
+      cfg.gridDim = dim3((unsigned)C);
+      cfg.blockDim = dim3(prk::NT);
+      cfg.dynamicSmemBytes = pad(1);
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = (unsigned)C;
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      int n = 0;
+      PR_CUDA(cudaOccupancyMaxActiveClusters(&n, f, &cfg));
+      known = std::max(n, 1);
+    }
+    places = known;
+  }
+  const int64_t share = (n_rows + places - 1) / places;
+  if (share < bps) *smem = pad((int)share);
+  return PR_OK;
+}
+
 // Launch shape of a batch: CTAs per row (C) and whether the persistent
 // kernel runs it.
 //  * the forced option: split 1 is the persistent kernel, 2 / 4 / 8 clusters;
@@ -149,24 +201,9 @@ pr_status launch_rows(pr_ctx* c, pr_dtype dt, int mode, prk::Args& a, cudaStream
   cfg.gridDim = dim3((unsigned)(a.n_rows * C), 1, 1);
   cfg.blockDim = dim3(prk::NT, 1, 1);
   cfg.stream = st;
-  // A launch that follows another of these finds its CTAs still on the SMs and
-  // would be spread around them, three on one SM and one on the next (16 decode
-  // steps of 256 rows then took 306, 388 or 428 us, whichever pattern the launches
-  // fell into).  Unused shared memory holds every SM to its even share; with
-  // the overlap option launches are meant to run side by side.
   if (!c->overlap) {
-    const int share = (int)((a.n_rows * C + c->num_sms - 1) / c->num_sms);
-    if (share < blocks_per_sm(c, dt, mode)) {
-      bool& ready = c->rows_ready[dt == PR_DTYPE_BF16 ? 1 : 0][mode][a.aligned ? 1 : 0];
-      void* f = row_kernel(dt, mode, a.aligned != 0);
-      const int fixed = (int)sizeof(prk::Smem) + 1024;  // and what the system takes per CTA
-      if (!ready) {
-        PR_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     c->sm_smem / 2 + 1024 - fixed));
-        ready = true;
-      }
-      cfg.dynamicSmemBytes = (size_t)std::max(0, c->sm_smem / (share + 1) + 256 - fixed) & ~(size_t)127;
-    }
+    const pr_status s = even_share(c, dt, mode, a.aligned != 0, a.n_rows, C, &cfg.dynamicSmemBytes);
+    if (s != PR_OK) return s;
   }
   cudaLaunchAttribute attr[2];
   int na = 0;

@@ -1,0 +1,49 @@
+"""Back-to-back split launches: every cluster of a step finds a place at once."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def step_us(B, ctx, n, V, dtype):
+    x = torch.randn(n, V, device="cuda").to(dtype)
+    z = torch.zeros(n, dtype=torch.int32, device="cuda")
+    slot = torch.arange(n, dtype=torch.int32, device="cuda")
+    eos = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    w, f = torch.zeros(11, device="cuda"), torch.empty(n, device="cuda")
+    ship, fl = torch.empty(n, dtype=torch.uint8, device="cuda"), z.clone()
+
+    def steps():
+        for _ in range(20):
+            B.pr_decode_step(ctx, x, slot, z, eos, w, 0.0, 0.5, f, ship, fl)
+
+    steps()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=torch.cuda.Stream()):
+        steps()
+    ts = []
+    for _ in range(7):
+        a, b = torch.cuda.Event(True), torch.cuda.Event(True)
+        a.record()
+        g.replay()
+        b.record()
+        torch.cuda.synchronize()
+        ts.append(a.elapsed_time(b) / 20 * 1e3)
+    return min(ts)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("few,more", [(14, 18), (30, 35), (100, 113)])
+def test_no_second_wave_of_clusters(dtype, few, more):
+    """The CTAs of a cluster lie within one GPC: with the even share counted in SMs, 16 to
+    19 rows waited for places that 14 did not need, 32 to 38 and 111 to 114 likewise (1.4 to
+    1.5 times the smaller step's time; one more resident CTA per SM costs 1.15)."""
+    from paper_2608_28726_gb300 import binding as B
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if sms != 152:
+        pytest.skip("row counts of 152 SMs")
+    ctx = B.pr_ctx_create(0, 1, 128)
+    a, b = (step_us(B, ctx, n, 32000, dtype) for n in (few, more))
+    B.pr_ctx_destroy(ctx)
+    assert b < 1.28 * a, (a, b)
