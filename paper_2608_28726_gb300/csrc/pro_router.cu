@@ -214,9 +214,17 @@ pr_status launch_rows(pr_ctx* c, pr_dtype dt, int mode, prk::Args& a, cudaStream
     attr[na].val.clusterDim.z = 1;
     ++na;
   }
-  attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[na].val.programmaticStreamSerializationAllowed = 1;
-  ++na;
+  // Long fp32 rows, one CTA each, are set up after the launch before them has ended:
+  // the memory bounds them, and CTAs placed around those of that launch load the SMs
+  // unevenly all the same (353 rows of V = 151,936 31.4 us a launch in a graph, 36.6 set
+  // up early; 609 of 100,000 36.0 against 42.7; V = 64,000, 256 KB a row, 153 rows
+  // 12.3 against 11.7; bf16 rows gain up to 262,144).
+  const bool long_rows = dt == PR_DTYPE_F32 && C == 1 && a.vocab >= 81920 && !c->overlap;
+  if (!long_rows) {
+    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
+  }
   cfg.attrs = attr;
   cfg.numAttrs = na;
   void* args[] = {&a};

@@ -47,3 +47,15 @@ def test_no_second_wave_of_clusters(dtype, few, more):
     a, b = (step_us(B, ctx, n, 32000, dtype) for n in (few, more))
     B.pr_ctx_destroy(ctx)
     assert b < 1.28 * a, (a, b)
+
+
+def test_long_fp32_rows_load_the_sms_evenly():
+    """353 fp32 rows of 151,936 tokens, one CTA each, take about 353 / 330 of the time of 330
+    (CTAs set up around those of the launch before took 1.18 times as long)."""
+    from paper_2608_28726_gb300 import binding as B
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("row counts of 152 SMs")
+    ctx = B.pr_ctx_create(0, 1, 400)
+    a, b = (step_us(B, ctx, n, 151936, torch.float32) for n in (330, 353))
+    B.pr_ctx_destroy(ctx)
+    assert b < 1.12 * a, (a, b)
