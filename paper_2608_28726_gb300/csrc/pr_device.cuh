@@ -413,8 +413,9 @@ struct WarpTopK {
   }
 };
 
-// Programmatic dependent launch.  Every kernel that begins a call is launched
-// with programmatic stream serialization: it may be set up while the previous
+// Programmatic dependent launch.  A kernel that begins a call is launched with
+// programmatic stream serialization (but for the row kernels' launches that it would
+// spread unevenly over the SMs): it may be set up while the previous
 // kernel on its stream still runs, and waits for that kernel (pdl_wait: complete,
 // its memory visible) before it reads or writes anything, so the stream's order
 // holds as with a plain launch; only the launch's own latency is hidden (16

@@ -1,4 +1,5 @@
-"""Back-to-back split launches: every cluster of a step finds a place at once."""
+"""Back-to-back launches of the row kernels: every cluster of a step finds a place at
+once, and the SMs get even shares."""
 import pytest
 import torch
 
@@ -59,3 +60,16 @@ def test_long_fp32_rows_load_the_sms_evenly():
     a, b = (step_us(B, ctx, n, 151936, torch.float32) for n in (330, 353))
     B.pr_ctx_destroy(ctx)
     assert b < 1.12 * a, (a, b)
+
+
+def test_persistent_launches_load_the_sms_evenly():
+    """The persistent kernel's CTAs with two rows go to different SMs: 609 rows on 456 CTAs
+    take less than 800 (0.95 of it when they were set up around the launch before, 0.85
+    otherwise)."""
+    from paper_2608_28726_gb300 import binding as B
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("row counts of 152 SMs")
+    ctx = B.pr_ctx_create(0, 1, 1024)
+    a, b = (step_us(B, ctx, n, 100000, torch.bfloat16) for n in (800, 609))
+    B.pr_ctx_destroy(ctx)
+    assert b < 0.9 * a, (a, b)
