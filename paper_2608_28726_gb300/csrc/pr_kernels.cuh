@@ -24,6 +24,11 @@ __device__ __forceinline__ uint4 ld_reread(const void* p) {
 
 // ---- pooling, scoring, ship rule (Section 3.1) -------------------------------------
 
+template <int N>
+struct Const {
+  static constexpr int value = N;
+};
+
 struct Pooled {
   float agg[NAGG];
   float score;
@@ -35,7 +40,8 @@ struct Pooled {
 // sums rows lo + j, lo + j + 32, ... in order, then a fixed butterfly combines
 // the lanes, so the result depends only on T.  All lanes return the result.
 // AHEAD rows of a lane are loaded at once: 4 where registers are short (the row
-// kernels' epilogue), more where a long request's latency counts.
+// kernels' epilogue), more where a long request's latency counts (4 all the same in
+// a request of up to 128 rows: the loads past its end take issue slots).
 template <int AHEAD>
 __device__ __forceinline__ Pooled pool_rows(const float* feat, const uint32_t* flags, int64_t lo,
                                             int64_t hi, const float* w, float b, float zthr,
@@ -53,6 +59,24 @@ __device__ __forceinline__ Pooled pool_rows(const float* feat, const uint32_t* f
     fl |= rf;
   };
   int64_t i = lo + lane;
+  // the last fewer than N rows of a lane
+  auto rest = [&](auto n) {
+    constexpr int N = decltype(n)::value;
+    if (i >= hi) return;
+    float4 a[N];
+    float h[N];
+    uint32_t rf[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+      if (i + 32 * k < hi) {
+        a[k] = __ldcg(reinterpret_cast<const float4*>(feat + (i + 32 * k) * NFEAT));
+        h[k] = __ldcg(feat + (i + 32 * k) * NFEAT + 4);
+        rf[k] = flags ? __ldcg(flags + i + 32 * k) : 0u;
+      }
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+      if (i + 32 * k < hi) add(a[k], h[k], rf[k]);
+  };
   for (; i + 32 * (AHEAD - 1) < hi; i += 32 * AHEAD) {
     float4 a[AHEAD];
     float h[AHEAD];
@@ -66,21 +90,8 @@ __device__ __forceinline__ Pooled pool_rows(const float* feat, const uint32_t* f
 #pragma unroll
     for (int k = 0; k < AHEAD; ++k) add(a[k], h[k], rf[k]);
   }
-  if (i < hi) {  // the last fewer than AHEAD rows
-    float4 a[AHEAD];
-    float h[AHEAD];
-    uint32_t rf[AHEAD];
-#pragma unroll
-    for (int k = 0; k < AHEAD; ++k)
-      if (i + 32 * k < hi) {
-        a[k] = __ldcg(reinterpret_cast<const float4*>(feat + (i + 32 * k) * NFEAT));
-        h[k] = __ldcg(feat + (i + 32 * k) * NFEAT + 4);
-        rf[k] = flags ? __ldcg(flags + i + 32 * k) : 0u;
-      }
-#pragma unroll
-    for (int k = 0; k < AHEAD; ++k)
-      if (i + 32 * k < hi) add(a[k], h[k], rf[k]);
-  }
+  if (AHEAD > 4 && hi - lo <= 128) rest(Const<4>());
+  else rest(Const<AHEAD>());
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
@@ -1792,12 +1803,15 @@ __global__ void __launch_bounds__(NT_WS, 3) verify_rows_ws(const Args a) {
 //
 // Up to POOL_FEW requests are bound by the latency of a request's loads: a warp
 // has 16 rows per lane in flight (512 of the request's rows) and a CTA of its
-// own.  24 requests of 17 to 1,024 rows take 3.7 us per launch in a CUDA graph,
-// 6.6 with four rows per lane and eight requests per CTA; 1,024 requests 5.9
-// against 7.4.  More requests are bound by the launch of CTAs and by occupancy
-// and take the latter (20,000 of 1 to 8 rows 9.9 us, 21.1 with a CTA each).
-
-constexpr int POOL_FEW = 4096;
+// own.  More requests are bound by the launch of CTAs and by occupancy: four to a
+// CTA, with four rows per lane.  These let the next launch in once they have their
+// rows, not at their start, where its CTAs would take the places that theirs still
+// wait for.  Back to back in a CUDA graph, requests of 1 to 8, 300 and 1,000 rows
+// take: 24 requests 2.5, 3.3 and 4.2 us; 1,024 2.8, 4.1 and 6.6; 2,048
+// (four to a CTA) 3.0, 4.9 and 9.8; 4,096 3.8 and 7.3.  A CTA each takes 2,048 to 3.9,
+// 5.6 and 11.4, 4,096 to 6.4 and 9.3; four to one takes 24 to 2.5, 3.4 and 5.4.
+constexpr int POOL_FEW = 1024;
+constexpr int POOL_WARPS = 4;
 
 struct AggArgs {
   const float* feat;
@@ -1817,7 +1831,8 @@ struct AggArgs {
 // internal linkage: the header is included by more than one translation unit
 template <int WARPS, int AHEAD>
 static __global__ void __launch_bounds__(32 * WARPS) pool_requests(const AggArgs a) {
-  pdl_enter(false);
+  pdl_wait();
+  if (WARPS == 1) pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int64_t r = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
   if (r >= a.n_req) return;
@@ -1834,6 +1849,7 @@ static __global__ void __launch_bounds__(32 * WARPS) pool_requests(const AggArgs
     return;
   }
   const Pooled p = pool_rows<AHEAD>(a.feat, a.row_flags, lo, hi, a.w, a.b, a.zthr, lane);
+  if (WARPS > 1) pdl_trigger();
   write_pooled(p, r, a.agg, a.score, a.ship, a.req_flags, lane);
 }
 

@@ -328,8 +328,9 @@ pr_status pr_aggregate_score(pr_ctx* c, const float* feat, const uint32_t* row_f
   const bool few = n_req <= prk::POOL_FEW;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
-  cfg.gridDim = dim3(few ? (unsigned)n_req : (unsigned)((n_req + prk::NWARP - 1) / prk::NWARP));
-  cfg.blockDim = dim3(few ? 32 : prk::NT);
+  const int warps = few ? 1 : prk::POOL_WARPS;
+  cfg.gridDim = dim3((unsigned)((n_req + warps - 1) / warps));
+  cfg.blockDim = dim3((unsigned)(32 * warps));
   cfg.stream = reinterpret_cast<cudaStream_t>(stream);
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -339,7 +340,7 @@ pr_status pr_aggregate_score(pr_ctx* c, const float* feat, const uint32_t* row_f
   void* args[] = {&a};
   PR_CUDA(cudaLaunchKernelExC(&cfg,
                               few ? reinterpret_cast<void*>(&prk::pool_requests<1, 16>)
-                                  : reinterpret_cast<void*>(&prk::pool_requests<prk::NWARP, 4>),
+                                  : reinterpret_cast<void*>(&prk::pool_requests<prk::POOL_WARPS, 4>),
                               args));
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return PR_OK;

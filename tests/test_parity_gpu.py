@@ -103,10 +103,10 @@ def test_features_unaligned_rows(ctx, dtype, shift, split):
     _set(ctx)
 
 
-@pytest.mark.parametrize("n_req", [1, 30, 4096, 4097])
+@pytest.mark.parametrize("n_req", [1, 30, 1024, 1025, 4096, 4097])
 def test_aggregate_lengths(ctx, n_req):
     """The pooling call at the edges of its rows in flight (32, 128 and 512 rows
-    per round) and on both sides of the switch to eight requests per CTA."""
+    per round) and on both sides of the switch to four requests per CTA."""
     edges = [1, 31, 32, 33, 127, 128, 129, 511, 512, 513, 1024, 1500, 0]
     lengths = [edges[r % len(edges)] if n_req <= 30 else r % 40 for r in range(n_req)]
     off = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
