@@ -93,6 +93,7 @@ struct QArgs {
   uint8_t* ship;
   uint32_t* req_flags;
   uint32_t* ctx_flags;
+  int32_t full;  // the launch fills the GPU: the next one may be set up at once
 };
 
 __device__ __forceinline__ uint32_t q_key(float x) {
@@ -530,7 +531,8 @@ __global__ void __launch_bounds__(Q_NT, 3) qmlp_requests(const QArgs a) {
   __shared__ uint32_t wfl[Q_NT / 32];
   __shared__ uint32_t qx[4][Q_SMALL];  // exchange between the two warps of a column
   __shared__ float zpart[2];
-  pdl_enter(false);
+  pdl_wait();
+  if (a.full) pdl_trigger();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t r = blockIdx.x;
   const int64_t lo = a.offsets[r], hi = a.offsets[r + 1];
@@ -545,17 +547,19 @@ __global__ void __launch_bounds__(Q_NT, 3) qmlp_requests(const QArgs a) {
   }
   const int T = (int)(hi - lo);
   // the MLP's weights, fetched now (coalesced) so that their latency overlaps
-  // the key loads and the sort; a selection, whose records take the registers,
-  // fetches them before it sorts
+  // the offsets', the key loads and the sort; a selection, whose records take the
+  // registers, fetches them again before it sorts
   float wr[QW_PER_T];
   auto fetch_w = [&]() {
 #pragma unroll
     for (int i = 0; i < QW_PER_T; ++i) {
       const int g = tid + i * Q_NT;
-      wr[i] = g < QW_SIZE ? a.w[g] : 0.f;
+      wr[i] = 0.f;
+      if (g < QW_SIZE)  // (volatile: not to be moved behind the request's offsets)
+        asm volatile("ld.global.f32 %0, [%1];" : "=f"(wr[i]) : "l"(a.w + g));
     }
   };
-  if (T <= Q_MID) fetch_w();
+  fetch_w();
   if (T == 0) {
     if (tid == 0) {
       a.score[r] = 0.f;

@@ -40,6 +40,12 @@ pr_status pr_quantile_score(pr_ctx* c, const float* feat, const uint32_t* row_fl
   a.ship = ship;
   a.req_flags = req_flags;
   a.ctx_flags = c->flags;
+  // Three CTAs fit an SM.  A launch of fewer than fill the GPU does not let the next
+  // one in before its CTAs end: that one's would take the free places, and its last
+  // ones go together on the SMs that end first (300 requests of 700 rows back to back
+  // 21.0 us, 27.0 with the early set-up; of 1 to 8 rows 6.7 and 8.1; 512 ragged ones
+  // 24.4 and 23.3).
+  a.full = n_req >= 3 * c->num_sms ? 1 : 0;
   if (!c->qmlp_ready) {
     PR_CUDA(cudaFuncSetAttribute(prk::qmlp_requests, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(prk::Q_DYN * sizeof(uint32_t))));

@@ -95,3 +95,26 @@ def test_many_short_requests_share_ctas():
     a, b = t(1024), t(4096)
     B.pr_ctx_destroy(ctx)
     assert b < 1.6 * a, (a, b)
+
+
+def test_quantile_launches_load_the_sms_evenly():
+    """300 requests of 700 rows, two CTAs on an SM, take less than 1.75 times the time of 150,
+    one on each (1.6 times; twice as long when the next launch took the free places)."""
+    from paper_2608_28726_gb300 import binding as B
+    from paper_2608_28726_gb300 import workloads as W
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("request counts of 152 SMs")
+    ctx = B.pr_ctx_create(0, 1, 1)
+    w = torch.from_numpy(W.qmlp_weights()).cuda()
+
+    def t(n):
+        off = torch.arange(n + 1, device="cuda") * 700
+        feat = torch.randn(700 * n, 8, device="cuda")
+        out = [torch.empty(n, 28, device="cuda"), torch.empty(n, device="cuda"),
+               torch.empty(n, dtype=torch.uint8, device="cuda"),
+               torch.empty(n, dtype=torch.int32, device="cuda")]
+        return replay_us(lambda: B.pr_quantile_score(ctx, feat, off, w, 0.5, None, *out))
+
+    a, b = t(150), t(300)
+    B.pr_ctx_destroy(ctx)
+    assert b < 1.75 * a, (a, b)
