@@ -475,9 +475,16 @@ struct SelSums {
 __device__ __forceinline__ uint32_t sel_at(uint32_t w) { return w + (w >> 5); }
 static_assert(2 * SB_LIGHT + SB_RADIX + SB_RADIX / 32 <= SB_WORDS,
               "a light bucket, its label prefix and the sub-bins");
+static_assert(2 * SB_LIGHT + SB_RADIX + SB_RADIX / 32 + SB_RADIX / 2 <= SB_WORDS,
+              "and the sub-bins' prefix counts in 16 bits");
+static_assert(SB_SHIFT - 12 <= 8, "at most 256 keys in a sub-bin");
 static_assert(1 << SB_VBITS == 32 * SB_NT, "a strip of 32 keys per thread");
 static_assert(SB_RADIX == 8 * SB_NT && SB_LIGHT == 8 * SB_NT, "eight per thread");
 
+// LARGE: for pools in which buckets of more than SB_LIGHT items over more keys than
+// are counted at once are the rule, not the exception (target above SB_LIGHT, from
+// 3.4e7 scores on).  Apart, as its registers would cost the other pools 3%.
+template <bool LARGE>
 __global__ void __launch_bounds__(SB_NT, 3) sel_bucket(const SelArgs a) {
   extern __shared__ __align__(16) uint32_t sb_dyn[];
   __shared__ uint32_t ws[2][SB_NT / 32], next, ranges[4], strip[2][SB_NT];
@@ -618,16 +625,14 @@ __global__ void __launch_bounds__(SB_NT, 3) sel_bucket(const SelArgs a) {
         visit(S, has_tau, key0 + first + 32u * s + lane, a0 + strip[0][s] + ic - c, q0 + strip[1][s] + ip - p, c, p);
       }
     };
-    if (m <= (uint32_t)SB_LIGHT) {
-      // ---- a light bucket: sorted, then a group per run of equal offsets.  The
-      // items go to sub-bins of the offset's leading bits (about one item in
-      // each), a thread sorts each sub-bin; piled-up offsets take a bitonic
-      // sort of the whole
+    // ---- up to SB_LIGHT items it[] (e * SB_NT + tid: offset from `base` << 1 | label;
+    // offsets below 2^(sh + 12)), a0 items and q0 correct ones below them: sorted,
+    // then a group per run of equal offsets.  The items go to sub-bins of the
+    // offset's leading bits (about one item in each), a thread sorts each sub-bin;
+    // piled-up offsets take a bitonic sort of the whole.  Returns the correct ones.
+    auto light = [&](uint32_t (&it)[8], uint32_t m, uint32_t sh, uint32_t base, uint32_t a0,
+                     uint32_t q0) -> uint32_t {
       uint32_t *v = sb_dyn, *pre = sb_dyn + SB_LIGHT, *sub = pre + SB_LIGHT;
-      const uint32_t sh = r - 12u;  // 2^r keys, SB_RADIX = 2^12 sub-bins
-      uint32_t it[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) it[e] = e * SB_NT + tid < m ? items[e * SB_NT + tid] : ~0u;
       for (uint32_t i = tid; i < SB_RADIX + SB_RADIX / 32; i += SB_NT) sub[i] = 0u;
       __syncthreads();
 #pragma unroll
@@ -694,8 +699,8 @@ __global__ void __launch_bounds__(SB_NT, 3) sel_bucket(const SelArgs a) {
         x += v[i] & 1u;
       }
       __syncthreads();
-      for (uint32_t base = 0; base < m; base += SB_NT) {
-        const uint32_t i = base + tid;
+      for (uint32_t i0 = 0; i0 < m; i0 += SB_NT) {
+        const uint32_t i = i0 + tid;
         uint32_t off = 0u, pi = 0u, c = 0u, p = 0u;
         if (i < m) {
           off = v[i] >> 1;
@@ -713,8 +718,15 @@ __global__ void __launch_bounds__(SB_NT, 3) sel_bucket(const SelArgs a) {
             p = (e < m ? pre[e] : xall) - pi;
           }
         }
-        visit(S, has_tau, key0 + off, s0 + i, p0 + pi, c, p);
+        visit(S, has_tau, key0 + base + off, a0 + i, q0 + pi, c, p);
       }
+      return xall;
+    };
+    if (m <= (uint32_t)SB_LIGHT) {
+      uint32_t it[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) it[e] = e * SB_NT + tid < m ? items[e * SB_NT + tid] : ~0u;
+      light(it, m, r - 12u, 0u, s0, p0);  // 2^r keys, SB_RADIX = 2^12 sub-bins
     } else if (m > (uint32_t)SB_HEAVY && r == (uint32_t)SB_VBITS) {
       // ---- a heavy bucket: already counted (sel_heavy)
       const unsigned long long* hc = a.hcnt + ((size_t)a.hidx[b] << SB_VBITS);
@@ -746,7 +758,75 @@ __global__ void __launch_bounds__(SB_NT, 3) sel_bucket(const SelArgs a) {
       if (lane < 4)
         atomicOr(ranges + lane, lane == 0 ? used[0] : lane == 1 ? used[1] : lane == 2 ? used[2] : used[3]);
       __syncthreads();
-      for (uint32_t ps = 0; ps < 1u << (r - vb); ++ps) {
+      uint32_t ps = 0u;  // first range
+      const uint32_t filled =
+          LARGE ? __popc(ranges[0]) + __popc(ranges[1]) + __popc(ranges[2]) + __popc(ranges[3]) : 0u;
+      if (LARGE && !wide && filled > m / 2048u + 2u) {
+        // spread over more ranges than it takes chunks of up to SB_LIGHT items (a pool
+        // of tens of millions over many coarse bins; 4e7 random bit patterns 7.3 ms
+        // range by range, 1.36 now): chunk by chunk, whole sub-bins of the offset's 12
+        // leading bits, their prefix counts in 16 bits behind what `light` uses
+        uint16_t* pre16 = reinterpret_cast<uint16_t*>(sb_dyn + SB_WORDS - SB_RADIX / 2);
+        const uint32_t sb = r - 12u;  // bits of a sub-bin
+        for (uint32_t i = tid; i < SB_RADIX; i += SB_NT) sb_dyn[i] = 0u;
+        __syncthreads();
+        for (uint32_t i = tid; i < m; i += SB_NT) atomicAdd(sb_dyn + (items[i] >> 1 >> sb), 1u);
+        __syncthreads();
+        uint32_t c8[8], x = 0, y = 0, xall, yall;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          c8[e] = sb_dyn[8 * tid + e];
+          x += c8[e];
+        }
+        sel_scan2<SB_NT>(x, y, xall, yall, ws);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          pre16[8 * tid + e] = (uint16_t)x;
+          x += c8[e];
+        }
+        auto before = [&](uint32_t sub) { return sub < (uint32_t)SB_RADIX ? (uint32_t)pre16[sub] : m; };
+        for (uint32_t b0 = 0; b0 < (uint32_t)SB_RADIX;) {
+          __syncthreads();
+          const uint32_t i0 = before(b0);
+          if (i0 == m) break;
+          uint32_t b1 = b0, step = SB_RADIX;  // the most sub-bins of up to SB_LIGHT items
+          for (; step; step >>= 1)
+            if (b1 + step <= (uint32_t)SB_RADIX && before(b1 + step) - i0 <= (uint32_t)SB_LIGHT)
+              b1 += step;
+          const bool dense = b1 == b0;  // more of them in one sub-bin (at most 256 keys)
+          if (dense) ++b1;
+          const uint32_t n = before(b1) - i0, low = b0 << sb;
+          if (tid == 0) ranges[0] = 0u;
+          if (dense)
+            for (uint32_t i = tid; i < 256u; i += SB_NT) sb_dyn[i] = 0u;
+          __syncthreads();
+          for (uint32_t i = tid; i < m; i += SB_NT) {
+            const uint32_t it = items[i], off = it >> 1, sub = off >> sb;
+            if (sub < b0 || sub >= b1) continue;
+            if (dense) atomicAdd(sb_dyn + (off - low), 1u + ((it & 1u) << 16));
+            else sb_dyn[atomicAdd(ranges, 1u)] = it - (low << 1);
+          }
+          __syncthreads();
+          if (dense) {
+            walk(low, 256u, a0, q0, true, [&](uint32_t w, uint32_t& c, uint32_t& p) {
+              c = sb_dyn[w] & 0xffffu;
+              p = sb_dyn[w] >> 16;
+            }, xall, yall);
+            q0 += yall;
+          } else {
+            uint32_t it[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) it[e] = e * SB_NT + tid < n ? sb_dyn[e * SB_NT + tid] : ~0u;
+            __syncthreads();
+            const int bits = 32 - __clz(((b1 - b0) << sb) - 1u);  // offsets below 2^bits
+            q0 += light(it, n, (uint32_t)max(bits - 12, 0), low, a0, q0);
+          }
+          a0 += n;
+          b0 = b1;
+        }
+        ps = 1u << (r - vb);
+      }
+      for (; ps < 1u << (r - vb); ++ps) {
         if (!(ranges[ps >> 5] >> (ps & 31u) & 1u)) continue;
         __syncthreads();
         for (uint32_t i = tid; i < (uint32_t)SB_WORDS; i += SB_NT) sb_dyn[i] = 0u;

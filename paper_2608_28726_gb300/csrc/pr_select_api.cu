@@ -25,9 +25,12 @@ size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 struct SelShape {
   uint32_t share, shares, target, nbcap, rows;
   SelShape(int64_t n, int num_sms) {
-    // two shares per SM, not below 4,096 items (a share pays for every bucket);
-    // a multiple of 4 for the vector loads
-    const int64_t even = ((n + 2 * num_sms - 1) / (2 * num_sms) + 3) & ~(int64_t)3;
+    // two shares per SM, or as many rounds of those as a share's counts need (4e7
+    // uniform scores 2.2 ms with shares of SB_SHARE, whose last round was nearly empty,
+    // now 1.0), not below 4,096 items (a share pays for every bucket); a multiple of 4
+    // for the vector loads
+    const int64_t round = 2 * (int64_t)num_sms, rounds = (n + round * prk::SB_SHARE - 1) / (round * prk::SB_SHARE);
+    const int64_t even = ((n + round * rounds - 1) / (round * rounds) + 3) & ~(int64_t)3;
     share = (uint32_t)std::min<int64_t>(prk::SB_SHARE, std::max<int64_t>(4096, even));
     shares = (uint32_t)((n + share - 1) / share);
     // a bin that holds most of a small pool is still cut into 64 buckets, whose keys
@@ -35,13 +38,12 @@ struct SelShape {
     target = (uint32_t)std::max<int64_t>(
         std::min<int64_t>(prk::SB_TARGET, std::max<int64_t>(prk::SB_FEW_TARGET, n / 64)),
         (n + 8191) / 8192);
-// the workspace's bounds do not fall when n grows: n / target buckets over the
+    // the workspace's bounds do not fall when n grows: n / target buckets over the
     // coarse bins', twice, and the shares
     nbcap = (uint32_t)(std::min<int64_t>(n, prk::SB_BINS) + 1 +
                        2 * std::max(std::min<int64_t>(n / prk::SB_FEW_TARGET, 65),
                                     std::min<int64_t>(n / prk::SB_TARGET, 8192)));
-    rows = (uint32_t)std::max<int64_t>(std::min<int64_t>((n + 4095) / 4096, 2 * num_sms),
-                                       (n + prk::SB_SHARE - 1) / prk::SB_SHARE);
+    rows = (uint32_t)std::min<int64_t>((n + 4095) / 4096, round * rounds);
   }
 };
 
@@ -117,7 +119,9 @@ pr_status pr_selective_metrics(pr_ctx* c, const float* scores, const uint8_t* la
     PR_CUDA(cudaFuncSetAttribute(prk::sel_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     PR_CUDA(cudaFuncSetAttribute(prk::sel_heavy, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)prk::SB_BUCKET_SMEM));
-    PR_CUDA(cudaFuncSetAttribute(prk::sel_bucket, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    PR_CUDA(cudaFuncSetAttribute(prk::sel_bucket<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)prk::SB_BUCKET_SMEM));
+    PR_CUDA(cudaFuncSetAttribute(prk::sel_bucket<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)prk::SB_BUCKET_SMEM));
     c->sel_ready = true;
   }
@@ -185,7 +189,8 @@ pr_status pr_selective_metrics(pr_ctx* c, const float* scores, const uint8_t* la
     PR_LAUNCH(prk::sel_heavy,
               (unsigned)std::min<int64_t>(n / prk::SB_CHUNK + 1, 3 * c->num_sms), prk::SB_NT,
               prk::SB_BUCKET_SMEM);
-  PR_LAUNCH(prk::sel_bucket, (unsigned)std::min<int64_t>(g.nbcap, 3 * c->num_sms), prk::SB_NT,
+  PR_LAUNCH(g.target > (uint32_t)prk::SB_LIGHT ? prk::sel_bucket<true> : prk::sel_bucket<false>,
+            (unsigned)std::min<int64_t>(g.nbcap, 3 * c->num_sms), prk::SB_NT,
             prk::SB_BUCKET_SMEM);
   PR_LAUNCH(prk::sel_finish, 1, prk::SB_NT, 0);
 #undef PR_LAUNCH

@@ -99,7 +99,7 @@ def test_selective_key_structures(B, ctx, n, kind):
     """Keys spread over both signs and many exponents, piled up in a few buckets,
     a few floats apart, at the ends of the float range; tie groups on both
     sides of the closed form, also at the very top ranks; buckets that are
-    sorted, counted and counted with wide counts."""
+    sorted and counted (with 32-bit counts: test_selective_large_pool)."""
     g = np.random.Generator(np.random.PCG64(n))
     if kind == "logits":
         s = g.normal(0.0, 2.0, n) ** 3
@@ -155,3 +155,21 @@ def test_selective_full_pool(B, ctx):
     s[::1000] = np.float32(0.5)
     check(run(B, ctx, s, y, 0.7), s, y, 0.7)
 
+
+
+def test_selective_large_pool(B, ctx):
+    """3.4e7 scores, more than 4,096 for each of 8,192 buckets: random bit patterns, whose
+    buckets are resolved chunk by chunk; one bin with 5,000 equal scores among its others,
+    a chunk that is counted; and one with 122,000 within 2^15 neighbouring keys, a bucket
+    counted with 32-bit counts."""
+    n = 34_000_000
+    g = np.random.Generator(np.random.PCG64(11))
+    s = g.integers(0, 2 ** 32, n, dtype=np.uint32).view(np.float32)
+    s[~np.isfinite(s)] = 0.25
+    at = g.permutation(n)[:127_000]
+    one = np.float32(3.0).view(np.uint32)                       # a 2^20-key bin starts here
+    s[at[:122_000]] = (one + (5 << 15) + g.integers(0, 2000, 122_000) ** 2 % (1 << 15)).astype(
+        np.uint32).view(np.float32)
+    s[at[122_000:]] = (np.float32(-7.0).view(np.uint32) + np.uint32(12345)).view(np.float32)
+    y = (g.random(n) < np.where(s > 0, 0.7, 0.4)).astype(np.uint8)
+    check(run(B, ctx, s, y, 0.3), s, y, 0.3)
