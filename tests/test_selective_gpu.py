@@ -173,3 +173,22 @@ def test_selective_large_pool(B, ctx):
     s[at[122_000:]] = (np.float32(-7.0).view(np.uint32) + np.uint32(12345)).view(np.float32)
     y = (g.random(n) < np.where(s > 0, 0.7, 0.4)).astype(np.uint8)
     check(run(B, ctx, s, y, 0.3), s, y, 0.3)
+
+
+@pytest.mark.parametrize("c", [2, 65, 300, 1000, 4000])
+def test_selective_ties_below_incorrect_answers(B, ctx, c):
+    """A tie group below 64 and below 1,024 times as many incorrect answers, where the
+    expansion of its sum in 1 / rank leaves most: at most 2^-34 of the sum (stated in the
+    kernel); 2^-33 with the roundings of the oracle's sum here."""
+    for times in (64.5, 100, 1025, 1100, 2000):
+        a = int(c * times)
+        s = np.full(a + c, 0.75, np.float32)
+        s[:a] = (np.float32(0.75).view(np.uint32) + np.arange(a, 0, -1, dtype=np.uint32)).view(
+            np.float32)
+        for p in sorted({1, c // 2, c - 1}):
+            y = np.zeros(a + c, np.uint8)
+            y[a:a + p] = 1
+            k = np.arange(a + 1, a + c + 1, dtype=np.float64)
+            want = float(np.sum((p / c) * np.arange(1, c + 1) / k) / (a + c))
+            got = run(B, ctx, s, y, 0.5)["auarc"]
+            assert abs(got - want) <= 2.0 ** -33 * want, (times, p, got, want)
