@@ -477,6 +477,7 @@ struct SelSums {
 // word of sub-bin w: one word of padding per 32, so that the runs of 8 that
 // threads scan lie in different banks
 __device__ __forceinline__ uint32_t sel_at(uint32_t w) { return w + (w >> 5); }
+static_assert(SB_SMALL < 256 && 3 * SB_SMALL * SB_NT / 32 <= SB_WORDS, "three arrays per warp");
 static_assert(2 * SB_LIGHT + SB_RADIX + SB_RADIX / 32 <= SB_WORDS,
               "a light bucket, its label prefix and the sub-bins");
 static_assert(2 * SB_LIGHT + SB_RADIX + SB_RADIX / 32 + SB_RADIX / 2 <= SB_WORDS,
@@ -512,16 +513,21 @@ __global__ void __launch_bounds__(SB_NT, 3) sel_bucket(const SelArgs a) {
     }
   };
   // ---- buckets of a few items (those of a pool spread over many coarse bins), a
-  // warp each: a lane counts the items below and equal to its own
-  uint32_t* mine = sb_dyn + warp * SB_SMALL;
+  // warp each: a lane counts the items below and equal to its own, and the first of
+  // each group leaves it at its rank, so that the sums' order is the groups' and not
+  // that in which the items came
+  uint32_t* mine = sb_dyn + warp * 3 * SB_SMALL;
+  uint32_t *goff = mine + SB_SMALL, *gcnt = goff + SB_SMALL;  // c | p << 8 | correct below << 16
   for (uint32_t b = blockIdx.x * (SB_NT / 32) + warp; b < nb; b += gridDim.x * (SB_NT / 32)) {
     const uint32_t s0 = a.start[b], m = a.start[b + 1] - s0, p0 = a.pstart[b];
     const bool has_tau = kk > 0 && itau - s0 < m;
     if (m > (uint32_t)SB_SMALL || !(metrics || has_tau)) continue;
     SelSums S = {0.f, 0.f, 0.0, 0ull};
     __syncwarp();
-    for (uint32_t i = lane; i < ((m + 3u) & ~3u); i += 32u)
+    for (uint32_t i = lane; i < ((m + 3u) & ~3u); i += 32u) {
       mine[i] = i < m ? a.items[s0 + i] : ~0u;  // no item's offset
+      gcnt[i] = 0u;
+    }
     __syncwarp();
     for (uint32_t base = 0; base < m; base += 32u) {
       const uint32_t i = base + lane, v = i < m ? mine[i] : ~0u, key = v & ~1u;
@@ -540,9 +546,16 @@ __global__ void __launch_bounds__(SB_NT, 3) sel_bucket(const SelArgs a) {
           }
         }
       }
-      if (i >= m || first != i) same = 0u;
-      visit(S, has_tau, (a.bkey[b] & ~31u) + (v >> 1), s0 + (below & 0xffffu), p0 + (below >> 16),
-            same & 0xffffu, same >> 16);
+      if (i < m && first == i) {
+        goff[below & 0xffffu] = v >> 1;
+        gcnt[below & 0xffffu] = (same & 0xffffu) | (same >> 16) << 8 | (below >> 16) << 16;
+      }
+    }
+    __syncwarp();
+    for (uint32_t base = 0; base < m; base += 32u) {
+      const uint32_t i = base + lane, g = i < m ? gcnt[i] : 0u;
+      visit(S, has_tau, (a.bkey[b] & ~31u) + (g ? goff[i] : 0u), s0 + i, p0 + (g >> 16), g & 0xffu,
+            (g >> 8) & 0xffu);
     }
     double d = ((double)S.fs + (double)S.fc) + S.ds;
     unsigned long long u = S.roc2;

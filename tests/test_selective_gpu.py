@@ -192,3 +192,20 @@ def test_selective_ties_below_incorrect_answers(B, ctx, c):
             want = float(np.sum((p / c) * np.arange(1, c + 1) / k) / (a + c))
             got = run(B, ctx, s, y, 0.5)["auarc"]
             assert abs(got - want) <= 2.0 ** -33 * want, (times, p, got, want)
+
+
+@pytest.mark.parametrize("n", [500, 900, 20000, 150000, 1000000])
+@pytest.mark.parametrize("kind", ["uniform", "bits", "logits"])
+def test_selective_repeats_bit_for_bit(B, ctx, n, kind):
+    """Pools whose buckets hold a few items, in whatever order these reach them."""
+    g = np.random.Generator(np.random.PCG64(n))
+    if kind == "bits":
+        s = g.integers(0, 2 ** 32, n, dtype=np.uint32).view(np.float32)
+        s[~np.isfinite(s)] = 0.25
+    else:
+        s = g.random(n).astype(np.float32) if kind == "uniform" else g.normal(0, 2, n).astype(np.float32) ** 3
+    y = torch.from_numpy((g.random(n) < 0.6).astype(np.uint8)).cuda()
+    s = torch.from_numpy(s).cuda()
+    first = B.pr_selective_metrics(ctx, s, 0.4, labels=y)
+    for _ in range(20):
+        assert B.pr_selective_metrics(ctx, s, 0.4, labels=y) == first
