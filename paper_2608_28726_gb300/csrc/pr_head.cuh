@@ -404,12 +404,11 @@ __global__ void __launch_bounds__(HA_M, HA_CTAS_PER_SM) head_attn(const HeadArgs
   // the offsets are inputs of the call, complete before its first kernel
   const int T = head_request(a, blockIdx.x, lo, hi) ? (int)(hi - lo) : 0;
   const int nqb = (T + HA_M - 1) / HA_M;
-  if ((int)blockIdx.z >= nqb) {
+  // a CTA without a query block has nothing to do, but for the first one, which goes
+  // on and waits: a grid whose requests are all empty or rejected must not end before
+  // the row kernel that it follows, on whose end everything after it relies
+  if ((int)blockIdx.z >= nqb && (blockIdx.x | blockIdx.y | blockIdx.z) != 0u) {
     pdl_trigger();
-    // one CTA of the grid always waits: a grid whose requests are all empty or
-    // rejected must not end before the row kernel that it follows, on whose end
-    // everything after it relies
-    if ((blockIdx.x | blockIdx.y | blockIdx.z) == 0) pdl_wait();
     return;
   }
   const int hh = blockIdx.y;
