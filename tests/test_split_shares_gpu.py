@@ -118,3 +118,23 @@ def test_quantile_launches_load_the_sms_evenly():
     a, b = t(150), t(300)
     B.pr_ctx_destroy(ctx)
     assert b < 1.75 * a, (a, b)
+
+
+@pytest.mark.parametrize("n", [5, 17, 60, 100, 300])
+def test_the_first_call_of_a_context_can_be_captured(n):
+    """What a launch asks the runtime once (residency, places for clusters) is not refused
+    while a stream is captured."""
+    from paper_2608_28726_gb300 import binding as B
+    x = torch.randn(n, 4000, device="cuda").bfloat16()
+    ch = torch.zeros(n, dtype=torch.int32, device="cuda")
+    outs = [[torch.zeros(n, 8, device="cuda"), torch.zeros(n, 2, dtype=torch.int32, device="cuda"),
+             torch.zeros(n, dtype=torch.int32, device="cuda")] for _ in range(2)]
+    ctx = B.pr_ctx_create(0, n, 1)
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=torch.cuda.Stream()):
+        B.pr_token_features(ctx, x, ch, 20, None, *outs[0])
+    g.replay()
+    B.pr_token_features(ctx, x, ch, 20, None, *outs[1])
+    assert all(torch.equal(a, b) for a, b in zip(*outs)) and outs[0][0].abs().sum() > 0
+    B.pr_ctx_destroy(ctx)
