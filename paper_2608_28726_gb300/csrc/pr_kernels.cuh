@@ -1292,6 +1292,7 @@ __device__ __noinline__ void finalize_ws(const Args& a, SmemWS& sm, int b, int64
   // ---- theta1: the kc-th largest of the published thread maxima and of the last
   // elements
   float th1;
+  bool one_warp;  // it is one warp's least maximum: sharper bounds are near
   {
     const uint32_t mine = sm.pub[b][lane], em = edge ? ord(xe) : 0u;
     int rk = 0, re = 0;
@@ -1310,7 +1311,9 @@ __device__ __noinline__ void finalize_ws(const Args& a, SmemWS& sm, int b, int64
     const unsigned hite = __ballot_sync(FULL, edge && re == kc - 1);
     const uint32_t v = hit ? __shfl_sync(FULL, mine, __ffs(hit) - 1)
                            : __shfl_sync(FULL, em, (__ffs(hite) - 1) & 31);
-    th1 = unord(max(v, __reduce_max_sync(FULL, sm.low[b][lane & (NWARP - 1)])));
+    const uint32_t lows = __reduce_max_sync(FULL, sm.low[b][lane & (NWARP - 1)]);
+    one_warp = lows > v && geo.gfull >= TILE;
+    th1 = unord(max(v, lows));
   }
   // ---- candidate tiles: lane l looks at the reports of threads l, 32 + l, ...  Once
   // more by a bound from all thread maxima if too many reach theta1, or fewer than
@@ -1337,9 +1340,11 @@ __device__ __noinline__ void finalize_ws(const Args& a, SmemWS& sm, int b, int64
     n = __shfl_sync(FULL, x, 31);  // candidate tiles
   };
   count();
-  // (32 candidates are read at once: where theta1 is sharp, more are already too many)
+  // (32 candidates are read at once: where theta1 is sharp, more are already too many;
+  // rows of V = 32,000 bf16 with 1,000 neighbouring tokens 10 above the others, 1,500
+  // of them, take 63 us with one warp's least maximum, 51 with the bound raised)
   const int many = kc <= 24 && geo.gfull >= TILE ? kc + 12 : many_tiles(kc);
-  if (geo.gfull > 32 * UNR && (n > many || !(th1 > -INFINITY))) {
+  if (geo.gfull > 32 * UNR && (n > many || !(th1 > -INFINITY) || one_warp)) {
     th1 = raise_ws(sm.tinfo[b], edge ? ord(xe) : 0u, th1, kc, lane);
     count();
   }
